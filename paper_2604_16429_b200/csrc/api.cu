@@ -39,7 +39,6 @@ int validate(const mosaic_bsa_params* p, Geo* g) {
   g->nbh = p->nlat / p->bh; g->nbw = p->nlon / p->bw; g->m = (int)m;
   g->b = p->bh * p->bw; g->cpb = cpb; g->crows = crows;
   g->rlat = p->rlat; g->rlon = p->rlon; g->topk = p->topk;
-  g->local_off = 0;
   g->local_groups = groups ? 1 : 0;
   g->f16 = (p->flags & MOSAIC_FLAG_FP16) ? 1 : 0;
   g->scale = p->scale > 0.f ? p->scale : 1.0f / sqrtf((float)p->d);
@@ -62,27 +61,25 @@ SelectWs select_layout(const Geo& g) {
 BranchWs branch_layout(const Geo& g) {
   BranchWs w;
   const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD), norms = align256(sizeof(float) * (size_t)g.U * g.m);
-  const size_t full = align256(2 * (size_t)g.U * g.N * kD);
   w.pq = kStatusBytes;
   w.pk = w.pq + pooled;
   w.pv = w.pk + pooled;
   w.nrm = w.pv + pooled;
   w.ocg = w.nrm + 2 * norms;
-  w.ofg = w.ocg + pooled;
-  w.ol = w.ofg + full;
-  w.total = w.ol + full;
+  w.total = w.ocg + pooled;
   return w;
 }
 
 namespace {
 
-struct BwdWs { size_t D, negD, nlse2, off, q, order, total; };
-BwdWs bwd_layout(const Geo& g) {
+struct BwdWs { size_t neg_d, neg_lse2, gate, off, q, order, total; };
+// `planes`: sets of row statistics (two, and the gates, in the three-branch form)
+BwdWs bwd_layout(const Geo& g, int planes, size_t at) {
   BwdWs w;
-  size_t at = kStatusBytes;
-  w.D = at; at = align256(at + sizeof(float) * (size_t)g.U * g.N);
-  w.negD = at; at = align256(at + sizeof(float) * (size_t)g.U * g.N);
-  w.nlse2 = at; at = align256(at + sizeof(float) * (size_t)g.U * g.N);
+  const size_t rows = align256(sizeof(float) * (size_t)planes * g.U * g.N);
+  w.neg_d = at; at += rows;
+  w.neg_lse2 = at; at += rows;
+  w.gate = at; at += planes > 1 ? rows : 0;
   w.off = at; at = align256(at + sizeof(int32_t) * (size_t)g.U * (g.m + 1));
   w.q = at; at = align256(at + sizeof(int32_t) * (size_t)g.U * g.m * (g.topk > 0 ? g.topk : 1));
   // dK/dV items (two 128-row tiles per 256-row item of a key/value unit), longest first, and their cost classes
@@ -90,32 +87,25 @@ BwdWs bwd_layout(const Geo& g) {
   w.total = at;
   return w;
 }
-// Scratch of the three-branch backward: the forward's (pooled sums, obar, both branch outputs), the branch
-// log-sum-exps, the block-level backward's vectors, the gated copies of dO, the branch gradients, and the
-// attention backward's own scratch (used by the two passes in turn).
+// Scratch of the three-branch backward: the forward's (pooled sums, obar), the block-level backward's vectors and the
+// attention backward's own scratch.
 struct BwdBranchWs {
   BranchWs f;
-  size_t lse_fg, lse_l, lse_cg, delta, dob, dqm, dkm, dvm, do_fg, do_l, dq_fg, dq_l, dk_fg, dk_l, dv_fg, dv_l, inner, total;
+  size_t lse_cg, delta, dob, dqm, dkm, dvm;
+  BwdWs b;
 };
 BwdBranchWs bwd_branch_layout(const Geo& g) {
   BwdBranchWs w;
   w.f = branch_layout(g);
-  const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD), rows = align256(sizeof(float) * (size_t)g.U * g.N);
-  const size_t blocks = align256(sizeof(float) * (size_t)g.U * g.m);
-  const size_t full = align256(2 * (size_t)g.U * g.N * kD);
+  const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD), blocks = align256(sizeof(float) * (size_t)g.U * g.m);
   size_t at = w.f.total;
-  w.lse_fg = at; at += rows;
-  w.lse_l = at; at += rows;
   w.lse_cg = at; at += blocks;
   w.delta = at; at += blocks;
   w.dob = at; at += pooled;
   w.dqm = at; at += pooled;
   w.dkm = at; at += pooled;
   w.dvm = at; at += pooled;
-  size_t* fulls[] = {&w.do_fg, &w.do_l, &w.dq_fg, &w.dq_l, &w.dk_fg, &w.dk_l, &w.dv_fg, &w.dv_l};
-  for (size_t* f : fulls) { *f = at; at += full; }
-  w.inner = at;  // the attention backward's layout starts with a status block of its own (unused here)
-  w.total = at + bwd_layout(g).total;
+  w.b = bwd_layout(g, 2, at);
   return w;
 }
 size_t select_total(const Geo& g) { return select_layout(g).total; }
@@ -159,9 +149,9 @@ size_t mosaic_bsa_workspace_bytes(const mosaic_bsa_params* p, int op) {
   switch (op) {
     case MOSAIC_OP_SELECT: return select_total(g);
     case MOSAIC_OP_FWD: return kStatusBytes;
-    case MOSAIC_OP_BWD: return bwd_layout(g).total;
+    case MOSAIC_OP_BWD: return bwd_layout(g, 1, kStatusBytes).total;
     case MOSAIC_OP_FWD_BRANCHES: return branch_layout(g).total;
-    case MOSAIC_OP_BWD_BRANCHES: return bwd_branch_layout(g).total;
+    case MOSAIC_OP_BWD_BRANCHES: return bwd_branch_layout(g).b.total;
     default: return 0;
   }
 }
@@ -192,7 +182,10 @@ int mosaic_bsa_fwd(const mosaic_bsa_params* p, const void* q, const void* k, con
       !aligned(block_idx, 4))
     return MOSAIC_E_MISALIGNED;
   if ((rc = begin(p, ws, ws_bytes, kStatusBytes, cuda_stream, &c))) return rc;
-  return launch_fwd_tc(c, q, k, v, block_idx, o, lse, c.status + 1);
+  FwdOut out = {};
+  out.o = (__nv_bfloat16*)o;
+  out.lse = lse;
+  return launch_fwd_tc(c, kFwdUnion, q, k, v, block_idx, out, c.status + 1);
 }
 
 int mosaic_bsa_fwd_branches(const mosaic_bsa_params* p, const void* q, const void* k, const void* v,
@@ -211,22 +204,20 @@ int mosaic_bsa_fwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   char* base = (char*)ws;
   float *pq = (float*)(base + w.pq), *pk = (float*)(base + w.pk), *pv = (float*)(base + w.pv);
   float *nrm = (float*)(base + w.nrm), *ocg = (float*)(base + w.ocg);
-  void *ofg = base + w.ofg, *ol = base + w.ol;
   // compression branch: pooled sums of Q, K (with their norms, unused here) and V, then block-level attention
   HostCtx cp = c;
   cp.g.topk = 0;  // pooling only
   if ((rc = launch_select(cp, q, k, nullptr, pq, pk, nrm, nrm + (size_t)g.U * g.m))) return rc;
   if ((rc = launch_pool_one(c, v, pv, nrm, g.Ukv))) return rc;
   if ((rc = launch_compress(c, pq, pk, pv, ocg, nullptr))) return rc;
-  // local branch: the neighbourhood only (no selected blocks); work queue in the second word of the status block
-  HostCtx cl = c;
-  cl.g.topk = 0;
-  if ((rc = launch_fwd_tc(cl, q, k, v, nullptr, ol, lse_l, c.status + 1))) return rc;
-  // selection branch: the selected blocks only; work queue in the third word
-  HostCtx cs = c;
-  cs.g.local_off = 1;
-  if ((rc = launch_fwd_tc(cs, q, k, v, block_idx, ofg, lse_fg, c.status + 2))) return rc;
-  return launch_combine(c, ocg, ofg, ol, gates, o);
+  // selection and local branch, each with its own softmax, and the gated sum
+  FwdOut out = {};
+  out.o = (__nv_bfloat16*)o;
+  out.lse = lse_fg;
+  out.lse_l = lse_l;
+  out.gates = gates;
+  out.ocg = ocg;
+  return launch_fwd_tc(c, kFwdBranches, q, k, v, block_idx, out, c.status + 1);
 }
 
 int mosaic_bsa_bwd(const mosaic_bsa_params* p, const void* q, const void* k, const void* v, const void* o,
@@ -243,12 +234,16 @@ int mosaic_bsa_bwd(const mosaic_bsa_params* p, const void* q, const void* k, con
     if (!aligned(x, 16)) return MOSAIC_E_MISALIGNED;
   if (!aligned(lse, 4) || !aligned(block_idx, 4)) return MOSAIC_E_MISALIGNED;
   if (2 * (size_t)g.m * sizeof(int) + (size_t)g.m * g.topk / 8 + 8 > 200 * 1024) return MOSAIC_E_UNSUPPORTED;  // transposed-pattern kernel
-  BwdWs w = bwd_layout(g);
+  const BwdWs w = bwd_layout(g, 1, kStatusBytes);
   if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c))) return rc;
   char* base = (char*)ws;
-  return launch_bwd(c, q, k, v, o, lse, d_o, block_idx, dq, dk, dv, (float*)(base + w.D),
-                    (float*)(base + w.negD), (float*)(base + w.nlse2), (int32_t*)(base + w.off),
-                    (int32_t*)(base + w.q), (int32_t*)(base + w.order), c.status + 1);
+  float *neg_d = (float*)(base + w.neg_d), *neg_lse2 = (float*)(base + w.neg_lse2);
+  if ((rc = launch_rowdot(c, o, d_o, lse, neg_d, neg_lse2))) return rc;
+  RowStats st = {};
+  st.neg_lse2 = neg_lse2;
+  st.neg_d = neg_d;
+  return launch_bwd(c, q, k, v, st, d_o, block_idx, dq, dk, dv, (int32_t*)(base + w.off), (int32_t*)(base + w.q),
+                    (int32_t*)(base + w.order), c.status + 1);
 }
 
 int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const void* k, const void* v,
@@ -266,52 +261,40 @@ int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   if (!aligned(gates, 4) || !aligned(dgates, 4) || !aligned(block_idx, 4)) return MOSAIC_E_MISALIGNED;
   if (2 * (size_t)g.m * sizeof(int) + (size_t)g.m * g.topk / 8 + 8 > 200 * 1024) return MOSAIC_E_UNSUPPORTED;  // transposed-pattern kernel
   const BwdBranchWs w = bwd_branch_layout(g);
-  if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, w.b.total, cuda_stream, &c))) return rc;
   char* base = (char*)ws;
   auto F = [&](size_t off) { return (float*)(base + off); };
   float *pq = F(w.f.pq), *pk = F(w.f.pk), *pv = F(w.f.pv), *nrm = F(w.f.nrm), *ocg = F(w.f.ocg);
-  void *ofg = base + w.f.ofg, *ol = base + w.f.ol;
-  // the forward again: pooled sums, block-level attention (with its log-sum-exp), both attention branches
+  // the forward again: pooled sums, block-level attention (with its log-sum-exp), and of the attention branches the gate
+  // gradients and row statistics
   HostCtx cp = c;
   cp.g.topk = 0;  // pooling only
   if ((rc = launch_select(cp, q, k, nullptr, pq, pk, nrm, nrm + (size_t)g.U * g.m))) return rc;
   if ((rc = launch_pool_one(c, v, pv, nrm, g.Ukv))) return rc;
   if ((rc = launch_compress(c, pq, pk, pv, ocg, F(w.lse_cg)))) return rc;
-  HostCtx cl = c;
-  cl.g.topk = 0;          // local branch: the neighbourhood only
-  HostCtx cs = c;
-  cs.g.local_off = 1;     // selection branch: the selected blocks only
-  const bool sel = g.topk > 0;
-  if ((rc = launch_fwd_tc(cl, q, k, v, nullptr, ol, F(w.lse_l), c.status + 1))) return rc;
-  if (sel) {
-    if ((rc = launch_fwd_tc(cs, q, k, v, block_idx, ofg, F(w.lse_fg), c.status + 2))) return rc;
-  } else if (cudaMemsetAsync(ofg, 0, 2 * (size_t)g.U * g.N * kD, c.stream) != cudaSuccess) {
-    return MOSAIC_E_CUDA;
-  }
-  // gate gradients, gated copies of dO, gated block sums of dO
-  if ((rc = launch_gate(c, d_o, ofg, ol, ocg, gates, dgates, base + w.do_fg, base + w.do_l, F(w.dob)))) return rc;
+  FwdOut out = {};
+  out.gates = gates;
+  out.ocg = ocg;
+  out.d_o = (const __nv_bfloat16*)d_o;
+  out.dgates = dgates;
+  out.neg_lse2 = F(w.b.neg_lse2);
+  out.neg_d = F(w.b.neg_d);
+  out.gate = F(w.b.gate);
+  if ((rc = launch_fwd_tc(c, kFwdStats, q, k, v, block_idx, out, c.status + 1))) return rc;
   // compression branch on the block level
+  if ((rc = launch_gated_pool(c, d_o, gates, F(w.dob)))) return rc;
   if ((rc = launch_compress_bwd(c, pq, pk, pv, F(w.dob), ocg, F(w.lse_cg), F(w.delta), F(w.dqm), F(w.dkm), F(w.dvm))))
     return rc;
-  // the two attention branches, one after the other on the same scratch
-  const BwdWs bw = bwd_layout(g);
-  char* in = base + w.inner;
-  auto attention_bwd = [&](const HostCtx& cx, const void* o_x, const float* lse_x, const void* do_x, const int32_t* idx,
-                           void* dq_x, void* dk_x, void* dv_x, int* counters) {
-    return launch_bwd(cx, q, k, v, o_x, lse_x, do_x, idx, dq_x, dk_x, dv_x, (float*)(in + bw.D), (float*)(in + bw.negD),
-                      (float*)(in + bw.nlse2), (int32_t*)(in + bw.off), (int32_t*)(in + bw.q), (int32_t*)(in + bw.order),
-                      counters);
-  };
-  if ((rc = attention_bwd(cl, ol, F(w.lse_l), base + w.do_l, nullptr, base + w.dq_l, base + w.dk_l, base + w.dv_l,
-                          c.status + 3)))
-    return rc;
-  if (sel && (rc = attention_bwd(cs, ofg, F(w.lse_fg), base + w.do_fg, block_idx, base + w.dq_fg, base + w.dk_fg,
-                                 base + w.dv_fg, c.status + 5)))
-    return rc;
-  // sums: both attention branches plus what the compression branch gives every token of a block
-  if ((rc = launch_grad_sum(c, g.U, base + w.dq_l, sel ? base + w.dq_fg : nullptr, F(w.dqm), dq))) return rc;
-  if ((rc = launch_grad_sum(c, g.Ukv, base + w.dk_l, sel ? base + w.dk_fg : nullptr, F(w.dkm), dk))) return rc;
-  return launch_grad_sum(c, g.Ukv, base + w.dv_l, sel ? base + w.dv_fg : nullptr, F(w.dvm), dv);
+  // both attention branches in one pass, with the block level's share added in the epilogues
+  RowStats st = {};
+  st.neg_lse2 = out.neg_lse2;
+  st.neg_d = out.neg_d;
+  st.gate = out.gate;
+  st.dqm = F(w.dqm);
+  st.dkm = F(w.dkm);
+  st.dvm = F(w.dvm);
+  return launch_bwd(c, q, k, v, st, d_o, block_idx, dq, dk, dv, (int32_t*)(base + w.b.off), (int32_t*)(base + w.b.q),
+                    (int32_t*)(base + w.b.order), c.status + 2);
 }
 
 int mosaic_bsa_rope(const mosaic_bsa_params* p, const void* q, const void* k, const float* pos, float theta, void* q_out,

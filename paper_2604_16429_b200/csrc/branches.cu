@@ -1,11 +1,10 @@
-// Compression branch and gated sum of the three-branch form of the operator.
+// Compression branch of the three-branch form of the operator.
 //
 // Paper: Eq. of the aggregated output (section "Native Sparse Attention") and the "Compression" paragraph of the
 // section "Block-Sparse Attention": block-level softmax attention abar_ij over ALL m blocks on the mean-pooled
 // queries and keys, obar_i = sum_j abar_ij vbar_j, the same vector for every token of query block i; then
 //   o_l = g_CG(l) obar_i + g_FG(l) oFG_l + g_L(l) oL_l .
-// The selection and local branch outputs oFG, oL come from two launches of the attention kernel (selected blocks
-// only / neighbourhood only, each with its own softmax).
+// The selection and local branch outputs oFG, oL and the gated sum come from the attention kernel.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -131,38 +130,6 @@ __global__ void __launch_bounds__(kCW * 32) compress_kernel(Geo g, const float* 
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// combine_kernel: o = g_CG * obar(block of the token) + g_FG * oFG + g_L * oL, eight lanes per token (16 bytes of
-// each bf16 tensor per lane), fp32 arithmetic, bf16 result.  HBM-bound: reads 2 * 128 B + 12 B per token (the
-// block's obar comes from L2), writes 128 B.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) combine_kernel(Geo g, const float* __restrict__ ocg, const uint4* __restrict__ o_fg,
-                                                      const uint4* __restrict__ o_l, const float* __restrict__ gates,
-                                                      uint4* __restrict__ o) {
-  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // token over all units
-  const int part = threadIdx.x & 7;
-  if (x >= (long long)g.U * g.N) return;
-  const int u = (int)(x / g.N);
-  const long long t = x - (long long)u * g.N;
-  const int lat = (int)(t / g.nlon), lon = (int)(t - (long long)lat * g.nlon);
-  const int blk = (lat / g.bh) * g.nbw + lon / g.bw;
-  const float gc = __ldg(gates + x * 3), gf = __ldg(gates + x * 3 + 1), gl = __ldg(gates + x * 3 + 2);
-  const float4* cg = reinterpret_cast<const float4*>(ocg + ((long long)u * g.m + blk) * kD + 8 * part);
-  const float4 c0 = __ldg(cg), c1 = __ldg(cg + 1);
-  const float cgv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-  const uint4 a = __ldg(o_fg + x * 8 + part), b = __ldg(o_l + x * 8 + part);
-  const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-  uint32_t r[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float a0, a1, b0, b1;
-    unpack16x2(av[i], g.f16 != 0, a0, a1);
-    unpack16x2(bv[i], g.f16 != 0, b0, b1);
-    r[i] = pack16x2(gc * cgv[2 * i] + gf * a0 + gl * b0, gc * cgv[2 * i + 1] + gf * a1 + gl * b1, g.f16 != 0);
-  }
-  o[x * 8 + part] = make_uint4(r[0], r[1], r[2], r[3]);
-}
-
 }  // namespace
 
 int launch_compress(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* pooled_v, float* ocg,
@@ -180,14 +147,6 @@ int launch_compress(const HostCtx& c, const float* pooled_q, const float* pooled
   }
   const int tiles = (g.m + kCW * kCR - 1) / (kCW * kCR);
   compress_kernel<<<(unsigned)(g.U * tiles), kCW * 32, smem, c.stream>>>(g, pooled_q, pooled_k, pooled_v, ocg, lse2);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
-}
-
-int launch_combine(const HostCtx& c, const float* ocg, const void* o_fg, const void* o_l, const float* gates, void* o) {
-  const Geo& g = c.g;
-  const long long blocks = ((long long)g.U * g.N * 8 + 255) / 256;
-  if (blocks > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  combine_kernel<<<(unsigned)blocks, 256, 0, c.stream>>>(g, ocg, (const uint4*)o_fg, (const uint4*)o_l, gates, (uint4*)o);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 

@@ -5,7 +5,7 @@
 // abar = softmax over all m blocks of the mean-pooled queries and keys).  With dO the gradient of o:
 //   gates:        dg_X(l) = <dO_l, oX_l>                                   (X = CG, FG, L)
 //   attention:    the selection and the local branch are softmax attentions of their own, so each takes the
-//                 attention backward with dO scaled by its gate (gate_kernel writes g_FG dO and g_L dO)
+//                 attention backward with dO scaled by its gate (both in one pass of the dQ and the dK/dV kernel)
 //   compression:  dobar_i = sum_{l in block i} g_CG(l) dO_l ;  with delta_i = <dobar_i, obar_i>,
 //                 dp_ij = <dobar_i, vbar_j>, ds_ij = abar_ij (dp_ij - delta_i):
 //                 dvbar_j = sum_i abar_ij dobar_i,  dqbar_i = scale sum_j ds_ij kbar_j,  dkbar_j = scale sum_i ds_ij qbar_i ;
@@ -20,70 +20,11 @@ namespace mosaic {
 
 namespace {
 
-__device__ __forceinline__ int token_block(const Geo& g, long long t) {
-  const int lat = (int)(t / g.nlon), lon = (int)(t - (long long)lat * g.nlon);
-  return (lat / g.bh) * g.nbw + lon / g.bw;
-}
 __device__ __forceinline__ void unpack8(const Geo& g, const uint4& v, float (&f)[8]) {
   const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) unpack16x2(x[i], g.f16 != 0, f[2 * i], f[2 * i + 1]);
 }
-__device__ __forceinline__ uint4 pack8(const Geo& g, const float (&f)[8]) {
-  uint32_t r[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r[i] = pack16x2(f[2 * i], f[2 * i + 1], g.f16 != 0);
-  return make_uint4(r[0], r[1], r[2], r[3]);
-}
-
-// ------------------------------------------------------------------------------------------
-// gate_kernel: per token the three gate gradients and the gated copies of dO for the two attention branches.
-// Eight lanes per token, 16 bytes of each bf16 tensor per lane.  HBM-bound: reads 3 * 128 B + 12 B, writes
-// 2 * 128 B + 12 B per token (the block's obar comes from L2).
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gate_kernel(Geo g, const uint4* __restrict__ d_o, const uint4* __restrict__ o_fg,
-                                                   const uint4* __restrict__ o_l, const float* __restrict__ ocg,
-                                                   const float* __restrict__ gates, float* __restrict__ dgates,
-                                                   uint4* __restrict__ do_fg, uint4* __restrict__ do_l) {
-  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // token over all units
-  const int part = threadIdx.x & 7;
-  const bool live = x < (long long)g.U * g.N;  // idle lanes of the last warp still take part in the shuffles
-  float dc = 0.f, df = 0.f, dl = 0.f;
-  if (live) {
-    const int u = (int)(x / g.N);
-    const int blk = token_block(g, x - (long long)u * g.N);
-    const float gf = __ldg(gates + x * 3 + 1), gl = __ldg(gates + x * 3 + 2);
-    const float4* cg = reinterpret_cast<const float4*>(ocg + ((long long)u * g.m + blk) * kD + 8 * part);
-    const float4 c0 = __ldg(cg), c1 = __ldg(cg + 1);
-    const float cgv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-    float go[8], a[8], b[8], sf[8], sl[8];
-    unpack8(g, __ldg(d_o + x * 8 + part), go);
-    unpack8(g, __ldg(o_fg + x * 8 + part), a);
-    unpack8(g, __ldg(o_l + x * 8 + part), b);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      dc = fmaf(go[i], cgv[i], dc);
-      df = fmaf(go[i], a[i], df);
-      dl = fmaf(go[i], b[i], dl);
-      sf[i] = gf * go[i];
-      sl[i] = gl * go[i];
-    }
-    do_fg[x * 8 + part] = pack8(g, sf);
-    do_l[x * 8 + part] = pack8(g, sl);
-  }
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    dc += __shfl_xor_sync(0xffffffffu, dc, o);
-    df += __shfl_xor_sync(0xffffffffu, df, o);
-    dl += __shfl_xor_sync(0xffffffffu, dl, o);
-  }
-  if (live && part == 0) {
-    dgates[x * 3] = dc;
-    dgates[x * 3 + 1] = df;
-    dgates[x * 3 + 2] = dl;
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // gated_pool_kernel: dobar_i = sum over the block's tokens (row-major) of g_CG dO, fp32.  Eight lanes per
 // (unit, block), eight channels per lane.  HBM-bound: reads dO once.
@@ -280,40 +221,10 @@ __global__ void __launch_bounds__(kBW * 32) compress_bwd_kernel(Geo g, const flo
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// sum_kernel: x = bf16(x_L + x_FG + xm[block of the token]) for one gradient tensor: the two attention branches'
-// gradients (bf16) plus what the compression branch gives every token of the block (fp32).  Eight lanes per
-// token.  HBM-bound: reads 2 * 128 B, writes 128 B per token.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) sum_kernel(Geo g, long long tokens, const uint4* __restrict__ x_l,
-                                                  const uint4* __restrict__ x_fg, const float* __restrict__ xm,
-                                                  uint4* __restrict__ out) {
-  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-  const int part = threadIdx.x & 7;
-  if (x >= tokens) return;
-  const long long u = x / g.N;
-  const int blk = token_block(g, x - u * g.N);
-  const float4* cm = reinterpret_cast<const float4*>(xm + (u * g.m + blk) * kD + 8 * part);
-  const float4 c0 = __ldg(cm), c1 = __ldg(cm + 1);
-  const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-  float a[8], b[8], r[8];
-  unpack8(g, __ldg(x_l + x * 8 + part), a);
-  if (x_fg) unpack8(g, __ldg(x_fg + x * 8 + part), b);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) r[i] = a[i] + (x_fg ? b[i] : 0.f) + cv[i];
-  out[x * 8 + part] = pack8(g, r);
-}
-
 }  // namespace
 
-int launch_gate(const HostCtx& c, const void* d_o, const void* o_fg, const void* o_l, const float* ocg,
-                const float* gates, float* dgates, void* do_fg, void* do_l, float* dob) {
+int launch_gated_pool(const HostCtx& c, const void* d_o, const float* gates, float* dob) {
   const Geo& g = c.g;
-  const long long blocks = ((long long)g.U * g.N * 8 + 255) / 256;
-  if (blocks > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  gate_kernel<<<(unsigned)blocks, 256, 0, c.stream>>>(g, (const uint4*)d_o, (const uint4*)o_fg, (const uint4*)o_l, ocg,
-                                                      gates, dgates, (uint4*)do_fg, (uint4*)do_l);
-  if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
   const long long pblocks = ((long long)g.U * g.m * 8 + 255) / 256;
   gated_pool_kernel<<<(unsigned)pblocks, 256, 0, c.stream>>>(g, (const uint4*)d_o, gates, dob);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
@@ -339,15 +250,6 @@ int launch_compress_bwd(const HostCtx& c, const float* pq, const float* pk, cons
   if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
   compress_bwd_kernel<true><<<(unsigned)(g.Ukv * tiles), kBW * 32, smem, c.stream>>>(g, pq, pk, pv, dob, ocg, lse2, delta,
                                                                                     dkm, dvm);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
-}
-
-int launch_grad_sum(const HostCtx& c, int units, const void* x_l, const void* x_fg, const float* xm, void* out) {
-  const Geo& g = c.g;
-  const long long tokens = (long long)units * g.N;
-  const long long blocks = (tokens * 8 + 255) / 256;
-  if (blocks > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  sum_kernel<<<(unsigned)blocks, 256, 0, c.stream>>>(g, tokens, (const uint4*)x_l, (const uint4*)x_fg, xm, (uint4*)out);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 

@@ -19,13 +19,12 @@ namespace mosaic {
 constexpr float kLog2e = 1.4426950408889634f;
 
 // ------------------------------------------------------------------------------------------
-// D_l = sum_c dO_lc * O_lc (also stored negated, with the negated base-2 log-sum-exp beside it).
+// -D_l = -sum_c dO_lc * O_lc, with the negated base-2 log-sum-exp beside it (the form the tensor-core kernels add).
 // HBM-bound: 8 lanes per token, 16 bytes of each tensor per lane.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uint4* __restrict__ o,
                                                      const uint4* __restrict__ d_o, const float* __restrict__ lse,
-                                                     float* __restrict__ D, float* __restrict__ neg_d,
-                                                     float* __restrict__ neg_lse2, bool f16) {
+                                                     float* __restrict__ neg_d, float* __restrict__ neg_lse2, bool f16) {
   long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   int part = threadIdx.x & 7;
   float acc = 0.f;
@@ -45,8 +44,7 @@ __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uin
   acc += __shfl_xor_sync(0xffffffffu, acc, 2);
   acc += __shfl_xor_sync(0xffffffffu, acc, 4);
   if (part == 0 && t < tokens) {
-    D[t] = acc;
-    neg_d[t] = -acc;                     // the key-stationary kernel reads these per query column
+    neg_d[t] = -acc;
     neg_lse2[t] = -lse[t] * kLog2e;      // log-sum-exp in base-2 units, negated
   }
 }
@@ -147,18 +145,17 @@ static int csr_segments(const Geo& g, size_t* smem) {
   return *smem <= budget ? nseg : 0;
 }
 
-int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, const void* o, const float* lse,
-               const void* d_o, const int32_t* block_idx, void* dq, void* dk, void* dv, float* Dbuf, float* neg_d,
-               float* neg_lse2,
-               int32_t* csr_off, int32_t* csr_q, int32_t* order, int* counters) {
+int launch_rowdot(const HostCtx& c, const void* o, const void* d_o, const float* lse, float* neg_d, float* neg_lse2) {
+  const long long tokens = (long long)c.g.U * c.g.N, threads = tokens * 8;
+  rowdot_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c.stream>>>(tokens, (const uint4*)o, (const uint4*)d_o, lse,
+                                                                         neg_d, neg_lse2, c.g.f16 != 0);
+  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+}
+
+int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, const RowStats& st, const void* d_o,
+               const int32_t* block_idx, void* dq, void* dk, void* dv, int32_t* csr_off, int32_t* csr_q, int32_t* order,
+               int* counters) {
   const Geo& g = c.g;
-  const long long tokens = (long long)g.U * g.N;
-  {
-    long long threads = tokens * 8;
-    rowdot_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c.stream>>>(tokens, (const uint4*)o,
-                                                                           (const uint4*)d_o, lse, Dbuf, neg_d, neg_lse2, g.f16 != 0);
-    if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
-  }
   if (g.topk > 0) {
     size_t smem = 0;
     const int nseg = csr_segments(g, &smem);
@@ -177,17 +174,10 @@ int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, co
       return MOSAIC_E_CUDA;
   }
   if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
-  {
-    // dQ on the tcgen05 path; its work queue counts in a word of the status block (zeroed when the op started)
-    const int rc = launch_dq_tc(c, q, k, v, d_o, lse, Dbuf, block_idx, dq, counters);
-    if (rc) return rc;
-  }
-  {
-    // dK, dV on the tcgen05 path; its work queue counts in the next word
-    const int rc = launch_dkdv_tc(c, q, k, v, d_o, neg_lse2, neg_d, csr_off, csr_q, dk, dv, counters + 1, order);
-    if (rc) return rc;
-  }
-  return MOSAIC_OK;
+  // the work queues count in words of the status block (zeroed when the op started)
+  const int rc = launch_dq_tc(c, q, k, v, d_o, st, block_idx, dq, counters);
+  if (rc) return rc;
+  return launch_dkdv_tc(c, q, k, v, d_o, st, csr_off, csr_q, dk, dv, counters + 1, order);
 }
 
 }  // namespace mosaic

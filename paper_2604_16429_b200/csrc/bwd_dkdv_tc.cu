@@ -37,20 +37,28 @@ constexpr int kWProd = kRowWarps, kWMma0 = kRowWarps + 1, kWMma1 = kRowWarps + 2
 constexpr uint32_t kTmemCols = 512;
 // dK, dV accumulators; per chunk of a pair S^T and dP^T (fp32, 64 columns) and P^T and dS^T (bf16 pairs, 32 columns)
 constexpr uint32_t kColDK = 0, kColDV = 64, kColS = 128, kColDP = 256, kColP = 384, kColDS = 448;
-constexpr uint32_t kChunkBytes = 2 * kTile + 2 * 64 * 4;
+// BR: backward of the three-branch form.  The local and the selected blocks have a softmax of their own, so a query row has
+// two sets of statistics, and its dO is scaled by the branch's gate: P enters dV as gate P, dS = P (gate dP - gate <dO, O>).
+// Statistics of a query row: -LSE*log2e, -D (and the gate, for the local, then for the selected blocks).
+template <bool BR>
+constexpr int kStats = BR ? 6 : 2;
+template <bool BR>
+constexpr uint32_t kChunkBytes = 2 * kTile + kStats<BR> * 64 * 4;
 
+template <bool BR>
 struct Slot {
   unsigned char q[2][kTile];     // per chunk 64 query rows x 128 B, swizzled; the two tiles form one 128-row operand
   unsigned char d_o[2][kTile];
-  float neg_lse2[2][64];         // -LSE * log2(e) of the chunks' query rows
-  float neg_d[2][64];            // -D of the chunks' query rows
+  float stat[kStats<BR>][2][64]; // statistics of the chunks' query rows
 };
-static_assert(sizeof(Slot) % 1024 == 0, "slots keep the 1024-byte alignment of the swizzled tiles");
+static_assert(sizeof(Slot<false>) % 1024 == 0 && sizeof(Slot<true>) % 1024 == 0,
+              "slots keep the 1024-byte alignment of the swizzled tiles");
 
+template <bool BR>
 struct Smem {
   unsigned char k[2 * kTile];              // 128 key rows x 128 B
   unsigned char v[2 * kTile];
-  Slot ring[kSlots];
+  Slot<BR> ring[kSlots];
   unsigned long long ring_full[kSlots], ring_empty[kSlots];
   unsigned long long kv_full, kv_empty, s_full, sdp_free, p_full[2], pv_done, acc_done, acc_free;
   unsigned long long mma_drain_bar[2];  // abort path: completion of each issuer's outstanding products
@@ -64,7 +72,8 @@ struct Smem {
 
 // Planner of the key-stationary kernel: per item (tile), the merged local neighbourhoods of its key blocks,
 // then each block's list of selecting query blocks, cut into list buffers.
-__device__ __forceinline__ void planner_kv_loop(Smem& sm, const Geo& g, const int32_t* __restrict__ csr_off,
+template <bool BR>
+__device__ __forceinline__ void planner_kv_loop(Smem<BR>& sm, const Geo& g, const int32_t* __restrict__ csr_off,
                                                 const int32_t* __restrict__ csr_q,
                                                 const int32_t* __restrict__ order, int* work_counter, int ipu,
                                                 int total_items, int lane, volatile int* abort, int* status) {
@@ -121,15 +130,15 @@ __device__ __forceinline__ void planner_kv_loop(Smem& sm, const Geo& g, const in
         if (!ok) break;
       }
       // local neighbourhoods (at most 64 entries per block, merged with masks), straight into the list buffer
-      if (use0) n = merge_block(g, -1, hb[0], bits0, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
-      if (use1) n = merge_block(g, -1, hb[1], bits1, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
+      if (use0) n = merge_block(g, true, -1, hb[0], bits0, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
+      if (use1) n = merge_block(g, true, -1, hb[1], bits1, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
       // query blocks that selected the key block (ascending ids), appended 32 at a time
       const int32_t* off = csr_off + (long long)qu * (g.m + 1);
       const int32_t* sel = csr_q + (long long)qu * g.m * g.topk;
 #pragma unroll
       for (int hh = 0; hh < 2 && ok; ++hh) {
         if (!(hh == 0 ? use0 : use1)) continue;
-        const unsigned char bits = hh == 0 ? bits0 : bits1;
+        const unsigned char bits = (unsigned char)((hh == 0 ? bits0 : bits1) << (BR ? 4 : 0));  // BR: tagged as selected
         const int s_beg = __ldg(off + hb[hh]), s_end = __ldg(off + hb[hh] + 1);
         for (int base = s_beg; base < s_end && ok; base += 32) {
           if (n + 32 > kMaxUnion) {
@@ -210,16 +219,17 @@ __global__ void __launch_bounds__(1024) dkdv_order_kernel(const Geo g, const int
     order[first_item + atomicAdd(&hist[bins[item]], 1)] = item;
 }
 
-template <bool F16>
+template <bool F16, bool BR>
 __global__ void __launch_bounds__(kThreads, 1)
     dkdv_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                    const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    const __grid_constant__ CUtensorMap map_nlse, const __grid_constant__ CUtensorMap map_nd,
-                   const int32_t* __restrict__ csr_off, const int32_t* __restrict__ csr_q,
-                   const int32_t* __restrict__ order, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv, int* status, int* work_counter,
-                   int ipu, int total_items) {
+                   const __grid_constant__ CUtensorMap map_gate, const int32_t* __restrict__ csr_off,
+                   const int32_t* __restrict__ csr_q, const int32_t* __restrict__ order, __nv_bfloat16* __restrict__ dk,
+                   __nv_bfloat16* __restrict__ dv, const float* __restrict__ dkm, const float* __restrict__ dvm,
+                   int* status, int* work_counter, int ipu, int total_items) {
   extern __shared__ unsigned char smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Smem<BR>& sm = *reinterpret_cast<Smem<BR>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
@@ -282,17 +292,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int slot = (int)(pr % kSlots), np = min(2, chunks - p0);
           ok = mbar_wait(s32(&sm.ring_empty[slot]), (uint32_t)((pr / kSlots) & 1) ^ 1, abort, status);
           if (!ok) break;
-          Slot& sl = sm.ring[slot];
+          Slot<BR>& sl = sm.ring[slot];
           const uint32_t bar = s32(&sm.ring_full[slot]);
-          mbar_expect_tx(bar, np * kChunkBytes);
+          mbar_expect_tx(bar, np * kChunkBytes<BR>);
           for (int h = 0; h < np; ++h) {
             const int e = (p0 + h) / g.cpb, c = (p0 + h) - e * g.cpb;
             const int i = sm.ids[buf][e], by = i / g.nbw, bx = i - by * g.nbw;
             const int x0 = bx * g.bw, y0 = by * g.bh + c * g.crows;
             tma_load_4d(s32(sl.q[h]), &map_q, bar, 0, x0, y0, u);
             tma_load_4d(s32(sl.d_o[h]), &map_do, bar, 0, x0, y0, u);
-            tma_load_3d(s32(sl.neg_lse2[h]), &map_nlse, bar, x0, y0, u);
-            tma_load_3d(s32(sl.neg_d[h]), &map_nd, bar, x0, y0, u);
+#pragma unroll
+            for (int pl = 0; pl < (BR ? 2 : 1); ++pl) {  // planes of the statistics: local, selected
+              tma_load_3d(s32(sl.stat[3 * pl][h]), &map_nlse, bar, x0, y0, u + pl * g.U);
+              tma_load_3d(s32(sl.stat[3 * pl + 1][h]), &map_nd, bar, x0, y0, u + pl * g.U);
+              if constexpr (BR) tma_load_3d(s32(sl.stat[3 * pl + 2][h]), &map_gate, bar, x0, y0, u + pl * g.U);
+            }
           }
         }
         if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
@@ -442,7 +456,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive(s32(&sm.sdp_free));
           continue;
         }
-        const bool connected = (sm.mask[buf][p / g.cpb] & hbit) != 0;
+        const uint32_t mk = sm.mask[buf][p / g.cpb];
+        const bool connected = ((BR ? mk | (mk >> 4) : mk) & hbit) != 0;
         uint32_t pp[16], ds[16];
         if (connected) {
           const int slot = (int)(pr % kSlots);
@@ -451,7 +466,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = mbar_wait(s32(&sm.ring_full[slot]), (uint32_t)((pr / kSlots) & 1), abort, status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          const Slot& sl = sm.ring[slot];
+          // statistics of the chunk's query columns for this half's kind of connection
+          const float(*stat)[2][64] = &sm.ring[slot].stat[BR && ((mk >> 4) & hbit) ? 3 : 0];
           uint32_t sv[32], dp[32];
           tmem_ld32(tb + col_s, sv);
           tmem_ld32(tb + col_dp, dp);
@@ -461,18 +477,27 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int i = 0; i < 32; i += 4) {
             // -LSE*log2(e) and -D of four query columns (the same for every thread: broadcast loads)
-            const float4 nl = *reinterpret_cast<const float4*>(&sl.neg_lse2[grp][32 * ch + i]);
-            const float4 nd = *reinterpret_cast<const float4*>(&sl.neg_d[grp][32 * ch + i]);
+            const float4 nl = *reinterpret_cast<const float4*>(&stat[0][grp][32 * ch + i]);
+            const float4 nd = *reinterpret_cast<const float4*>(&stat[1][grp][32 * ch + i]);
+            const float4 gt = BR ? *reinterpret_cast<const float4*>(&stat[2][grp][32 * ch + i]) : nd;
             float x0, x1, x2, x3, d0, d1, d2, d3;
             unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), scale2, pack2(nl.x, nl.y)), x0, x1);
             unpack2(fma2(pack2(__uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3])), scale2, pack2(nl.z, nl.w)), x2, x3);
             const float e0 = ex2(x0), e1 = ex2(x1), e2 = ex2(x2), e3 = ex2(x3);
-            const uint64_t t01 = add2(pack2(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1])), pack2(nd.x, nd.y));
-            const uint64_t t23 = add2(pack2(__uint_as_float(dp[i + 2]), __uint_as_float(dp[i + 3])), pack2(nd.z, nd.w));
+            const uint64_t dp01 = pack2(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1]));
+            const uint64_t dp23 = pack2(__uint_as_float(dp[i + 2]), __uint_as_float(dp[i + 3]));
+            const uint64_t g01 = pack2(gt.x, gt.y), g23 = pack2(gt.z, gt.w);
+            const uint64_t t01 = BR ? fma2(dp01, g01, pack2(nd.x, nd.y)) : add2(dp01, pack2(nd.x, nd.y));
+            const uint64_t t23 = BR ? fma2(dp23, g23, pack2(nd.z, nd.w)) : add2(dp23, pack2(nd.z, nd.w));
             unpack2(mul2(pack2(e0, e1), t01), d0, d1);
             unpack2(mul2(pack2(e2, e3), t23), d2, d3);
-            pp[i >> 1] = pack2<F16>(e0, e1);
-            pp[(i >> 1) + 1] = pack2<F16>(e2, e3);
+            float w0 = e0, w1 = e1, w2 = e2, w3 = e3;
+            if (BR) {
+              unpack2(mul2(pack2(e0, e1), g01), w0, w1);
+              unpack2(mul2(pack2(e2, e3), g23), w2, w3);
+            }
+            pp[i >> 1] = pack2<F16>(w0, w1);
+            pp[(i >> 1) + 1] = pack2<F16>(w2, w3);
             ds[i >> 1] = pack2<F16>(d0, d1);
             ds[(i >> 1) + 1] = pack2<F16>(d2, d3);
           }
@@ -512,10 +537,21 @@ __global__ void __launch_bounds__(kThreads, 1)
               uint32_t ov[16];
               tmem_ld16(tb + (which ? kColDV : kColDK) + 16 * cq, ov);
               tmem_wait_ld();
+              float x[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(ov[i]) * f;
+              if (BR) {  // what the compression branch gives every token of the block
+                const float4* add = reinterpret_cast<const float4*>(
+                    (which ? dvm : dkm) + ((long long)sm.info[buf].kvunit * g.m + sm.info[buf].hb[hh]) * kD + 16 * cq);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const float4 a = __ldg(add + i);
+                  x[4 * i] += a.x; x[4 * i + 1] += a.y; x[4 * i + 2] += a.z; x[4 * i + 3] += a.w;
+                }
+              }
               uint32_t w[8];
 #pragma unroll
-              for (int i = 0; i < 8; ++i)
-                w[i] = pack2<F16>(__uint_as_float(ov[2 * i]) * f, __uint_as_float(ov[2 * i + 1]) * f);
+              for (int i = 0; i < 8; ++i) w[i] = pack2<F16>(x[2 * i], x[2 * i + 1]);
               dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
               dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
             }
@@ -525,15 +561,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(s32(&sm.acc_free));
           ++items;
-        } else if ((sm.info[buf].hvalid >> hh) & 1) {
-          // a tile that no query block is connected to (possible when the local set is switched off): zero gradients
-          const long long tok = (long long)sm.info[buf].kvunit * g.N +
-                                chunk_token(g, sm.info[buf].hb[hh], sm.info[buf].hc[hh], (quad & 1) * 32 + lane);
-          const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-          uint4* dst_k = reinterpret_cast<uint4*>(dk + tok * kD + 16 * cq);
-          uint4* dst_v = reinterpret_cast<uint4*>(dv + tok * kD + 16 * cq);
-          dst_k[0] = zero; dst_k[1] = zero;
-          dst_v[0] = zero; dst_v[1] = zero;
         }
         item_chunks = 0;
       }
@@ -546,19 +573,21 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // `work_counter` must be zero when the kernel starts (a word of the workspace status block).
-template <bool F16>
+template <bool F16, bool BR>
 static int launch_dkdv_tc_t(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o,
-                   const float* neg_lse2, const float* neg_d, const int32_t* csr_off, const int32_t* csr_q, void* dk,
+                   const RowStats& st, const int32_t* csr_off, const int32_t* csr_q, void* dk,
                    void* dv, int* work_counter, int32_t* order) {
   const Geo& g = c.g;
-  CUtensorMap mq, mdo, mk, mv, mnl, mnd;
+  CUtensorMap mq, mdo, mk, mv, mnl, mnd, mgt;
+  const int planes = BR ? 2 : 1;
   if (!make_map(&mq, q, g, g.U) || !make_map(&mdo, d_o, g, g.U) || !make_map(&mk, k, g, g.Ukv) || !make_map(&mv, v, g, g.Ukv) ||
-      !make_map_rows(&mnl, neg_lse2, g) || !make_map_rows(&mnd, neg_d, g))
+      !make_map_rows(&mnl, st.neg_lse2, g, planes * g.U) || !make_map_rows(&mnd, st.neg_d, g, planes * g.U) ||
+      !make_map_rows(&mgt, BR ? st.gate : st.neg_d, g, planes * g.U))
     return MOSAIC_E_CUDA;
-  const size_t smem = sizeof(Smem) + 1024;
+  const size_t smem = sizeof(Smem<BR>) + 1024;
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
   int sms = 0;
-  if (const int rc = launch_setup(reinterpret_cast<const void*>(dkdv_tc_kernel<F16>), smem, &configured, &sms)) return rc;
+  if (const int rc = launch_setup(reinterpret_cast<const void*>(dkdv_tc_kernel<F16, BR>), smem, &configured, &sms)) return rc;
   const int ipu = items_per_unit(g);
   const long long total = 2ll * g.Ukv * ipu;  // one item per 128-row tile of a key/value unit
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
@@ -573,16 +602,19 @@ static int launch_dkdv_tc_t(const HostCtx& c, const void* q, const void* k, cons
   dkdv_order_kernel<<<(unsigned)((total + win_items - 1) / win_items), 1024, 0, c.stream>>>(
       g, csr_off, ipu, (int)total, (int)win_items, order, order + total);
   if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
-  dkdv_tc_kernel<F16><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mdo, mk, mv, mnl, mnd, csr_off, csr_q, order,
-                                                               (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, c.status,
-                                                               work_counter, ipu, (int)total);
+  dkdv_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
+      g, mq, mdo, mk, mv, mnl, mnd, mgt, csr_off, csr_q, order, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, st.dkm, st.dvm,
+      c.status, work_counter, ipu, (int)total);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 
-int launch_dkdv_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o,
-                   const float* neg_lse2, const float* neg_d, const int32_t* csr_off, const int32_t* csr_q, void* dk,
-                   void* dv, int* work_counter, int32_t* order) {
-  return c.g.f16 ? launch_dkdv_tc_t<true>(c, q, k, v, d_o, neg_lse2, neg_d, csr_off, csr_q, dk, dv, work_counter, order) : launch_dkdv_tc_t<false>(c, q, k, v, d_o, neg_lse2, neg_d, csr_off, csr_q, dk, dv, work_counter, order);
+int launch_dkdv_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,
+                   const int32_t* csr_off, const int32_t* csr_q, void* dk, void* dv, int* work_counter, int32_t* order) {
+  if (st.gate)
+    return c.g.f16 ? launch_dkdv_tc_t<true, true>(c, q, k, v, d_o, st, csr_off, csr_q, dk, dv, work_counter, order)
+                   : launch_dkdv_tc_t<false, true>(c, q, k, v, d_o, st, csr_off, csr_q, dk, dv, work_counter, order);
+  return c.g.f16 ? launch_dkdv_tc_t<true, false>(c, q, k, v, d_o, st, csr_off, csr_q, dk, dv, work_counter, order)
+                 : launch_dkdv_tc_t<false, false>(c, q, k, v, d_o, st, csr_off, csr_q, dk, dv, work_counter, order);
 }
 
 }  // namespace mosaic

@@ -40,18 +40,22 @@ struct Smem {
   ItemInfo info[kLists];
   int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
+  unsigned short steps[kLists][2][kMaxUnion];  // [list][tile]
   int tmp_ids[kMaxUnion];            // planner scratch: merged list before reordering
   unsigned char tmp_mask[kMaxUnion];
 };
 
 }  // namespace
 
-template <bool F16>
+// BR: backward of the three-branch form.  The local and the selected blocks have a softmax of their own, so a row has two
+// sets of statistics and its dO is scaled by the branch's gate: dS = P (gate dP - gate <dO, O>); the block's share from
+// the compression branch (dqm) is added at the end.
+template <bool F16, bool BR>
 __global__ void __launch_bounds__(kThreads, 1)
     dq_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                 const int32_t* __restrict__ block_idx, const float* __restrict__ lse, const float* __restrict__ D,
-                 __nv_bfloat16* __restrict__ dq, int* status, int* work_counter, int ipu, int total_items) {
+                 const int32_t* __restrict__ block_idx, const RowStats st, __nv_bfloat16* __restrict__ dq, int* status,
+                 int* work_counter, int ipu, int total_items) {
   extern __shared__ unsigned char smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -78,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort = &sm.abort;
 
   if (warp == 11) {
-    planner_loop(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
+    planner_loop<BR ? kPlanTagged : kPlanUnion>(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -109,6 +113,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int e = 0; e < n && ok; ++e) {
           const int j = sm.ids[buf][e], by = j / g.nbw, bx = j - by * g.nbw;
+          const uint32_t mk = who_attends(sm.mask[buf][e]);
           for (int c = 0; c < g.cpb; ++c, ++step) {
             const int st = (int)(step % kStages);
             ok = mbar_wait(s32(&sm.kv_empty[st]), (uint32_t)((step / kStages) & 1) ^ 1, abort, status);
@@ -116,6 +121,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_expect_tx(s32(&sm.kv_full[st]), 2 * kTile);
             tma_load_4d(s32(sm.kv[st][0]), &map_k, s32(&sm.kv_full[st]), 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
             tma_load_4d(s32(sm.kv[st][1]), &map_v, s32(&sm.kv_full[st]), 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
+            // a tile that does not attend this entry never looks at the stage: its release is given here
+            if (!(mk & 3u)) mbar_arrive(s32(&sm.kv_empty[st]));
+            if (!(mk & 12u)) mbar_arrive(s32(&sm.kv_empty[st]));
           }
         }
         if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
@@ -139,8 +147,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t qdesc = smem_desc(s32(sm.q[t])), dodesc = smem_desc(s32(sm.d_o[t]));
     const uint32_t tcol_dq = tmem + kColDQ + 64 * t, tcol_s = tmem + kColS + 128 * t, tcol_dp = tcol_s + 64;
     const uint32_t tcol_ds = tmem + kColDS + 32 * t;
-    const uint32_t tbits = 3u << (2 * t);
-    long long step = 0;   // ring position (all chunks, attended by this tile or not)
+    uint32_t base = 0;    // ring position of the item's first chunk
     uint32_t nt = 0;      // products started by this tile so far (phase of the per-product barriers)
     bool ok = true;
     // dQ += dS K of the product whose K chunk sits in ring stage `pst` (the previous product of this tile)
@@ -164,26 +171,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
-      int last = -1;
-      for (int e = 0; e < n; ++e)
-        if (sm.mask[buf][e] & tbits) last = e;
+      const int cnt = sm.info[buf].nsteps[t];
       // the tiles are loaded for every item; they must have landed before their buffers are handed back
       ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.q_full[t]), it & 1, abort, status));
       if (!ok) break;
-      if (last < 0 && elect_one()) mbar_arrive(s32(&sm.q_empty[t]));
+      if (cnt == 0 && elect_one()) mbar_arrive(s32(&sm.q_empty[t]));
       bool first = true, pend = false, pend_first = false;
       int pend_st = 0;
-      for (int e = 0; e < n && ok; ++e) {
-        const bool act = (sm.mask[buf][e] & tbits) != 0;
+      uint32_t pend_step = 0;
+      for (int i = 0; i < cnt && ok; ++i) {
+        uint32_t step = base + (sm.steps[buf][t][i] >> 8) * (uint32_t)g.cpb;
         for (int c = 0; c < g.cpb && ok; ++c, ++step) {
-          const int st = (int)(step % kStages);
-          ok = __all_sync(0xffffffffu,
-                          mbar_wait(s32(&sm.kv_full[st]), (uint32_t)((step / kStages) & 1), abort, status));
-          if (!ok) break;
-          if (!act) {
-            if (elect_one()) mbar_arrive(s32(&sm.kv_empty[st]));
-            continue;
+          const uint32_t st = step % kStages;
+          // across a long gap in the tile's entries the chunk only lands once the pending product frees its stage
+          if (pend && step - pend_step >= (uint32_t)kStages) {
+            issue_dq(pend_st, pend_first);
+            pend = false;
+            if (!ok) break;
           }
+          ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status));
+          if (!ok) break;
           // S and dP may be overwritten once the row threads hold the previous product's values in registers
           if (nt > 0) {
             ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.sdp_free[t]), (nt - 1) & 1, abort, status));
@@ -191,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           tc_fence_after();
           const uint64_t kdesc = smem_desc(s32(sm.kv[st][0])), vdesc = smem_desc(s32(sm.kv[st][1]));
-          const bool release_q = e == last && c == g.cpb - 1;
+          const bool release_q = i == cnt - 1 && c == g.cpb - 1;
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) umma_ss(tcol_s, qdesc + 2 * kk, kdesc + 2 * kk, idesc_nt, kk > 0);
@@ -203,11 +210,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           if (pend) issue_dq(pend_st, pend_first);  // previous product: its dS is ready or about to be
           if (!ok) break;
-          pend = true; pend_st = st; pend_first = first;
+          pend = true; pend_st = (int)st; pend_step = step; pend_first = first;
           first = false;
           ++nt;
         }
       }
+      base += (uint32_t)(n * g.cpb);
       if (ok && pend) issue_dq(pend_st, pend_first);  // the item's last product
       if (ok && elect_one()) mbar_arrive(s32(&sm.list_empty[buf]));
     }
@@ -223,7 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t ts = tmem + lane_off + kColS + 128 * t, tdp = ts + 64, tdq = tmem + lane_off + kColDQ + 64 * t;
     const uint32_t tds = tmem + lane_off + kColDS + 32 * t;
-    const uint32_t tbits = 3u << (2 * t), hbit = 1u << h;
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
     uint32_t nt = 0;
     bool ok = true;
@@ -237,15 +244,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool valid = (sm.info[buf].hvalid >> h) & 1;
       const long long tok =
           (long long)sm.info[buf].unit * g.N + chunk_token(g, sm.info[buf].hb[h], sm.info[buf].hc[h], tid & 63);
-      // log-sum-exp (in base-2 units) and D of this thread's query row
-      const float lse2 = valid ? __ldg(lse + tok) * 1.4426950408889634f : 0.f;
-      const float dv = valid ? __ldg(D + tok) : 0.f;
-      const uint64_t neg_lse2 = pack2(-lse2, -lse2), neg_d2 = pack2(-dv, -dv);
-      uint32_t done = 0;
-      for (int e = 0; e < n && ok; ++e) {
-        const uint32_t mk = sm.mask[buf][e];
-        if (!(mk & tbits)) continue;
-        const bool attends = (mk & hbit) != 0;
+      // negated log-sum-exp (in base-2 units), negated D and gate of this thread's query row, per branch
+      float nl[2], nd[2], gt[2];
+#pragma unroll
+      for (int x = 0; x < (BR ? 2 : 1); ++x) {
+        const long long at = (x ? (long long)g.U * g.N : 0) + tok;
+        nl[x] = valid ? __ldg(st.neg_lse2 + at) : 0.f;
+        nd[x] = valid ? __ldg(st.neg_d + at) : 0.f;
+        gt[x] = BR && valid ? __ldg(st.gate + at) : 0.f;
+      }
+      uint64_t neg_lse2 = pack2(nl[0], nl[0]), neg_d2 = pack2(nd[0], nd[0]), gate2 = pack2(gt[0], gt[0]);
+      const int cnt = sm.info[buf].nsteps[t];
+      const unsigned short* steps = sm.steps[buf][t];
+      for (int i0 = 0; i0 < cnt && ok; ++i0) {
+        const uint32_t code = steps[i0];
+        const bool attends = (code >> hh) & 1u;
+        if (BR) {
+          const bool sel = (code >> (2 + hh)) & 1u;
+          const float a = sel ? nl[1] : nl[0], b = sel ? nd[1] : nd[0], c = sel ? gt[1] : gt[0];
+          neg_lse2 = pack2(a, a);
+          neg_d2 = pack2(b, b);
+          gate2 = pack2(c, c);
+        }
         for (int c = 0; c < g.cpb; ++c) {
           ok = mbar_wait(s32(&sm.s_full[t]), nt & 1, abort, status);
           ok = __all_sync(0xffffffffu, ok);
@@ -266,7 +286,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int i = 0; i < 64; i += 2) {
               float x0, x1, d0, d1;
               unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), scale2, neg_lse2), x0, x1);
-              const uint64_t dmd = add2(pack2(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1])), neg_d2);
+              const uint64_t dp2 = pack2(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1]));
+              const uint64_t dmd = BR ? fma2(dp2, gate2, neg_d2) : add2(dp2, neg_d2);
               unpack2(mul2(pack2(ex2(x0), ex2(x1)), dmd), d0, d1);
               pk[i >> 1] = pack2<F16>(d0, d1);
             }
@@ -277,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int i = 0; i < 32; ++i) pk[i] = 0u;
           }
           // dS has one buffer: the previous product's dQ += dS K must have consumed it
-          if (done > 0) {
+          if (i0 + c > 0) {
             ok = mbar_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -288,11 +309,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_before();
           mbar_arrive(s32(&sm.p_full[t]));
           ++nt;
-          ++done;
         }
       }
       if (!ok) break;
-      if (done > 0) {
+      if (cnt > 0) {
         ok = mbar_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -304,20 +324,24 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t ov[32];
             tmem_ld32(tdq + 32 * part, ov);
             tmem_wait_ld();
-            uint32_t w[16];
+            float v[32];
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              w[i] = pack2<F16>(__uint_as_float(ov[2 * i]) * g.scale, __uint_as_float(ov[2 * i + 1]) * g.scale);
+            for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(ov[i]) * g.scale;
+            if (BR) {
+              const float4* add = reinterpret_cast<const float4*>(
+                  st.dqm + ((long long)sm.info[buf].unit * g.m + sm.info[buf].hb[h]) * kD + 32 * part);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float4 x = __ldg(add + i);
+                v[4 * i] += x.x; v[4 * i + 1] += x.y; v[4 * i + 2] += x.z; v[4 * i + 3] += x.w;
+              }
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-              dst[part * 4 + i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+              dst[part * 4 + i] = make_uint4(pack2<F16>(v[8 * i], v[8 * i + 1]), pack2<F16>(v[8 * i + 2], v[8 * i + 3]),
+                                             pack2<F16>(v[8 * i + 4], v[8 * i + 5]), pack2<F16>(v[8 * i + 6], v[8 * i + 7]));
           }
         }
-      } else if (valid) {
-        // a tile whose rows attend nothing (possible when the local set is switched off): zero gradient
-        uint4* dst = reinterpret_cast<uint4*>(dq + tok * kD);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
       }
       tc_fence_before();
       __syncwarp();
@@ -328,9 +352,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // `work_counter` must be zero when the kernel starts (a word of the workspace status block).
-template <bool F16>
-static int launch_dq_tc_t(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* D, const int32_t* block_idx, void* dq, int* work_counter) {
+template <bool F16, bool BR>
+static int launch_dq_tc_t(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o,
+                          const RowStats& st, const int32_t* block_idx, void* dq, int* work_counter) {
   const Geo& g = c.g;
   CUtensorMap mq, mdo, mk, mv;
   if (!make_map(&mq, q, g, g.U) || !make_map(&mdo, d_o, g, g.U) || !make_map(&mk, k, g, g.Ukv) || !make_map(&mv, v, g, g.Ukv))
@@ -338,20 +362,23 @@ static int launch_dq_tc_t(const HostCtx& c, const void* q, const void* k, const 
   const size_t smem = sizeof(Smem) + 1024;
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
   int sms = 0;
-  if (const int rc = launch_setup(reinterpret_cast<const void*>(dq_tc_kernel<F16>), smem, &configured, &sms)) return rc;
+  if (const int rc = launch_setup(reinterpret_cast<const void*>(dq_tc_kernel<F16, BR>), smem, &configured, &sms)) return rc;
   const int ipu = items_per_unit(g);
   const long long total = (long long)g.U * ipu;
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
   const long long grid = total < (long long)sms ? total : (long long)sms;
-  dq_tc_kernel<F16><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mdo, mk, mv, block_idx, lse, D,
-                                                             (__nv_bfloat16*)dq, c.status, work_counter, ipu,
-                                                             (int)total);
+  dq_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
+      g, mq, mdo, mk, mv, block_idx, st, (__nv_bfloat16*)dq, c.status, work_counter, ipu, (int)total);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 
-int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* D, const int32_t* block_idx, void* dq, int* work_counter) {
-  return c.g.f16 ? launch_dq_tc_t<true>(c, q, k, v, d_o, lse, D, block_idx, dq, work_counter) : launch_dq_tc_t<false>(c, q, k, v, d_o, lse, D, block_idx, dq, work_counter);
+int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,
+                 const int32_t* block_idx, void* dq, int* work_counter) {
+  if (st.gate)
+    return c.g.f16 ? launch_dq_tc_t<true, true>(c, q, k, v, d_o, st, block_idx, dq, work_counter)
+                   : launch_dq_tc_t<false, true>(c, q, k, v, d_o, st, block_idx, dq, work_counter);
+  return c.g.f16 ? launch_dq_tc_t<true, false>(c, q, k, v, d_o, st, block_idx, dq, work_counter)
+                 : launch_dq_tc_t<false, false>(c, q, k, v, d_o, st, block_idx, dq, work_counter);
 }
 
 }  // namespace mosaic

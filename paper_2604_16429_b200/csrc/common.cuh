@@ -27,7 +27,6 @@ struct Geo {
   int cpb;          // 64-token chunks per block (b / 64)
   int crows;        // grid rows per chunk (64 / bw)
   int rlat, rlon, topk;
-  int local_off;    // 1: the local neighbourhood is not attended (selection branch of the three-branch form)
   int local_groups; // 1: the local set is the aligned group of rlat x rlon blocks that holds the block
   int f16;          // 1: the 16-bit tensors are IEEE binary16, 0: bf16
   float scale;      // softmax scale
@@ -130,30 +129,45 @@ struct SelectWs { size_t pq, pk, nq, nk, total; };
 SelectWs select_layout(const Geo& g);
 int launch_select(const HostCtx& c, const void* q, const void* k, int32_t* block_idx, float* pooled_q,
                   float* pooled_k, float* norm_q, float* norm_k);
-int launch_fwd_tc(const HostCtx& c, const void* q, const void* k, const void* v, const int32_t* block_idx,
-                  void* o, float* lse, int* work_counter);
+// What the attention kernel computes: kFwdUnion one softmax over local and selected blocks (o, lse); kFwdBranches the
+// gated sum of the three branches (o, lse of the selection branch, lse_l of the local one; reads gates and the block-level
+// output ocg); kFwdStats only what the three-branch backward needs of the forward: the gate gradients and, in two planes
+// of [U, N] (local, selected), the negated base-2 log-sum-exp, -gate * <dO, O> and the gate.
+enum { kFwdUnion = 0, kFwdBranches = 1, kFwdStats = 2 };
+struct FwdOut {
+  __nv_bfloat16* o;
+  float *lse, *lse_l;
+  const float *gates, *ocg;
+  const __nv_bfloat16* d_o;
+  float *dgates, *neg_lse2, *neg_d, *gate;
+};
+int launch_fwd_tc(const HostCtx& c, int mode, const void* q, const void* k, const void* v, const int32_t* block_idx,
+                  const FwdOut& out, int* work_counter);
 // Layout of the three-branch forward's scratch behind the status block
-struct BranchWs { size_t pq, pk, pv, nrm, ocg, ofg, ol, total; };
+struct BranchWs { size_t pq, pk, pv, nrm, ocg, total; };
 BranchWs branch_layout(const Geo& g);
 int launch_pool_one(const HostCtx& c, const void* x, float* pooled, float* norm, int units);
 // `lse2` (may be null): base-2 log-sum-exp of every query block's block-level logits, [U, m]
 int launch_compress(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* pooled_v, float* ocg,
                     float* lse2);
 // backward of the three-branch form (branches_bwd.cu)
-int launch_gate(const HostCtx& c, const void* d_o, const void* o_fg, const void* o_l, const float* ocg,
-                const float* gates, float* dgates, void* do_fg, void* do_l, float* dob);
+int launch_gated_pool(const HostCtx& c, const void* d_o, const float* gates, float* dob);
 int launch_compress_bwd(const HostCtx& c, const float* pq, const float* pk, const float* pv, const float* dob,
                         const float* ocg, const float* lse2, float* delta, float* dqm, float* dkm, float* dvm);
 int launch_rope(const HostCtx& c, const void* q, const void* k, const float* pos, double theta, void* q_out, void* k_out);
-int launch_grad_sum(const HostCtx& c, int units, const void* x_l, const void* x_fg, const float* xm, void* out);
-int launch_combine(const HostCtx& c, const float* ocg, const void* o_fg, const void* o_l, const float* gates, void* o);
-int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* D, const int32_t* block_idx, void* dq, int* work_counter);
-int launch_dkdv_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o,
-                   const float* neg_lse2, const float* neg_d, const int32_t* csr_off, const int32_t* csr_q, void* dk,
-                   void* dv, int* work_counter, int32_t* order);
-int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, const void* o, const float* lse,
-               const void* d_o, const int32_t* block_idx, void* dq, void* dk, void* dv, float* Dbuf, float* neg_d,
-               float* neg_lse2, int32_t* csr_off, int32_t* csr_q, int32_t* order, int* counters);
+// What the attention backward reads per query row, [U, N] fp32: the negated base-2 log-sum-exp and -<dO, O>.  Three-branch
+// form (gate set): two planes of each (local blocks, selected blocks), the second of them scaled by the gate, the gates
+// themselves, and what the compression branch gives every token of a block: dqm [U, m, d], dkm, dvm [Ukv, m, d].
+struct RowStats {
+  const float *neg_lse2, *neg_d, *gate, *dqm, *dkm, *dvm;
+};
+int launch_rowdot(const HostCtx& c, const void* o, const void* d_o, const float* lse, float* neg_d, float* neg_lse2);
+int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,
+                 const int32_t* block_idx, void* dq, int* work_counter);
+int launch_dkdv_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,
+                   const int32_t* csr_off, const int32_t* csr_q, void* dk, void* dv, int* work_counter, int32_t* order);
+int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, const RowStats& st, const void* d_o,
+               const int32_t* block_idx, void* dq, void* dk, void* dv, int32_t* csr_off, int32_t* csr_q, int32_t* order,
+               int* counters);
 
 }  // namespace mosaic

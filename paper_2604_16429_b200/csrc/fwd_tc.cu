@@ -36,6 +36,8 @@
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
 
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace mosaic {
@@ -64,18 +66,62 @@ struct Smem {
   ItemInfo info[kLists];
   int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
+  unsigned short steps[kLists][2][kMaxUnion];  // [list][tile]
   int tmp_ids[kMaxUnion];            // planner scratch: merged list before reordering
   unsigned char tmp_mask[kMaxUnion];
 };
 
+// 32 channels of a token's output row (fp32 in `a`) times f, stored in 16 bits; `add`: plus the row that `dst` holds already
+// and gc times the block-level vector cg.
+template <bool F16>
+__device__ __forceinline__ void store_row(uint4* dst, const uint32_t* a, float f, bool add, float gc, const float* cg) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    float v[8];
+#pragma unroll
+    for (int y = 0; y < 8; ++y) v[y] = __uint_as_float(a[8 * x + y]) * f;
+    if (add) {
+      const uint4 old = dst[x];
+      const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+      const float4 c0 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x), c1 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x + 1);
+      const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        float lo, hi;
+        unpack16x2(ow[y], F16, lo, hi);
+        v[2 * y] += lo + gc * cv[2 * y];
+        v[2 * y + 1] += hi + gc * cv[2 * y + 1];
+      }
+    }
+    dst[x] = make_uint4(pack2<F16>(v[0], v[1]), pack2<F16>(v[2], v[3]), pack2<F16>(v[4], v[5]), pack2<F16>(v[6], v[7]));
+  }
+}
+// 32 channels of <dO, O> and of <dO, block-level vector>
+template <bool F16>
+__device__ __forceinline__ void dot_row(const uint4* d_o, const uint32_t* a, const float* cg, float& dot, float& dotc) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const uint4 w = __ldg(d_o + x);
+    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+    const float4 c0 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x), c1 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x + 1);
+    const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      float lo, hi;
+      unpack16x2(ww[y], F16, lo, hi);
+      dot = fmaf(lo, __uint_as_float(a[8 * x + 2 * y]), fmaf(hi, __uint_as_float(a[8 * x + 2 * y + 1]), dot));
+      dotc = fmaf(lo, cv[2 * y], fmaf(hi, cv[2 * y + 1], dotc));
+    }
+  }
+}
+
 }  // namespace
 
-template <bool F16>
+template <bool F16, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ block_idx,
-                  __nv_bfloat16* __restrict__ o, float* __restrict__ lse, int* status, int* work_counter,
-                  int ipu, int total_items) {
+                  const __grid_constant__ FwdOut out, int* status, int* work_counter, int ipu, int total_items) {
   extern __shared__ unsigned char smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -106,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort = &sm.abort;
 
   if (warp == 11) {
-    planner_loop(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
+    planner_loop<MODE == kFwdUnion ? kPlanUnion : kPlanSplit>(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -172,8 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int t = warp - 9;
     constexpr uint32_t idesc_qk = make_idesc(false, 64u, F16), idesc_pv = make_idesc(true, 64u, F16);
     const uint32_t tcol_o = tmem + kColO + 64 * t, tcol_s = tmem + kColS + 128 * t, tcol_q = tmem + kColQ + 32 * t;
-    const uint32_t tbits = 3u << (2 * t);
-    long long step = 0;   // ring position (all chunks, attended by this tile or not)
+    uint32_t base = 0;    // ring position of the item's first chunk
     uint32_t nt = 0;      // products issued by this tile so far: buffer nt & 1, phase (nt >> 1) & 1
     bool ok = true;
     // P V of product `pn` (its V chunk sits in ring stage `pst`); `pfirst` starts a new accumulation
@@ -203,14 +248,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.q_ready[t]), it & 1, abort, status));
       if (!ok) break;
       bool first = true, pend = false, pend_first = false;
-      uint32_t pend_n = 0;
+      uint32_t pend_n = 0, pend_step = 0;
       int pend_st = 0;
-      for (int e = 0; e < n && ok; ++e) {
-        if (!(sm.mask[buf][e] & tbits)) { step += g.cpb; continue; }  // not attended: the producer released the stages
+      const int cnt = sm.info[buf].nsteps[t];
+      for (int i = 0; i < cnt && ok; ++i) {
+        uint32_t step = base + (sm.steps[buf][t][i] >> 8) * (uint32_t)g.cpb;
         for (int c = 0; c < g.cpb && ok; ++c, ++step) {
-          const int st = (int)(step % kStages);
-          ok = __all_sync(0xffffffffu,
-                          mbar_wait(s32(&sm.kv_full[st]), (uint32_t)((step / kStages) & 1), abort, status));
+          const uint32_t st = step % kStages;
+          // across a long gap in the tile's entries the chunk only lands once the pending P V frees its stage
+          if (pend && step - pend_step >= (uint32_t)kStages) {
+            issue_pv(pend_n, pend_st, pend_first);
+            pend = false;
+            if (!ok) break;
+          }
+          ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status));
           if (!ok) break;
           // S buffer nt & 1 (aliased by P) was last read by P V of product nt - 2, which this warp issued
           // earlier: tensor-core operations of one thread execute in issue order, so this QK^T cannot
@@ -226,11 +277,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           __syncwarp();
           if (pend) issue_pv(pend_n, pend_st, pend_first);
-          pend = true; pend_n = nt; pend_st = st; pend_first = first;
+          pend = true; pend_n = nt; pend_st = (int)st; pend_step = step; pend_first = first;
           first = false;
           ++nt;
         }
       }
+      base += (uint32_t)(n * g.cpb);
       if (ok && pend) issue_pv(pend_n, pend_st, pend_first);  // the item's last product
       if (ok && elect_one()) mbar_arrive(s32(&sm.list_empty[buf]));
     }
@@ -246,7 +298,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t ts = tmem + lane_off + kColS + 128 * t, to = tmem + lane_off + kColO + 64 * t;
     const uint32_t tq = tmem + lane_off + kColQ + 32 * t;
-    const uint32_t tbits = 3u << (2 * t), hbit = 1u << h;
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
     uint32_t nt = 0;
     bool ok = true;
@@ -280,11 +331,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int it = 0; ok && n >= 0; ++it) {
       const int buf = it % kLists;
       float m_ref = -INFINITY, l = 0.f;
-      uint32_t done = 0;
-      for (int e = 0; e < n && ok; ++e) {
-        const uint32_t mk = sm.mask[buf][e];
-        if (!(mk & tbits)) continue;
-        const bool attends = (mk & hbit) != 0;
+      const unsigned short* steps = sm.steps[buf][t];
+      const int cnt = sm.info[buf].nsteps[t];
+      for (int i0 = 0; i0 < cnt && ok; ++i0) {
+        const bool attends = (steps[i0] >> hh) & 1u;
         for (int c = 0; c < g.cpb; ++c) {
           const uint32_t b = nt & 1, tsb = ts + 64 * b;
           ok = mbar_wait(s32(&sm.s_full[t][b]), (nt >> 1) & 1, abort, status);
@@ -356,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             l += s0 + s1;
             if (__any_sync(0xffffffffu, need)) {
               // the accumulator may only be touched between P V products: wait for the previous one
-              if (done > 0) {
+              if (i0 + c > 0) {
                 ok = mbar_wait(s32(&sm.pv_done[t][b ^ 1]), ((nt - 1) >> 1) & 1, abort, status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -388,7 +438,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_before();
           mbar_arrive(s32(&sm.p_full[t][b]));
           ++nt;
-          ++done;
         }
       }
       if (!ok) break;
@@ -396,40 +445,50 @@ __global__ void __launch_bounds__(kThreads, 1)
       // and its first products run while this item's output is written
       const int n_next = stage_q(it + 1);
       if (!ok) break;
-      if (done > 0) {
+      if (cnt > 0) {
         ok = mbar_wait(s32(&sm.pv_done[t][(nt - 1) & 1]), ((nt - 1) >> 1) & 1, abort, status);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        if ((sm.info[buf].hvalid >> h) & 1) {
-          const int e = tid & 63;
-          const long long tok =
-              (long long)sm.info[buf].unit * g.N + chunk_token(g, sm.info[buf].hb[h], sm.info[buf].hc[h], e);
-          const float inv = l > 0.f ? 1.f / l : 0.f;  // a row that attends nothing (empty selection): O = 0
-          uint4* dst = reinterpret_cast<uint4*>(o + tok * kD);
+      }
+      if ((sm.info[buf].hvalid >> h) & 1) {
+        const int u = sm.info[buf].unit, blk = sm.info[buf].hb[h], branch = sm.info[buf].branch;
+        const long long tok = (long long)u * g.N + chunk_token(g, blk, sm.info[buf].hc[h], tid & 63);
+        const float inv = l > 0.f ? 1.f / l : 0.f;  // a row that attends nothing (empty selection): O = 0
+        const float lse2 = l > 0.f ? m_ref + log2f(l) : -INFINITY;
+        const float* cg = MODE == kFwdUnion ? nullptr : out.ocg + ((long long)u * g.m + blk) * kD;
+        const float gx = MODE == kFwdUnion ? 1.f : __ldg(out.gates + 3 * tok + 1 + branch);
+        const float gc = MODE == kFwdBranches && branch ? __ldg(out.gates + 3 * tok) : 0.f;
+        float dot = 0.f, dotc = 0.f;
 #pragma unroll
-          for (int part = 0; part < 2; ++part) {
-            uint32_t ov[32];
+        for (int part = 0; part < 2; ++part) {
+          uint32_t ov[32];
+          if (cnt > 0) {  // (the same for the whole warp)
             tmem_ld32(to + 32 * part, ov);
             tmem_wait_ld();
-            uint32_t w[16];
+          } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              w[i] = pack2<F16>(__uint_as_float(ov[2 * i]) * inv, __uint_as_float(ov[2 * i + 1]) * inv);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              dst[part * 4 + i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+            for (int x = 0; x < 32; ++x) ov[x] = 0u;
           }
-          lse[tok] = l > 0.f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+          if (MODE == kFwdStats)
+            dot_row<F16>(reinterpret_cast<const uint4*>(out.d_o + tok * kD) + 4 * part, ov, cg + 32 * part, dot, dotc);
+          else
+            store_row<F16>(reinterpret_cast<uint4*>(out.o + tok * kD) + 4 * part, ov, inv * gx,
+                           MODE == kFwdBranches && branch == 1, gc, cg + 32 * part);
         }
-      } else if ((sm.info[buf].hvalid >> h) & 1) {
-        // the tile attends nothing in this item (selection branch with empty rows): O = 0, log-sum-exp = -inf
-        const long long tok =
-            (long long)sm.info[buf].unit * g.N + chunk_token(g, sm.info[buf].hb[h], sm.info[buf].hc[h], tid & 63);
-        uint4* dst = reinterpret_cast<uint4*>(o + tok * kD);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-        lse[tok] = -INFINITY;
+        if (MODE == kFwdUnion) {
+          out.lse[tok] = lse2 * 0.6931471805599453f;
+        } else if (MODE == kFwdBranches) {
+          (branch ? out.lse_l : out.lse)[tok] = lse2 * 0.6931471805599453f;
+        } else {
+          dot *= inv;
+          out.dgates[3 * tok + 1 + branch] = dot;
+          if (branch) out.dgates[3 * tok] = dotc;
+          const long long at = (branch ? 0 : (long long)g.U * g.N) + tok;  // plane 0: local, plane 1: selected
+          out.neg_lse2[at] = -lse2;
+          out.neg_d[at] = -gx * dot;
+          out.gate[at] = gx;
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -442,32 +501,37 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ---------------------------------------------------------------------------------------------
 namespace {
-template <bool F16>
+template <bool F16, int MODE>
 int launch_fwd_tc_t(const HostCtx& c, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                    const int32_t* block_idx, void* o, float* lse, int* work_counter) {
+                    const int32_t* block_idx, const FwdOut& out, int* work_counter) {
   const Geo& g = c.g;
   const size_t smem = sizeof(Smem) + 1024;
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
   int sms = 0;
-  if (const int rc = launch_setup(reinterpret_cast<const void*>(fwd_tc_kernel<F16>), smem, &configured, &sms)) return rc;
+  if (const int rc = launch_setup(reinterpret_cast<const void*>(fwd_tc_kernel<F16, MODE>), smem, &configured, &sms)) return rc;
   const int ipu = items_per_unit(g);
   const long long total = (long long)g.U * ipu;
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
   const long long grid = total < (long long)sms ? total : (long long)sms;
-  fwd_tc_kernel<F16><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mk, mv, block_idx, (__nv_bfloat16*)o, lse,
-                                                                  c.status, work_counter, ipu, (int)total);
+  fwd_tc_kernel<F16, MODE><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mk, mv, block_idx, out, c.status,
+                                                                        work_counter, ipu, (int)total);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 }  // namespace
 
 // `work_counter` must be zero when the kernel starts (a word of the workspace status block).
-int launch_fwd_tc(const HostCtx& c, const void* q, const void* k, const void* v, const int32_t* block_idx, void* o,
-                  float* lse, int* work_counter) {
+int launch_fwd_tc(const HostCtx& c, int mode, const void* q, const void* k, const void* v, const int32_t* block_idx,
+                  const FwdOut& out, int* work_counter) {
   const Geo& g = c.g;
   CUtensorMap mq, mk, mv;
   if (!make_map(&mq, q, g, g.U) || !make_map(&mk, k, g, g.Ukv) || !make_map(&mv, v, g, g.Ukv)) return MOSAIC_E_CUDA;
-  return g.f16 ? launch_fwd_tc_t<true>(c, mq, mk, mv, block_idx, o, lse, work_counter)
-               : launch_fwd_tc_t<false>(c, mq, mk, mv, block_idx, o, lse, work_counter);
+  auto go = [&](auto f16) {
+    constexpr bool F16 = decltype(f16)::value;
+    return mode == kFwdUnion      ? launch_fwd_tc_t<F16, kFwdUnion>(c, mq, mk, mv, block_idx, out, work_counter)
+           : mode == kFwdBranches ? launch_fwd_tc_t<F16, kFwdBranches>(c, mq, mk, mv, block_idx, out, work_counter)
+                                  : launch_fwd_tc_t<F16, kFwdStats>(c, mq, mk, mv, block_idx, out, work_counter);
+  };
+  return g.f16 ? go(std::true_type{}) : go(std::false_type{});
 }
 
 }  // namespace mosaic

@@ -19,7 +19,6 @@ constexpr long long kSpinCycles = MOSAIC_TEST_SPIN_CYCLES;
 #else
 constexpr long long kSpinCycles = 4000000000ll;  // bound of a single wait (~2 s)
 #endif
-constexpr uint32_t kSuspendHintNs = 20000;       // longest park of one mbarrier poll
 
 struct ItemInfo {
   int n;        // entries of the merged list; -1 = no more work
@@ -28,6 +27,8 @@ struct ItemInfo {
   int hb[4];    // query block of half h
   int hc[4];    // 64-token chunk of that block
   int more;     // 1: the item's list continues in the next list buffer (lists longer than a buffer)
+  int nsteps[2]; // entries that tile 0 and tile 1 attend
+  int branch;   // split lists: 0 = the selected blocks, 1 = the local ones
   int kvunit;   // key-stationary kernel: the key/value unit of the item's tile (`unit` is the query unit of this buffer's list)
 };
 
@@ -42,14 +43,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// One poll.  The time hint lets the hardware park the thread for up to that long (it wakes as soon as the
-// phase completes), so warps that wait do not take issue slots from warps that work.
+// One poll.  The hardware parks the thread (for about 8000 cycles at most; it wakes as soon as the phase completes), so
+// warps that wait do not take issue slots from warps that work.  No time hint: with one the wake-up takes 120 cycles
+// after the arrival instead of 90.
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
+      : "r"(bar), "r"(parity)
       : "memory");
   return ok != 0;
 }
@@ -367,14 +369,15 @@ __device__ __forceinline__ int item_halves(const Geo& g, int it, int (&hb)[4], i
   return valid;
 }
 
-// Warp-cooperative attended list of query block i (local set, then valid selected ids) written to
+// Warp-cooperative attended list of query block i (local set if with_local, then valid selected ids) written to
 // ids[n0..); returns the new count.  `j` is this lane's entry of the block's row of block_idx (-1 beyond top-k).
-__device__ __forceinline__ int warp_attended(const Geo& g, int j, int i, int* ids, int n0, int lane, int* status) {
+__device__ __forceinline__ int warp_attended(const Geo& g, bool with_local, int j, int i, int* ids, int n0, int lane,
+                                             int* status) {
   const int by = i / g.nbw, bx = i - by * g.nbw;
   int id = -1 - lane;  // lanes without a block hold distinct negative values
   int nl;
   if (g.local_groups) {   // the aligned group of rlat x rlon blocks that holds block i (ragged at the grid's edge)
-    nl = g.local_off ? 0 : g.rlat * g.rlon;
+    nl = with_local ? g.rlat * g.rlon : 0;
     if (lane < nl) {
       const int dy = lane / g.rlon, dx = lane - dy * g.rlon;
       const int y = (by / g.rlat) * g.rlat + dy, x = (bx / g.rlon) * g.rlon + dx;
@@ -382,7 +385,7 @@ __device__ __forceinline__ int warp_attended(const Geo& g, int j, int i, int* id
     }
   } else {
     const int wl = 2 * g.rlon + 1;
-    nl = g.local_off ? 0 : (2 * g.rlat + 1) * wl;
+    nl = with_local ? (2 * g.rlat + 1) * wl : 0;
     if (lane < nl) {
       const int dy = lane / wl - g.rlat, dx = lane - (lane / wl) * wl - g.rlon;
       const int y = min(max(by + dy, 0), g.nbh - 1);
@@ -409,11 +412,11 @@ __device__ __forceinline__ int warp_attended(const Geo& g, int j, int i, int* id
 
 // Merge the attended list of query block `blk` into the item's list (ids/mask, n entries so far):
 // entries already present get `bits` OR-ed into their mask, new ones are appended.  Returns the new n.
-// `jsel` is this lane's entry of the block's row of block_idx (-1 beyond top-k).
-__device__ __forceinline__ int merge_block(const Geo& g, int jsel, int blk, unsigned char bits, int* ids,
+// `jsel` is this lane's entry of the block's row of block_idx (-1 beyond top-k, or where only the local set is wanted).
+__device__ __forceinline__ int merge_block(const Geo& g, bool with_local, int jsel, int blk, unsigned char bits, int* ids,
                                            unsigned char* mask, int n, int lane, int* status) {
   const int n0 = n;
-  const int nb = warp_attended(g, jsel, blk, ids, n0, lane, status) - n0;  // staged behind the list
+  const int nb = warp_attended(g, with_local, jsel, blk, ids, n0, lane, status) - n0;  // staged behind the list
   __syncwarp();
   if (n0 == 0) {
     for (int e = lane; e < nb; e += 32) mask[e] = bits;
@@ -464,6 +467,9 @@ __device__ __forceinline__ bool elect_one() {
 // tile attends alternate with products only its lower half attends, and since S is double-buffered the idle
 // half's warps run ahead into the next product.  The order of a softmax sum does not matter to the result
 // beyond rounding; the order is a function of the list alone.
+// An entry's mask: bit h = half h attends it; in tagged lists bit 4 + h = half h attends it as a selected block, bit h as
+// a local one.
+__device__ __forceinline__ unsigned who_attends(unsigned m) { return (m | (m >> 4)) & 15u; }
 __device__ __forceinline__ int list_class(unsigned m) {
   const unsigned t0 = m & 3u, t1 = (m >> 2) & 3u;
   return t1 == 0u ? (int)t0 - 1 : t0 == 0u ? 3 + (int)t1 : 3;
@@ -476,7 +482,7 @@ __device__ __forceinline__ void interleave_tiles(const int* sid, const unsigned 
   for (int y = 0; y < NC; ++y) cnt[y] = 0;
   for (int e0 = 0; e0 < n; e0 += 32) {
     const int e = e0 + lane;
-    const int cls = e < n ? list_class(smask[e]) : -1;
+    const int cls = e < n ? list_class(who_attends(smask[e])) : -1;
 #pragma unroll
     for (int y = 0; y < NC; ++y) cnt[y] += __popc(__ballot_sync(0xffffffffu, cls == y));
   }
@@ -486,7 +492,7 @@ __device__ __forceinline__ void interleave_tiles(const int* sid, const unsigned 
   for (int e0 = 0; e0 < n; e0 += 32) {
     const int e = e0 + lane;
     const unsigned m = e < n ? smask[e] : 0u;
-    const int cls = e < n ? list_class(m) : -1;
+    const int cls = e < n ? list_class(who_attends(m)) : -1;
     const unsigned lower = (1u << lane) - 1u;
     int k = 0, nx = 1;
 #pragma unroll
@@ -515,25 +521,53 @@ __device__ __forceinline__ void interleave_tiles(const int* sid, const unsigned 
   __syncwarp();
 }
 
+// The entries of an item's list that each tile attends: per entry the tile's halves (bits 0, 1), whether they attend it as
+// a selected block (bits 2, 3, tagged lists) and, from bit 8, the entry's place in the list.
+__device__ __forceinline__ void tile_steps(const unsigned char* mask, int n, unsigned short (*steps)[kMaxUnion], int* nsteps,
+                                           int lane) {
+  int cnt[2] = {0, 0};
+  for (int e0 = 0; e0 < n; e0 += 32) {
+    const int e = e0 + lane;
+    const unsigned m = e < n ? mask[e] : 0u;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const unsigned code = (who_attends(m) >> (2 * t)) & 3u;
+      const unsigned act = __ballot_sync(0xffffffffu, code != 0u);
+      if (code)
+        steps[t][cnt[t] + __popc(act & ((1u << lane) - 1u))] =
+            (unsigned short)(code | (((m >> (4 + 2 * t)) & 3u) << 2) | ((unsigned)e << 8));
+      cnt[t] += __popc(act);
+    }
+  }
+  if (lane == 0) { nsteps[0] = cnt[0]; nsteps[1] = cnt[1]; }
+}
+
 // Planner warp: draws work items from the queue (the first item of a CTA is its own index) and builds each
 // item's merged, interleaved key list one or more items ahead of the warps that consume it.  `SM` is the
-// kernel's shared-memory struct (info, ids, mask, tmp_ids, tmp_mask, list_full, list_empty).
-template <class SM>
+// kernel's shared-memory struct (info, ids, mask, steps, tmp_ids, tmp_mask, list_full, list_empty).
+//   kPlanUnion:  one list, the union of the local and the selected blocks
+//   kPlanSplit:  two lists per item, the selected blocks (info.branch 0), then the local ones (1)
+//   kPlanTagged: one list like kPlanUnion's whose masks tell the two kinds apart
+enum { kPlanUnion = 0, kPlanSplit = 1, kPlanTagged = 2 };
+template <int PLAN, class SM>
 __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t* __restrict__ block_idx,
                                              int* work_counter, int ipu, int total_items, int lane,
                                              volatile int* abort, int* status) {
-  for (int it = 0;; ++it) {
-    const int buf = it % kLists;
+  int lb = 0;  // list buffers handed out so far
+  bool ok = true;
+  auto acquire = [&]() {  // wait until list buffer lb % kLists is free
+    if (lane == 0) ok = mbar_wait(s32(&sm.list_empty[lb % kLists]), ((lb / kLists) & 1) ^ 1, abort, status);
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+  };
+  for (int it = 0; ok; ++it) {
     int item = 0;
     // the first item of a CTA is its own index; later ones come from the queue, which counts from 0
     if (lane == 0) item = it == 0 ? (int)blockIdx.x : atomicAdd(work_counter, 1) + (int)gridDim.x;
     item = __shfl_sync(0xffffffffu, item, 0);
-    bool ok = true;
-    if (lane == 0) ok = mbar_wait(s32(&sm.list_empty[buf]), ((it / kLists) & 1) ^ 1, abort, status);
-    ok = __shfl_sync(0xffffffffu, ok, 0);
+    acquire();
     if (!ok) break;
     if (item >= total_items) {
-      if (lane == 0) { sm.info[buf].n = -1; mbar_arrive(s32(&sm.list_full[buf])); }
+      if (lane == 0) { sm.info[lb % kLists].n = -1; mbar_arrive(s32(&sm.list_full[lb % kLists])); }
       break;
     }
     const int u = item / ipu;
@@ -543,62 +577,79 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
 #pragma unroll
     for (int h = 0; h < 4; ++h)
       jsel[h] = lane < g.topk ? __ldg(block_idx + ((long long)u * g.m + hb[h]) * g.topk + lane) : -1;
-    int n = 0;
+    for (int part = 0; part < (PLAN == kPlanSplit ? 2 : 1); ++part) {
+      if (part > 0) {
+        acquire();
+        if (!ok) break;
+      }
+      int n = 0;
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      if (!((valid >> h) & 1)) continue;
-      bool first = true;  // first half of its block: merge the block's list once, for all its halves
-      unsigned char bits = 0;
+      for (int h = 0; h < 4; ++h) {
+        if (!((valid >> h) & 1)) continue;
+        bool first = true;  // first half of its block: merge the block's list once, for all its halves
+        unsigned char bits = 0;
 #pragma unroll
-      for (int h2 = 0; h2 < 4; ++h2) {
-        if (((valid >> h2) & 1) && hb[h2] == hb[h]) {
-          if (h2 < h) first = false;
-          bits |= (unsigned char)(1 << h2);
+        for (int h2 = 0; h2 < 4; ++h2) {
+          if (((valid >> h2) & 1) && hb[h2] == hb[h]) {
+            if (h2 < h) first = false;
+            bits |= (unsigned char)(1 << h2);
+          }
+        }
+        if (!first) continue;
+        if (PLAN == kPlanTagged) {
+          n = merge_block(g, true, -1, hb[h], bits, sm.tmp_ids, sm.tmp_mask, n, lane, status);
+          n = merge_block(g, false, jsel[h], hb[h], (unsigned char)(bits << 4), sm.tmp_ids, sm.tmp_mask, n, lane, status);
+        } else {
+          n = merge_block(g, PLAN == kPlanUnion || part == 1, part == 1 ? -1 : jsel[h], hb[h], bits, sm.tmp_ids,
+                          sm.tmp_mask, n, lane, status);
         }
       }
-      if (first) n = merge_block(g, jsel[h], hb[h], bits, sm.tmp_ids, sm.tmp_mask, n, lane, status);
-    }
-    if (g.cpb == 1 && valid == 0xF) {
-      // Four different query blocks: which two share a 128-row tile is free.  Take the pairing whose tiles have
-      // the most entries in common (fewest products with a masked half); ties keep the first pairing.
-      int o01 = 0, o23 = 0, o02 = 0, o13 = 0, o03 = 0, o12 = 0;
-      for (int e0 = 0; e0 < n; e0 += 32) {
-        const unsigned mk = e0 + lane < n ? sm.tmp_mask[e0 + lane] : 0u;
-        o01 += __popc(__ballot_sync(0xffffffffu, (mk & 3u) == 3u));
-        o23 += __popc(__ballot_sync(0xffffffffu, (mk & 12u) == 12u));
-        o02 += __popc(__ballot_sync(0xffffffffu, (mk & 5u) == 5u));
-        o13 += __popc(__ballot_sync(0xffffffffu, (mk & 10u) == 10u));
-        o03 += __popc(__ballot_sync(0xffffffffu, (mk & 9u) == 9u));
-        o12 += __popc(__ballot_sync(0xffffffffu, (mk & 6u) == 6u));
-      }
-      const int s0 = o01 + o23, s1 = o02 + o13, s2 = o03 + o12;
-      const int pick = (s1 > s0 && s1 >= s2) ? 1 : (s2 > s0 && s2 > s1) ? 2 : 0;
-      if (pick != 0) {
-        // new half k is old half perm[k]: (0,2,1,3) pairs the blocks vertically, (0,3,1,2) diagonally
-        const int p1 = pick == 1 ? 2 : 3, p2 = 1, p3 = pick == 1 ? 3 : 2;
-        for (int e = lane; e < n; e += 32) {
-          const unsigned mk = sm.tmp_mask[e];
-          sm.tmp_mask[e] = (unsigned char)((mk & 1u) | (((mk >> p1) & 1u) << 1) | (((mk >> p2) & 1u) << 2) |
-                                           (((mk >> p3) & 1u) << 3));
+      if (g.cpb == 1 && valid == 0xF && part == 0) {
+        // Four different query blocks: which two share a 128-row tile is free.  Take the pairing whose tiles have
+        // the most entries in common (fewest products with a masked half); ties keep the first pairing.  (Split
+        // lists: the selected blocks decide; the local sets of neighbouring blocks overlap alike.)
+        int o01 = 0, o23 = 0, o02 = 0, o13 = 0, o03 = 0, o12 = 0;
+        for (int e0 = 0; e0 < n; e0 += 32) {
+          const unsigned mk = e0 + lane < n ? who_attends(sm.tmp_mask[e0 + lane]) : 0u;
+          o01 += __popc(__ballot_sync(0xffffffffu, (mk & 3u) == 3u));
+          o23 += __popc(__ballot_sync(0xffffffffu, (mk & 12u) == 12u));
+          o02 += __popc(__ballot_sync(0xffffffffu, (mk & 5u) == 5u));
+          o13 += __popc(__ballot_sync(0xffffffffu, (mk & 10u) == 10u));
+          o03 += __popc(__ballot_sync(0xffffffffu, (mk & 9u) == 9u));
+          o12 += __popc(__ballot_sync(0xffffffffu, (mk & 6u) == 6u));
         }
-        const int b1 = hb[p1], b2 = hb[p2], b3 = hb[p3], c1 = hc[p1], c2 = hc[p2], c3 = hc[p3];
-        hb[1] = b1; hb[2] = b2; hb[3] = b3;
-        hc[1] = c1; hc[2] = c2; hc[3] = c3;
-        __syncwarp();
+        const int s0 = o01 + o23, s1 = o02 + o13, s2 = o03 + o12;
+        const int pick = (s1 > s0 && s1 >= s2) ? 1 : (s2 > s0 && s2 > s1) ? 2 : 0;
+        if (pick != 0) {
+          // new half k is old half perm[k]: (0,2,1,3) pairs the blocks vertically, (0,3,1,2) diagonally
+          const int p1 = pick == 1 ? 2 : 3, p2 = 1, p3 = pick == 1 ? 3 : 2;
+          for (int e = lane; e < n; e += 32) {
+            const unsigned mk = sm.tmp_mask[e];
+            sm.tmp_mask[e] = (unsigned char)((mk & 0x11u) | (((mk >> p1) & 0x11u) << 1) | (((mk >> p2) & 0x11u) << 2) |
+                                             (((mk >> p3) & 0x11u) << 3));
+          }
+          const int b1 = hb[p1], b2 = hb[p2], b3 = hb[p3], c1 = hc[p1], c2 = hc[p2], c3 = hc[p3];
+          hb[1] = b1; hb[2] = b2; hb[3] = b3;
+          hc[1] = c1; hc[2] = c2; hc[3] = c3;
+          __syncwarp();
+        }
       }
-    }
-    interleave_tiles(sm.tmp_ids, sm.tmp_mask, n, sm.ids[buf], sm.mask[buf], lane);
-    if (lane == 0) {
-      ItemInfo& inf = sm.info[buf];
-      inf.n = n; inf.unit = u; inf.hvalid = valid; inf.more = 0;
+      const int buf = lb % kLists;
+      interleave_tiles(sm.tmp_ids, sm.tmp_mask, n, sm.ids[buf], sm.mask[buf], lane);
+      tile_steps(sm.mask[buf], n, sm.steps[buf], sm.info[buf].nsteps, lane);
+      if (lane == 0) {
+        ItemInfo& inf = sm.info[buf];
+        inf.n = n; inf.unit = u; inf.hvalid = valid; inf.more = 0; inf.branch = part;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) { inf.hb[h] = hb[h]; inf.hc[h] = hc[h]; }
-    }
-    __syncwarp();
+        for (int h = 0; h < 4; ++h) { inf.hb[h] = hb[h]; inf.hc[h] = hc[h]; }
+      }
+      __syncwarp();
+      ++lb;
 #ifdef MOSAIC_TEST_WITHHOLD_FIRST_LIST  // test build only: the CTA's first list is never published, so every consumer's wait runs out
-    if (it == 0) continue;
+      if (lb == 1) continue;
 #endif
-    if (lane == 0) mbar_arrive(s32(&sm.list_full[buf]));
+      if (lane == 0) mbar_arrive(s32(&sm.list_full[buf]));
+    }
   }
 }
 
@@ -617,8 +668,8 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 // again encodes nothing.
 // [units, nlat, nlon, d] bf16 view, box = one 64-token chunk {d, bw, 64/bw, 1}, 128-byte swizzle.
 bool make_map(CUtensorMap* map, const void* base, const Geo& g, int units);
-// [U, nlat, nlon] fp32 view (one value per token), box = the 64 tokens of one chunk {bw, 64/bw, 1}, no swizzle.
-bool make_map_rows(CUtensorMap* map, const void* base, const Geo& g);
+// [units, nlat, nlon] fp32 view (one value per token), box = the 64 tokens of one chunk {bw, 64/bw, 1}, no swizzle.
+bool make_map_rows(CUtensorMap* map, const void* base, const Geo& g, int units);
 // Current device, its SM count (cached), and the opt-in to `smem` bytes of dynamic shared memory for `func`
 // (set once per device; `done` is the caller's per-kernel bit set of devices already configured).
 int launch_setup(const void* func, size_t smem, unsigned long long* done, int* sms);

@@ -90,7 +90,7 @@ std::atomic<int> g_sms[kMaxDevices];
 }  // namespace
 
 bool make_map(CUtensorMap* map, const void* base, const Geo& g, int units) { return cached_map(map, base, g, 0, units); }
-bool make_map_rows(CUtensorMap* map, const void* base, const Geo& g) { return cached_map(map, base, g, 1, g.U); }
+bool make_map_rows(CUtensorMap* map, const void* base, const Geo& g, int units) { return cached_map(map, base, g, 1, units); }
 
 int launch_setup(const void* func, size_t smem, unsigned long long* done, int* sms) {
   int dev = 0;
