@@ -322,77 +322,85 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == kWMma0) {
-    // ------------------------------------------------------------- issuer of S^T = K Q^T and dP^T = V dO^T (one thread)
-    // The buffers may be overwritten once the row threads hold the previous pair in registers, so this thread runs
-    // one pair ahead of their arithmetic.
-    if (lane == 0) {
-      constexpr uint32_t idesc1 = make_idesc(false, 64u, F16), idesc2 = make_idesc(false, 128u, F16);
-      const uint64_t kdesc = smem_desc(s32(sm.k)), vdesc = smem_desc(s32(sm.v));
-      long long pr = 0;
-      int items = 0;
-      bool ok = true, fresh = true;
-      for (int lb = 0; ok; ++lb) {
-        const int buf = lb % kLists;
-        ok = mbar_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
+    // ------------------------------------------------------------- issuer of S^T = K Q^T and dP^T = V dO^T
+    // The buffers may be overwritten once the row threads hold the previous pair in registers, so this warp runs
+    // one pair ahead of their arithmetic.  (The whole warp walks the loop, one elected lane issues: operands that are the
+    // same for the warp stay in uniform registers.)
+    constexpr uint32_t idesc1 = make_idesc(false, 64u, F16), idesc2 = make_idesc(false, 128u, F16);
+    const uint64_t kdesc = smem_desc(s32(sm.k)), vdesc = smem_desc(s32(sm.v));
+    uint32_t pr = 0, items = 0;
+    bool ok = true, fresh = true;
+    for (int lb = 0; ok; ++lb) {
+      const int buf = lb % kLists;
+      ok = warp_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
+      if (!ok) break;
+      const int n = sm.info[buf].n;
+      if (n < 0) break;
+      const bool more = sm.info[buf].more != 0;
+      if (fresh) {
+        ok = warp_wait(s32(&sm.kv_full), items & 1, abort, status);
         if (!ok) break;
-        const int n = sm.info[buf].n;
-        if (n < 0) break;
-        const bool more = sm.info[buf].more != 0;
-        if (fresh) {
-          ok = mbar_wait(s32(&sm.kv_full), items & 1, abort, status);
-          if (!ok) break;
-          ++items;
-        }
-        fresh = !more;
-        const int chunks = n * g.cpb;
-        for (int p0 = 0; p0 < chunks && ok; p0 += 2, ++pr) {
-          const int slot = (int)(pr % kSlots);
-          ok = mbar_wait(s32(&sm.ring_full[slot]), (uint32_t)((pr / kSlots) & 1), abort, status);
-          if (ok && pr > 0) ok = mbar_wait(s32(&sm.sdp_free), (uint32_t)((pr - 1) & 1), abort, status);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t idesc = chunks - p0 >= 2 ? idesc2 : idesc1;
-          const uint64_t qdesc = smem_desc(s32(sm.ring[slot].q[0])), dodesc = smem_desc(s32(sm.ring[slot].d_o[0]));
+        ++items;
+      }
+      fresh = !more;
+      const int chunks = n * g.cpb;
+      for (int p0 = 0; p0 < chunks; p0 += 2, ++pr) {
+        const uint32_t slot = pr % kSlots;
+        ok = warp_wait(s32(&sm.ring_full[slot]), (pr / kSlots) & 1u, abort, status);
+        if (ok) ok = warp_wait(s32(&sm.sdp_free), (pr & 1u) ^ 1u, abort, status);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t idesc = chunks - p0 >= 2 ? idesc2 : idesc1;
+        const uint64_t qdesc = smem_desc(s32(sm.ring[slot].q[0])), dodesc = smem_desc(s32(sm.ring[slot].d_o[0]));
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) umma_ss(tmem + kColS, kdesc + 2 * kk, qdesc + 2 * kk, idesc, kk > 0);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) umma_ss(tmem + kColDP, vdesc + 2 * kk, dodesc + 2 * kk, idesc, kk > 0);
           tc_commit(s32(&sm.s_full));
         }
-        // the K and V tiles are read by this thread's products only: all of the item's are behind this commit
-        if (ok && !more) tc_commit(s32(&sm.kv_empty));
-        if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
+        __syncwarp();
       }
-      if (*abort) mma_drain(s32(&sm.mma_drain_bar[0]));  // products already issued must finish before the release
+      if (ok && elect_one()) {
+        // the K and V tiles are read by this warp's products only: all of the item's are behind this commit
+        if (!more) tc_commit(s32(&sm.kv_empty));
+        mbar_arrive(s32(&sm.list_empty[buf]));
+      }
+      __syncwarp();
     }
+    if (*abort && elect_one()) mma_drain(s32(&sm.mma_drain_bar[0]));  // products already issued must finish before the release
+    __syncwarp();
   } else if (warp == kWMma1) {
-    // ------------------------------------------------------------- issuer of dV += P^T dO and dK += dS^T Q (one thread)
-    if (lane == 0) {
-      constexpr uint32_t idesc_nn = make_idesc(true, 64u, F16);
-      long long pr = 0;
-      uint32_t jg[2] = {0u, 0u};  // products each group of row threads has handed over (phase of p_full)
-      uint32_t items = 0;         // items whose accumulators have been handed to the row threads
-      bool ok = true, first = true;
-      for (int lb = 0; ok; ++lb) {
-        const int buf = lb % kLists;
-        ok = mbar_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
-        if (!ok) break;
-        const int n = sm.info[buf].n;
-        if (n < 0) break;
-        const bool more = sm.info[buf].more != 0;
-        const int chunks = n * g.cpb;
-        for (int p0 = 0; p0 < chunks && ok; p0 += 2, ++pr) {
-          const int slot = (int)(pr % kSlots), np = min(2, chunks - p0);
-          // the slot landed before S^T could be produced; this wait makes the copied Q and dO visible here too
-          ok = mbar_wait(s32(&sm.ring_full[slot]), (uint32_t)((pr / kSlots) & 1), abort, status);
-          for (int h = 0; h < np && ok; ++h) {
-            ok = mbar_wait(s32(&sm.p_full[h]), jg[h] & 1, abort, status);
-            // a new accumulation overwrites dK and dV: every row thread must have read the previous item's
-            if (ok && first && items > 0) ok = mbar_wait(s32(&sm.acc_free), (items - 1) & 1, abort, status);
-            if (!ok) break;
-            ++jg[h];
-            tc_fence_after();
-            const uint64_t qmn = smem_desc(s32(sm.ring[slot].q[h])), domn = smem_desc(s32(sm.ring[slot].d_o[h]));
+    // ------------------------------------------------------------- issuer of dV += P^T dO and dK += dS^T Q
+    constexpr uint32_t idesc_nn = make_idesc(true, 64u, F16);
+    uint32_t pr = 0;
+    uint32_t jg[2] = {0u, 0u};  // products each group of row threads has handed over (phase of p_full)
+    uint32_t items = 0;         // items whose accumulators have been handed to the row threads
+    bool ok = true, first = true;
+    for (int lb = 0; ok; ++lb) {
+      const int buf = lb % kLists;
+      ok = warp_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
+      if (!ok) break;
+      const int n = sm.info[buf].n;
+      if (n < 0) break;
+      const bool more = sm.info[buf].more != 0;
+      const int chunks = n * g.cpb;
+      for (int p0 = 0; p0 < chunks && ok; p0 += 2, ++pr) {
+        const uint32_t slot = pr % kSlots;
+        const bool two = chunks - p0 >= 2;
+        // the slot landed before S^T could be produced; this wait makes the copied Q and dO visible here too
+        ok = warp_wait(s32(&sm.ring_full[slot]), (pr / kSlots) & 1u, abort, status);
+        // a new accumulation overwrites dK and dV: every row thread must have read the previous item's
+        if (ok && first && items > 0) ok = warp_wait(s32(&sm.acc_free), (items - 1) & 1, abort, status);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (h == 1 && !two) break;
+          if (ok) ok = warp_wait(s32(&sm.p_full[h]), jg[h] & 1, abort, status);
+          if (!ok) break;
+          ++jg[h];
+          tc_fence_after();
+          const uint64_t qmn = smem_desc(s32(sm.ring[slot].q[h])), domn = smem_desc(s32(sm.ring[slot].d_o[h]));
+          if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
               umma_ts(tmem + kColDV, tmem + kColP + 32 * h + 8 * kk, domn + (uint64_t)((2048 * kk) >> 4), idesc_nn,
@@ -401,22 +409,30 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int kk = 0; kk < 4; ++kk)
               umma_ts(tmem + kColDK, tmem + kColDS + 32 * h + 8 * kk, qmn + (uint64_t)((2048 * kk) >> 4), idesc_nn,
                       (!first || kk > 0));
-            first = false;
+            if (h == 1 || !two) {
+              // the pair's S^T and dP^T completed before P^T could be formed, so this warp's completion frees the slot
+              tc_commit(s32(&sm.pv_done));
+              tc_commit(s32(&sm.ring_empty[slot]));
+            }
           }
-          if (!ok) break;
-          // the pair's S^T and dP^T completed before P^T could be formed, so this thread's completion frees the slot
-          tc_commit(s32(&sm.ring_empty[slot]));
-          tc_commit(s32(&sm.pv_done));
+          __syncwarp();
+          first = false;
         }
-        if (ok && !more && !first) {  // the item's accumulators are complete behind this commit
-          tc_commit(s32(&sm.acc_done));
-          ++items;
-          first = true;
-        }
-        if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
       }
-      if (*abort) mma_drain(s32(&sm.mma_drain_bar[1]));
+      if (!ok) break;
+      const bool complete = !more && !first;
+      if (elect_one()) {
+        if (complete) tc_commit(s32(&sm.acc_done));  // the item's accumulators are complete behind this commit
+        mbar_arrive(s32(&sm.list_empty[buf]));
+      }
+      __syncwarp();
+      if (complete) {
+        ++items;
+        first = true;
+      }
     }
+    if (*abort && elect_one()) mma_drain(s32(&sm.mma_drain_bar[1]));
+    __syncwarp();
   } else if (warp < kRowWarps) {
     // ------------------------------------------------------------- row threads (TMEM lane = key row)
     // Group 0 takes the first chunk of every pair, group 1 the second, so the two work side by side.  Inside a
@@ -432,39 +448,40 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
     const uint32_t col_s = kColS + 64 * grp + 32 * ch, col_dp = kColDP + 64 * grp + 32 * ch;
     const uint32_t col_p = kColP + 32 * grp + 16 * ch, col_ds = kColDS + 32 * grp + 16 * ch;
-    long long pr = 0;    // pairs seen so far
+    uint32_t pr = 0;     // pairs seen so far
     uint32_t item_chunks = 0, items = 0;
+    const bool cpb1 = g.cpb == 1;  // (larger blocks have an even number of chunks)
     bool ok = true;
     for (int lb = 0; ok; ++lb) {
       const int buf = lb % kLists;
-      ok = mbar_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = warp_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
       const bool more = sm.info[buf].more != 0;
       const int chunks = n * g.cpb;
       item_chunks += (uint32_t)chunks;
+      int e = cpb1 ? grp : 0, ec = cpb1 ? 0 : grp;  // list entry of this group's chunk, and its chunk of that entry
       for (int p0 = 0; p0 < chunks; p0 += 2, ++pr) {
-        ok = mbar_wait(s32(&sm.s_full), (uint32_t)(pr & 1), abort, status);
-        ok = __all_sync(0xffffffffu, ok);
+        const int ecur = e;
+        if (cpb1) e += 2;
+        else if ((ec += 2) >= g.cpb) { ec -= g.cpb; ++e; }
+        ok = warp_wait(s32(&sm.s_full), pr & 1u, abort, status);
         if (!ok) break;
         tc_fence_after();
-        const int p = p0 + grp;
-        if (p >= chunks) {  // a pair of one: nothing for group 1, the buffers go back at once
+        if (p0 + grp >= chunks) {  // a pair of one: nothing for group 1, the buffers go back at once
           tc_fence_before();
           mbar_arrive(s32(&sm.sdp_free));
           continue;
         }
-        const uint32_t mk = sm.mask[buf][p / g.cpb];
+        const uint32_t mk = sm.mask[buf][ecur];
         const bool connected = ((BR ? mk | (mk >> 4) : mk) & hbit) != 0;
         uint32_t pp[16], ds[16];
         if (connected) {
-          const int slot = (int)(pr % kSlots);
+          const uint32_t slot = pr % kSlots;
           // the slot landed before the MMA warp could produce this S^T; waiting on its barrier here as well
           // makes the copied -LSE and -D visible to this thread
-          ok = mbar_wait(s32(&sm.ring_full[slot]), (uint32_t)((pr / kSlots) & 1), abort, status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = warp_wait(s32(&sm.ring_full[slot]), (pr / kSlots) & 1u, abort, status);
           if (!ok) break;
           // statistics of the chunk's query columns for this half's kind of connection
           const float(*stat)[2][64] = &sm.ring[slot].stat[BR && ((mk >> 4) & hbit) ? 3 : 0];
@@ -508,12 +525,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 16; ++i) { pp[i] = 0u; ds[i] = 0u; }
         }
         // P^T and dS^T have one buffer per group: the previous pair's dV / dK updates must have consumed them
-        if (pr > 0) {
-          ok = mbar_wait(s32(&sm.pv_done), (uint32_t)((pr - 1) & 1), abort, status);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          tc_fence_after();
-        }
+        ok = warp_wait(s32(&sm.pv_done), (pr & 1u) ^ 1u, abort, status);
+        if (!ok) break;
+        tc_fence_after();
         tmem_st16(tb + col_p, pp);
         tmem_st16(tb + col_ds, ds);
         tmem_wait_st();
@@ -523,8 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       if (!more) {
         if (item_chunks > 0) {
-          ok = mbar_wait(s32(&sm.acc_done), items & 1, abort, status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = warp_wait(s32(&sm.acc_done), items & 1, abort, status);
           if (!ok) break;
           tc_fence_after();
           if ((sm.info[buf].hvalid >> hh) & 1) {

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     // dQ += dS K of the product whose K chunk sits in ring stage `pst` (the previous product of this tile)
     auto issue_dq = [&](int pst, bool pfirst) {
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.p_full[t]), (nt - 1) & 1, abort, status));
+      ok = warp_wait(s32(&sm.p_full[t]), (nt - 1) & 1, abort, status);
       if (!ok) return;
       tc_fence_after();
       const uint64_t kmn = smem_desc(s32(sm.kv[pst][0]));
@@ -167,13 +167,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     for (int it = 0; ok; ++it) {
       const int buf = it % kLists;
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status));
+      ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
       const int cnt = sm.info[buf].nsteps[t];
       // the tiles are loaded for every item; they must have landed before their buffers are handed back
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.q_full[t]), it & 1, abort, status));
+      ok = warp_wait(s32(&sm.q_full[t]), it & 1, abort, status);
       if (!ok) break;
       if (cnt == 0 && elect_one()) mbar_arrive(s32(&sm.q_empty[t]));
       bool first = true, pend = false, pend_first = false;
@@ -189,11 +189,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             pend = false;
             if (!ok) break;
           }
-          ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status));
+          ok = warp_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status);
           if (!ok) break;
           // S and dP may be overwritten once the row threads hold the previous product's values in registers
           if (nt > 0) {
-            ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.sdp_free[t]), (nt - 1) & 1, abort, status));
+            ok = warp_wait(s32(&sm.sdp_free[t]), (nt - 1) & 1, abort, status);
             if (!ok) break;
           }
           tc_fence_after();
@@ -236,8 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (int it = 0; ok; ++it) {
       const int buf = it % kLists;
-      ok = mbar_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
@@ -267,8 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           gate2 = pack2(c, c);
         }
         for (int c = 0; c < g.cpb; ++c) {
-          ok = mbar_wait(s32(&sm.s_full[t]), nt & 1, abort, status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = warp_wait(s32(&sm.s_full[t]), nt & 1, abort, status);
           if (!ok) break;
           tc_fence_after();
           uint32_t pk[32];
@@ -299,8 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           // dS has one buffer: the previous product's dQ += dS K must have consumed it
           if (i0 + c > 0) {
-            ok = mbar_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
-            ok = __all_sync(0xffffffffu, ok);
+            ok = warp_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
             if (!ok) break;
             tc_fence_after();
           }
@@ -313,8 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       if (cnt > 0) {
-        ok = mbar_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
-        ok = __all_sync(0xffffffffu, ok);
+        ok = warp_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
         if (!ok) break;
         tc_fence_after();
         if (valid) {

@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // P V of product `pn` (its V chunk sits in ring stage `pst`); `pfirst` starts a new accumulation
     auto issue_pv = [&](uint32_t pn, int pst, bool pfirst) {
       const uint32_t b = pn & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.p_full[t][b]), (pn >> 1) & 1, abort, status));
+      ok = warp_wait(s32(&sm.p_full[t][b]), (pn >> 1) & 1, abort, status);
       if (!ok) return;
       tc_fence_after();
       const uint64_t vdesc = smem_desc(s32(sm.kv[pst][1]));
@@ -240,12 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     for (int it = 0; ok; ++it) {
       const int buf = it % kLists;
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status));
+      ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
       // the item's query rows are in TMEM (copied there by the softmax threads)
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.q_ready[t]), it & 1, abort, status));
+      ok = warp_wait(s32(&sm.q_ready[t]), it & 1, abort, status);
       if (!ok) break;
       bool first = true, pend = false, pend_first = false;
       uint32_t pend_n = 0, pend_step = 0;
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             pend = false;
             if (!ok) break;
           }
-          ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status));
+          ok = warp_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status);
           if (!ok) break;
           // S buffer nt & 1 (aliased by P) was last read by P V of product nt - 2, which this warp issued
           // earlier: tensor-core operations of one thread execute in issue order, so this QK^T cannot
@@ -306,11 +306,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Returns the item's list length (-1: no more work).
     auto stage_q = [&](int it2) -> int {
       const int buf2 = it2 % kLists, qb2 = it2 & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.list_full[buf2]), (it2 / kLists) & 1, abort, status));
+      ok = warp_wait(s32(&sm.list_full[buf2]), (it2 / kLists) & 1, abort, status);
       if (!ok) return -1;
       const int n2 = sm.info[buf2].n;
       if (n2 < 0) return -1;
-      ok = __all_sync(0xffffffffu, mbar_wait(s32(&sm.q_full[qb2][t]), (it2 >> 1) & 1, abort, status));
+      ok = warp_wait(s32(&sm.q_full[qb2][t]), (it2 >> 1) & 1, abort, status);
       if (!ok) return -1;
       const int r = tid & 127;  // row of the tile; rows 0-63 and 64-127 are two 8 KB chunks
       const unsigned char* rowp = sm.q[qb2][t] + (r >> 6) * kTile + (r & 63) * 128;
@@ -337,8 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool attends = (steps[i0] >> hh) & 1u;
         for (int c = 0; c < g.cpb; ++c) {
           const uint32_t b = nt & 1, tsb = ts + 64 * b;
-          ok = mbar_wait(s32(&sm.s_full[t][b]), (nt >> 1) & 1, abort, status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = warp_wait(s32(&sm.s_full[t][b]), (nt >> 1) & 1, abort, status);
           if (!ok) break;
           tc_fence_after();
           if (attends) {
@@ -407,8 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (__any_sync(0xffffffffu, need)) {
               // the accumulator may only be touched between P V products: wait for the previous one
               if (i0 + c > 0) {
-                ok = mbar_wait(s32(&sm.pv_done[t][b ^ 1]), ((nt - 1) >> 1) & 1, abort, status);
-                ok = __all_sync(0xffffffffu, ok);
+                ok = warp_wait(s32(&sm.pv_done[t][b ^ 1]), ((nt - 1) >> 1) & 1, abort, status);
                 if (!ok) break;
                 tc_fence_after();
               }
@@ -446,8 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int n_next = stage_q(it + 1);
       if (!ok) break;
       if (cnt > 0) {
-        ok = mbar_wait(s32(&sm.pv_done[t][(nt - 1) & 1]), ((nt - 1) >> 1) & 1, abort, status);
-        ok = __all_sync(0xffffffffu, ok);
+        ok = warp_wait(s32(&sm.pv_done[t][(nt - 1) & 1]), ((nt - 1) >> 1) & 1, abort, status);
         if (!ok) break;
         tc_fence_after();
       }

@@ -98,21 +98,14 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
     if (clock64() - t0 > kDrainCycles) return false;
   return true;
 }
-// Warp-wide wait: lane 0 polls, the warp learns the outcome and synchronises (polls by all 32 lanes serialise on the
-// barrier word and cost several times as much).  What lane 0 acquired is visible to the warp after the barrier.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, int* status, int lane) {
-  bool ok = true;
-  if (lane == 0) ok = mbar_wait(bar, parity, abort, status);
-  ok = __all_sync(0xffffffffu, ok);
-  __syncwarp();
-  return ok;
+// The same for a converged warp whose lanes all wait for the same phase: the outcome is the same in every lane, and the
+// usual case is one poll and one vote.
+__device__ __noinline__ bool warp_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort, status));
 }
-__device__ __forceinline__ bool warp_test(uint32_t bar, uint32_t parity, int lane) {
-  bool ok = true;
-  if (lane == 0) ok = mbar_test(bar, parity);
-  ok = __all_sync(0xffffffffu, ok);
-  __syncwarp();
-  return ok;
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return warp_wait_slow(bar, parity, abort, status);
 }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
