@@ -60,12 +60,11 @@ SelectWs select_layout(const Geo& g) {
 
 BranchWs branch_layout(const Geo& g) {
   BranchWs w;
-  const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD), norms = align256(sizeof(float) * (size_t)g.U * g.m);
+  const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD);
   w.pq = kStatusBytes;
   w.pk = w.pq + pooled;
   w.pv = w.pk + pooled;
-  w.nrm = w.pv + pooled;
-  w.ocg = w.nrm + 2 * norms;
+  w.ocg = w.pv + pooled;
   w.total = w.ocg + pooled;
   return w;
 }
@@ -91,7 +90,7 @@ BwdWs bwd_layout(const Geo& g, int planes, size_t at) {
 // attention backward's own scratch.
 struct BwdBranchWs {
   BranchWs f;
-  size_t lse_cg, delta, dob, dqm, dkm, dvm;
+  size_t lse_cg, dob, dqm, dkm, dvm;
   BwdWs b;
 };
 BwdBranchWs bwd_branch_layout(const Geo& g) {
@@ -100,13 +99,20 @@ BwdBranchWs bwd_branch_layout(const Geo& g) {
   const size_t pooled = align256(sizeof(float) * (size_t)g.U * g.m * kD), blocks = align256(sizeof(float) * (size_t)g.U * g.m);
   size_t at = w.f.total;
   w.lse_cg = at; at += blocks;
-  w.delta = at; at += blocks;
   w.dob = at; at += pooled;
   w.dqm = at; at += pooled;
   w.dkm = at; at += pooled;
   w.dvm = at; at += pooled;
   w.b = bwd_layout(g, 2, at);
   return w;
+}
+PoolArgs branch_pool(const Geo& g, const void* q, const void* k, const void* v, float* pq, float* pk, float* pv) {
+  PoolArgs a = {};
+  a.n = 3;
+  a.job[0] = {q, pq, nullptr, nullptr, g.U};
+  a.job[1] = {k, pk, nullptr, nullptr, g.Ukv};
+  a.job[2] = {v, pv, nullptr, nullptr, g.Ukv};
+  return a;
 }
 size_t select_total(const Geo& g) { return select_layout(g).total; }
 
@@ -123,7 +129,8 @@ int device_ok() {
   return major == 10 ? MOSAIC_OK : MOSAIC_E_UNSUPPORTED;
 }
 
-int begin(const mosaic_bsa_params* p, void* ws, size_t ws_bytes, size_t need, void* stream, HostCtx* c) {
+// `reset`: the status block is cleared here (otherwise the op's first kernel does it)
+int begin(const mosaic_bsa_params* p, void* ws, size_t ws_bytes, size_t need, void* stream, HostCtx* c, bool reset) {
   int rc = validate(p, &c->g);
   if (rc) return rc;
   if (!ws) return MOSAIC_E_INVALID_ARG;
@@ -132,7 +139,7 @@ int begin(const mosaic_bsa_params* p, void* ws, size_t ws_bytes, size_t need, vo
   if ((rc = device_ok())) return rc;
   c->stream = (cudaStream_t)stream;
   c->status = (int*)ws;
-  if (cudaMemsetAsync(ws, 0, kStatusBytes, c->stream) != cudaSuccess) return MOSAIC_E_CUDA;
+  if (reset && cudaMemsetAsync(ws, 0, kStatusBytes, c->stream) != cudaSuccess) return MOSAIC_E_CUDA;
   return MOSAIC_OK;
 }
 
@@ -164,7 +171,7 @@ int mosaic_bsa_select(const mosaic_bsa_params* p, const void* q, const void* k, 
   if (rc) return rc;
   if (!q || !k || (!block_idx && g.topk > 0)) return MOSAIC_E_INVALID_ARG;
   if (!aligned(q, 16) || !aligned(k, 16) || !aligned(block_idx, 4)) return MOSAIC_E_MISALIGNED;
-  if ((rc = begin(p, ws, ws_bytes, select_total(g), cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, select_total(g), cuda_stream, &c, false))) return rc;
   const SelectWs w = select_layout(g);
   char* base = (char*)ws;
   return launch_select(c, q, k, block_idx, (float*)(base + w.pq), (float*)(base + w.pk), (float*)(base + w.nq),
@@ -181,7 +188,7 @@ int mosaic_bsa_fwd(const mosaic_bsa_params* p, const void* q, const void* k, con
   if (!aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(o, 16) || !aligned(lse, 4) ||
       !aligned(block_idx, 4))
     return MOSAIC_E_MISALIGNED;
-  if ((rc = begin(p, ws, ws_bytes, kStatusBytes, cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, kStatusBytes, cuda_stream, &c, true))) return rc;
   FwdOut out = {};
   out.o = (__nv_bfloat16*)o;
   out.lse = lse;
@@ -200,15 +207,12 @@ int mosaic_bsa_fwd_branches(const mosaic_bsa_params* p, const void* q, const voi
       !aligned(lse_fg, 4) || !aligned(lse_l, 4) || !aligned(block_idx, 4))
     return MOSAIC_E_MISALIGNED;
   const BranchWs w = branch_layout(g);
-  if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c, false))) return rc;
   char* base = (char*)ws;
   float *pq = (float*)(base + w.pq), *pk = (float*)(base + w.pk), *pv = (float*)(base + w.pv);
-  float *nrm = (float*)(base + w.nrm), *ocg = (float*)(base + w.ocg);
-  // compression branch: pooled sums of Q, K (with their norms, unused here) and V, then block-level attention
-  HostCtx cp = c;
-  cp.g.topk = 0;  // pooling only
-  if ((rc = launch_select(cp, q, k, nullptr, pq, pk, nrm, nrm + (size_t)g.U * g.m))) return rc;
-  if ((rc = launch_pool_one(c, v, pv, nrm, g.Ukv))) return rc;
+  float* ocg = (float*)(base + w.ocg);
+  // compression branch: pooled sums of Q, K and V, then block-level attention
+  if ((rc = launch_pool(c, branch_pool(g, q, k, v, pq, pk, pv)))) return rc;
   if ((rc = launch_compress(c, pq, pk, pv, ocg, nullptr))) return rc;
   // selection and local branch, each with its own softmax, and the gated sum
   FwdOut out = {};
@@ -235,7 +239,7 @@ int mosaic_bsa_bwd(const mosaic_bsa_params* p, const void* q, const void* k, con
   if (!aligned(lse, 4) || !aligned(block_idx, 4)) return MOSAIC_E_MISALIGNED;
   if (2 * (size_t)g.m * sizeof(int) + (size_t)g.m * g.topk / 8 + 8 > 200 * 1024) return MOSAIC_E_UNSUPPORTED;  // transposed-pattern kernel
   const BwdWs w = bwd_layout(g, 1, kStatusBytes);
-  if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, w.total, cuda_stream, &c, false))) return rc;
   char* base = (char*)ws;
   float *neg_d = (float*)(base + w.neg_d), *neg_lse2 = (float*)(base + w.neg_lse2);
   if ((rc = launch_rowdot(c, o, d_o, lse, neg_d, neg_lse2))) return rc;
@@ -261,16 +265,15 @@ int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   if (!aligned(gates, 4) || !aligned(dgates, 4) || !aligned(block_idx, 4)) return MOSAIC_E_MISALIGNED;
   if (2 * (size_t)g.m * sizeof(int) + (size_t)g.m * g.topk / 8 + 8 > 200 * 1024) return MOSAIC_E_UNSUPPORTED;  // transposed-pattern kernel
   const BwdBranchWs w = bwd_branch_layout(g);
-  if ((rc = begin(p, ws, ws_bytes, w.b.total, cuda_stream, &c))) return rc;
+  if ((rc = begin(p, ws, ws_bytes, w.b.total, cuda_stream, &c, false))) return rc;
   char* base = (char*)ws;
   auto F = [&](size_t off) { return (float*)(base + off); };
-  float *pq = F(w.f.pq), *pk = F(w.f.pk), *pv = F(w.f.pv), *nrm = F(w.f.nrm), *ocg = F(w.f.ocg);
-  // the forward again: pooled sums, block-level attention (with its log-sum-exp), and of the attention branches the gate
-  // gradients and row statistics
-  HostCtx cp = c;
-  cp.g.topk = 0;  // pooling only
-  if ((rc = launch_select(cp, q, k, nullptr, pq, pk, nrm, nrm + (size_t)g.U * g.m))) return rc;
-  if ((rc = launch_pool_one(c, v, pv, nrm, g.Ukv))) return rc;
+  float *pq = F(w.f.pq), *pk = F(w.f.pk), *pv = F(w.f.pv), *ocg = F(w.f.ocg);
+  // the forward again: pooled sums (and the gated block sums of dO), block-level attention with its log-sum-exp, and of the
+  // attention branches the gate gradients and row statistics
+  PoolArgs pool = branch_pool(g, q, k, v, pq, pk, pv);
+  pool.job[pool.n++] = {d_o, F(w.dob), nullptr, gates, g.U};
+  if ((rc = launch_pool(c, pool))) return rc;
   if ((rc = launch_compress(c, pq, pk, pv, ocg, F(w.lse_cg)))) return rc;
   FwdOut out = {};
   out.gates = gates;
@@ -282,9 +285,8 @@ int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   out.gate = F(w.b.gate);
   if ((rc = launch_fwd_tc(c, kFwdStats, q, k, v, block_idx, out, c.status + 1))) return rc;
   // compression branch on the block level
-  if ((rc = launch_gated_pool(c, d_o, gates, F(w.dob)))) return rc;
-  if ((rc = launch_compress_bwd(c, pq, pk, pv, F(w.dob), ocg, F(w.lse_cg), F(w.delta), F(w.dqm), F(w.dkm), F(w.dvm))))
-    return rc;
+  const CompressBwd cb = {pq, pk, pv, F(w.dob), ocg, F(w.lse_cg), F(w.dqm), F(w.dkm), F(w.dvm)};
+  if ((rc = launch_compress_bwd(c, cb))) return rc;
   // both attention branches in one pass, with the block level's share added in the epilogues
   RowStats st = {};
   st.neg_lse2 = out.neg_lse2;

@@ -24,7 +24,9 @@ constexpr float kLog2e = 1.4426950408889634f;
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uint4* __restrict__ o,
                                                      const uint4* __restrict__ d_o, const float* __restrict__ lse,
-                                                     float* __restrict__ neg_d, float* __restrict__ neg_lse2, bool f16) {
+                                                     float* __restrict__ neg_d, float* __restrict__ neg_lse2, bool f16,
+                                                     int* status) {
+  if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0;  // the op's first kernel
   long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   int part = threadIdx.x & 7;
   float acc = 0.f;
@@ -52,16 +54,18 @@ __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uin
 // ------------------------------------------------------------------------------------------
 // Transposed pattern: for every key block j the ascending list of query blocks that selected it.
 // One CTA per unit.  The query blocks are cut into `nseg` contiguous segments:
-//   1. one thread per query block validates its row of block_idx (ids outside [0, m), ids of the row's own
+//   1. a warp validates up to 32 / topk rows of block_idx at a time (ids outside [0, m), ids of the row's own
 //      neighbourhood and repeats are dropped, exactly as the forward drops them), marks the valid entries in a
 //      bit array and counts them per (segment, key block);
-//   2. per key block, a running sum over the segments and an exclusive scan over the key blocks turn the counts
+//   2. per key block, a running sum over the segments and an exclusive scan of the CTA over the key blocks turn the counts
 //      into the position where each segment's part of each list starts;
 //   3. every warp fills its segments in entry order, so each list comes out sorted by query block id (this
 //      fixes the dK/dV summation order).
 // Shared memory: (nseg + 1) * m counters + m * topk bits.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) csr_kernel(Geo g, const int32_t* __restrict__ block_idx,
+// Latency-bound (one CTA per unit): with a thread per row and eight segments 9216 entries took 66 us.
+constexpr int kCsrThreads = 512;
+__global__ void __launch_bounds__(kCsrThreads) csr_kernel(Geo g, const int32_t* __restrict__ block_idx,
                                                   int32_t* __restrict__ csr_off, int32_t* __restrict__ csr_q, int nseg) {
   extern __shared__ int csr_sm[];
   int* tot = csr_sm;                        // [m] list lengths, then list starts
@@ -75,16 +79,18 @@ __global__ void __launch_bounds__(256) csr_kernel(Geo g, const int32_t* __restri
   for (int x = tid; x < (nseg + 1) * g.m; x += blockDim.x) csr_sm[x] = 0;
   for (int x = tid; x < (E + 31) / 32; x += blockDim.x) bits[x] = 0u;
   __syncthreads();
-  for (int i = tid; i < g.m; i += blockDim.x) {
-    const int32_t* row = idx + (long long)i * g.topk;
-    int* cnt = seg + (long long)(i / rps) * g.m;
-    for (int r = 0; r < g.topk; ++r) {
-      bool report;
-      if (selected_entry_ok(g, row, i, r, &report)) {
-        atomicAdd(&cnt[row[r]], 1);
-        const int e = i * g.topk + r;
-        atomicOr(&bits[e >> 5], 1u << (e & 31));
-      }
+  int lanes = 1;  // lanes of a row: the power of two that holds topk
+  while (lanes < g.topk) lanes *= 2;
+  const int per = 32 / lanes, sub = lane / lanes, r = lane - sub * lanes;
+#pragma unroll 2
+  for (int i0 = warp * per; i0 < g.m; i0 += kCsrThreads / 32 * per) {  // a lane per entry
+    const int i = i0 + sub, e = i * g.topk + r;
+    const int j = i < g.m && r < g.topk ? __ldg(idx + e) : -1;
+    const bool in = j >= 0 && j < g.m;
+    const unsigned twins = __match_any_sync(0xffffffffu, in ? j * 32 + sub : -1 - lane);
+    if (in && (__ffs(twins) - 1) == lane && !is_local(g, i, j)) {
+      atomicAdd(&seg[(long long)(i / rps) * g.m + j], 1);
+      atomicOr(&bits[e >> 5], 1u << (e & 31));
     }
   }
   __syncthreads();
@@ -98,22 +104,35 @@ __global__ void __launch_bounds__(256) csr_kernel(Geo g, const int32_t* __restri
     tot[j] = t;
   }
   __syncthreads();
-  if (tid < 32) {
-    int carry = 0;
-    for (int base = 0; base < g.m; base += 32) {
-      const int j = base + lane;
-      const int v = j < g.m ? tot[j] : 0;
-      int incl = v;
+  __shared__ int wsum[kCsrThreads / 32];
+  int carry = 0;
+  for (int base = 0; base < g.m; base += kCsrThreads) {
+    const int j = base + tid;
+    const int v = j < g.m ? tot[j] : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int nb = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += nb;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      int s = lane < kCsrThreads / 32 ? wsum[lane] : 0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int nb = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += nb;
+        const int nb = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += nb;
       }
-      if (j < g.m) { off[j] = carry + incl - v; tot[j] = carry + incl - v; }
-      carry += __shfl_sync(0xffffffffu, incl, 31);
+      if (lane < kCsrThreads / 32) wsum[lane] = s;
     }
-    if (lane == 0) off[g.m] = carry;
+    __syncthreads();
+    const int at = carry + incl - v + (warp > 0 ? wsum[warp - 1] : 0);
+    if (j < g.m) { off[j] = at; tot[j] = at; }
+    carry += wsum[kCsrThreads / 32 - 1];
+    __syncthreads();
   }
+  if (tid == 0) off[g.m] = carry;
   __syncthreads();
   for (int sgm = warp; sgm < nseg; sgm += (int)(blockDim.x >> 5)) {
     int* cur = seg + (long long)sgm * g.m;  // only this warp touches this segment's cursors
@@ -136,10 +155,10 @@ __global__ void __launch_bounds__(256) csr_kernel(Geo g, const int32_t* __restri
   }
 }
 
-// segments of the transposed-pattern kernel that fit the shared memory (8 when possible: one per warp)
+// segments of the transposed-pattern kernel that fit the shared memory (one per warp when possible)
 static int csr_segments(const Geo& g, size_t* smem) {
   const size_t budget = 200 * 1024, bits = 4 * (((size_t)g.m * g.topk + 31) / 32);
-  int nseg = 8;
+  int nseg = kCsrThreads / 32;
   while (nseg > 1 && (size_t)(nseg + 1) * g.m * sizeof(int) + bits > budget) --nseg;
   *smem = (size_t)(nseg + 1) * g.m * sizeof(int) + bits;
   return *smem <= budget ? nseg : 0;
@@ -148,7 +167,7 @@ static int csr_segments(const Geo& g, size_t* smem) {
 int launch_rowdot(const HostCtx& c, const void* o, const void* d_o, const float* lse, float* neg_d, float* neg_lse2) {
   const long long tokens = (long long)c.g.U * c.g.N, threads = tokens * 8;
   rowdot_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c.stream>>>(tokens, (const uint4*)o, (const uint4*)d_o, lse,
-                                                                         neg_d, neg_lse2, c.g.f16 != 0);
+                                                                         neg_d, neg_lse2, c.g.f16 != 0, c.status);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 
@@ -168,7 +187,7 @@ int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, co
         return MOSAIC_E_CUDA;
       configured |= 1ull << dev;
     }
-    csr_kernel<<<g.U, 256, smem, c.stream>>>(g, block_idx, csr_off, csr_q, nseg);
+    csr_kernel<<<g.U, kCsrThreads, smem, c.stream>>>(g, block_idx, csr_off, csr_q, nseg);
   } else {
     if (cudaMemsetAsync(csr_off, 0, sizeof(int32_t) * (size_t)g.U * (g.m + 1), c.stream) != cudaSuccess)
       return MOSAIC_E_CUDA;

@@ -77,22 +77,6 @@ __device__ __forceinline__ bool is_local(const Geo& g, int i, int j) {
   return row_ok && col_ok;
 }
 
-// Is entry r of a row of block_idx (query block i) one the kernels use?  Ids outside [0, m), ids inside the
-// row's local set (already attended through the neighbourhood) and repeats of an earlier entry of the row are
-// not: they are skipped, and reported unless the entry is the padding value -1.
-__device__ __forceinline__ bool selected_entry_ok(const Geo& g, const int32_t* __restrict__ idx_row, int i, int r,
-                                                  bool* report) {
-  const int j = idx_row[r];
-  *report = false;
-  if (j == -1) return false;
-  *report = true;
-  if (j < 0 || j >= g.m || is_local(g, i, j)) return false;
-  for (int a = 0; a < r; ++a)
-    if (idx_row[a] == j) return false;
-  *report = false;
-  return true;
-}
-
 // First token (row-major grid index inside the unit) of row `r` of chunk `c` of block j.
 __device__ __forceinline__ long long chunk_row_token(const Geo& g, int j, int c, int r) {
   int by = j / g.nbw, bx = j - by * g.nbw;
@@ -120,6 +104,9 @@ struct HostCtx {
 };
 
 int validate(const mosaic_bsa_params* p, Geo* g);
+// Current device, its SM count (cached), and the opt-in to `smem` bytes of dynamic shared memory for `func`
+// (set once per device; `done` is the caller's per-kernel bit set of devices already configured).
+int launch_setup(const void* func, size_t smem, unsigned long long* done, int* sms);
 size_t align256(size_t x);
 
 // kernel launchers (one per translation unit)
@@ -144,16 +131,33 @@ struct FwdOut {
 int launch_fwd_tc(const HostCtx& c, int mode, const void* q, const void* k, const void* v, const int32_t* block_idx,
                   const FwdOut& out, int* work_counter);
 // Layout of the three-branch forward's scratch behind the status block
-struct BranchWs { size_t pq, pk, pv, nrm, ocg, total; };
+struct BranchWs { size_t pq, pk, pv, ocg, total; };
 BranchWs branch_layout(const Geo& g);
-int launch_pool_one(const HostCtx& c, const void* x, float* pooled, float* norm, int units);
+// Block sums (pool.cu).  A job is one tensor of `units` units, with or without norm bounds; with gates ([units, N, 3] fp32)
+// every token is weighted by its first gate.  The launch also resets the status block.
+constexpr int kPoolJobs = 4;
+struct PoolJob {
+  const void* src;
+  float *dst, *norm;
+  const float* gates;
+  int units;
+};
+struct PoolArgs {
+  PoolJob job[kPoolJobs];
+  int n;
+  int* status;
+};
+int launch_pool(const HostCtx& c, PoolArgs a);
 // `lse2` (may be null): base-2 log-sum-exp of every query block's block-level logits, [U, m]
 int launch_compress(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* pooled_v, float* ocg,
                     float* lse2);
-// backward of the three-branch form (branches_bwd.cu)
-int launch_gated_pool(const HostCtx& c, const void* d_o, const float* gates, float* dob);
-int launch_compress_bwd(const HostCtx& c, const float* pq, const float* pk, const float* pv, const float* dob,
-                        const float* ocg, const float* lse2, float* delta, float* dqm, float* dkm, float* dvm);
+// backward of the compression branch: pooled sums, dobar, obar and its log-sum-exp in; what every token of a block receives
+// out (dqm [U, m, d], dkm, dvm [Ukv, m, d])
+struct CompressBwd {
+  const float *pq, *pk, *pv, *dob, *ocg, *lse2;
+  float *dqm, *dkm, *dvm;
+};
+int launch_compress_bwd(const HostCtx& c, const CompressBwd& a);
 int launch_rope(const HostCtx& c, const void* q, const void* k, const float* pos, double theta, void* q_out, void* k_out);
 // What the attention backward reads per query row, [U, N] fp32: the negated base-2 log-sum-exp and -<dO, O>.  Three-branch
 // form (gate set): two planes of each (local blocks, selected blocks), the second of them scaled by the gate, the gates

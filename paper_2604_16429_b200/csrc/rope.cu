@@ -6,8 +6,10 @@
 // [d/2, d) to the latitude; inside a half of width D = d/2 the pair (2i, 2i+1) turns by pos * theta^(-2i/D).
 //
 // HBM-bound: every element of Q and K is read and written once.  Eight lanes per token, a lane owns eight channels
-// (four pairs, 16 bytes) and walks all units of both tensors with the same four (cos, sin), which it computes once
-// in fp64; the rotation is fp64 too (a few fp64 FMAs per 16 bytes moved), rounded to fp32 and then to the storage type.
+// (four pairs, 16 bytes) and walks its share of the units of both tensors with the same four (cos, sin), which it computes
+// once in fp64; the rotation is fp64 too, rounded to fp32 and then to the storage type.  The conversions set the pace if
+// they are left to the conversion unit (16 a clock and SM; two an element took 94 us for 377 MB): the 16-bit patterns are
+// moved into the exponent and mantissa of a double instead, which leaves a power of two that the (cos, sin) carry.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -16,23 +18,53 @@ namespace mosaic {
 
 namespace {
 
-__device__ __forceinline__ uint4 rotate8(const uint4& v, const double (&c)[4], const double (&s)[4], bool f16) {
+// Value of a 16-bit pattern times 2^-896 (bf16) or 2^-1008 (binary16), exactly: sign, exponent and mantissa at their places
+// in a double.  Infinities and NaNs (all exponent bits set) come out finite and are the caller's to catch.
+template <bool F16>
+__device__ __forceinline__ double scaled_lo(uint32_t x) {
+  const uint32_t s = x << 16;
+  return __hiloint2double((int)((s & 0x80000000u) | ((s >> (F16 ? 6 : 3)) & (F16 ? 0x01ffffffu : 0x0fffffffu))), 0);
+}
+template <bool F16>
+__device__ __forceinline__ double scaled_hi(uint32_t x) {
+  const uint32_t s = x & 0xffff0000u;
+  return __hiloint2double((int)((s & 0x80000000u) | ((s >> (F16 ? 6 : 3)) & (F16 ? 0x01ffffffu : 0x0fffffffu))), 0);
+}
+
+template <bool F16>
+__device__ __forceinline__ uint4 rotate8(const uint4& v, const double (&c)[4], const double (&s)[4]) {
+  constexpr uint32_t kExp = F16 ? 0x7c007c00u : 0x7f807f80u, kOne = F16 ? 0x04000400u : 0x00800080u;
+  constexpr double kUnscale = F16 ? 0x1p-1008 : 0x1p-896;
   const uint32_t x[4] = {v.x, v.y, v.z, v.w};
   uint32_t r[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float lo, hi;
-    unpack16x2(x[i], f16, lo, hi);
-    const double x0 = (double)lo, x1 = (double)hi;
-    const float y0 = __double2float_rn(x0 * c[i] - x1 * s[i]), y1 = __double2float_rn(x0 * s[i] + x1 * c[i]);
-    r[i] = pack16x2(y0, y1, f16);
+    float y0, y1;
+    if (((x[i] & kExp) + kOne) & 0x80008000u) {  // an infinity or a NaN in the pair
+      float lo, hi;
+      unpack16x2(x[i], F16, lo, hi);
+      const double cc = c[i] * kUnscale, ss = s[i] * kUnscale;
+      y0 = __double2float_rn((double)lo * cc - (double)hi * ss);
+      y1 = __double2float_rn((double)lo * ss + (double)hi * cc);
+    } else {
+      const double x0 = scaled_lo<F16>(x[i]), x1 = scaled_hi<F16>(x[i]);
+      y0 = __double2float_rn(x0 * c[i] - x1 * s[i]);
+      y1 = __double2float_rn(x0 * s[i] + x1 * c[i]);
+    }
+    r[i] = pack16x2(y0, y1, F16);
   }
   return make_uint4(r[0], r[1], r[2], r[3]);
 }
 
+constexpr int kFreqs = kD / 4;  // frequencies of a half
+
+template <bool F16>
 __global__ void __launch_bounds__(256) rope_kernel(Geo g, const uint4* __restrict__ q, const uint4* __restrict__ k,
                                                    const float* __restrict__ pos, double theta,
                                                    uint4* __restrict__ q_out, uint4* __restrict__ k_out) {
+  __shared__ double freq[kFreqs];
+  if (threadIdx.x < kFreqs) freq[threadIdx.x] = pow(theta, -2.0 * threadIdx.x / (kD / 2));
+  __syncthreads();
   const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // token of the grid
   const int part = threadIdx.x & 7;
   if (x >= g.N) return;
@@ -40,18 +72,22 @@ __global__ void __launch_bounds__(256) rope_kernel(Geo g, const uint4* __restric
   double c[4], s[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int i = 4 * (part & 3) + j;                         // pair inside the half, D = kD / 2
-    sincos(p * pow(theta, -2.0 * i / (kD / 2)), &s[j], &c[j]);
+    sincos(p * freq[4 * (part & 3) + j], &s[j], &c[j]);  // pair 4 (part & 3) + j inside the half
+    s[j] *= F16 ? 0x1p1008 : 0x1p896;
+    c[j] *= F16 ? 0x1p1008 : 0x1p896;
+  }
+  // this block's share of the units of Q, then of K
+  const int total = g.U + g.Ukv, per = (total + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int u0 = (int)blockIdx.y * per, u1 = min(total, u0 + per);
+#pragma unroll 4
+  for (int u = u0; u < min(u1, g.U); ++u) {
+    const long long at = ((long long)u * g.N + x) * 8 + part;
+    q_out[at] = rotate8<F16>(__ldg(q + at), c, s);
   }
 #pragma unroll 4
-  for (int u = 0; u < g.U; ++u) {
+  for (int u = max(u0, g.U) - g.U; u < u1 - g.U; ++u) {
     const long long at = ((long long)u * g.N + x) * 8 + part;
-    q_out[at] = rotate8(__ldg(q + at), c, s, g.f16 != 0);
-  }
-#pragma unroll 4
-  for (int u = 0; u < g.Ukv; ++u) {
-    const long long at = ((long long)u * g.N + x) * 8 + part;
-    k_out[at] = rotate8(__ldg(k + at), c, s, g.f16 != 0);
+    k_out[at] = rotate8<F16>(__ldg(k + at), c, s);
   }
 }
 
@@ -61,8 +97,14 @@ int launch_rope(const HostCtx& c, const void* q, const void* k, const float* pos
   const Geo& g = c.g;
   const long long blocks = (g.N * 8 + 255) / 256;
   if (blocks > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  rope_kernel<<<(unsigned)blocks, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pos, theta, (uint4*)q_out,
-                                                      (uint4*)k_out);
+  // short sequences: the units are split too, until the GPU is full (148 SMs x 8 CTAs) or a share is down to four units
+  int split = 1;
+  while (blocks * split < 1184 && split * 8 <= g.U + g.Ukv) split *= 2;
+  const dim3 grid((unsigned)blocks, (unsigned)split);
+  if (g.f16)
+    rope_kernel<true><<<grid, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pos, theta, (uint4*)q_out, (uint4*)k_out);
+  else
+    rope_kernel<false><<<grid, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pos, theta, (uint4*)q_out, (uint4*)k_out);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 

@@ -1,4 +1,4 @@
-// Selection: block pooling, block-level scores, per-query-block top-k.
+// Selection: block-level scores on the pooled sums, per-query-block top-k.
 //
 // Paper, section "Block-Sparse Attention": paragraph "Compression" defines the pooled block
 // representations (phi = mean pooling) and the block-level score; paragraph "Selection" takes the
@@ -12,64 +12,6 @@
 #include "common.cuh"
 
 namespace mosaic {
-
-// ------------------------------------------------------------------------------------------
-// pool_kernel: eight lanes per (tensor, unit, block), four blocks per warp; a lane owns eight
-// consecutive channels (one 16-byte load per token) and adds them in token order, row-major inside
-// the block, so every channel is one sequential fp64 chain.  HBM-bound: reads 2*U*N*d*2 bytes once;
-// the loads of a whole block row are in flight together.  Beside the pooled sums it writes an upper
-// bound of each pooled vector's Euclidean norm, which the ranking kernel's screening pass needs.
-// ------------------------------------------------------------------------------------------
-template <int BW>
-__global__ void __launch_bounds__(256) pool_kernel(Geo g, const uint4* __restrict__ q, const uint4* __restrict__ k,
-                                                   float* __restrict__ pq, float* __restrict__ pk,
-                                                   float* __restrict__ nq, float* __restrict__ nk, int ntens, int units) {
-  const int sub = threadIdx.x & 7;  // which 8 channels
-  const long long grp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-  const long long per_tensor = (long long)units * g.m;
-  const bool live = grp < ntens * per_tensor;  // the last warp may be partly idle; it still takes part in the shuffles
-  const int which = live && grp >= per_tensor;
-  const long long w = live ? grp - which * per_tensor : 0;
-  const int u = (int)(w / g.m), j = (int)(w - (long long)u * g.m);
-  const uint4* src = (which ? k : q) + (long long)u * g.N * (kD / 8) + sub;
-  const int by = j / g.nbw, bx = j - by * g.nbw;
-  double acc[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-  for (int r = 0; r < g.bh && live; ++r) {
-    const uint4* row = src + ((long long)(by * g.bh + r) * g.nlon + bx * BW) * (kD / 8);
-    uint4 v[BW];
-#pragma unroll
-    for (int c = 0; c < BW; ++c) v[c] = __ldg(row + c * (kD / 8));
-#pragma unroll
-    for (int c = 0; c < BW; ++c) {
-      const uint32_t x[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float lo, hi;
-        unpack16x2(x[e], g.f16 != 0, lo, hi);
-        acc[2 * e] += (double)lo;
-        acc[2 * e + 1] += (double)hi;
-      }
-    }
-  }
-  float p[8];
-  double ss = 0.0;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    p[c] = (float)acc[c];
-    ss += (double)p[c] * (double)p[c];
-  }
-  ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-  ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-  ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-  if (!live) return;
-  float4* dst = reinterpret_cast<float4*>((which ? pk : pq) + ((long long)u * g.m + j) * kD + 8 * sub);
-  dst[0] = make_float4(p[0], p[1], p[2], p[3]);
-  dst[1] = make_float4(p[4], p[5], p[6], p[7]);
-  // rounded up twice, so that it is never below the norm of the fp32 vector (NaN and inf pass through)
-  if (sub == 0) (which ? nk : nq)[(long long)u * g.m + j] = __fmul_ru(__double2float_ru(sqrt(ss)), 1.000001f);
-}
 
 // ------------------------------------------------------------------------------------------
 // topk_kernel<NW, RI, CAP>: ranking of the key blocks of NW * RI query blocks of one unit (warp w owns RI
@@ -510,36 +452,14 @@ int launch_topk(const HostCtx& c, const float* pooled_q, const float* pooled_k, 
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 
-// block sums (and norm bounds) of one tensor of `units` units
-int launch_pool_one(const HostCtx& c, const void* x, float* pooled, float* norm, int units) {
-  const Geo& g = c.g;
-  const long long threads = 1ll * units * g.m * 8;
-  const unsigned blocks = (unsigned)((threads + 255) / 256);
-  if (g.bw == 8)
-    pool_kernel<8><<<blocks, 256, 0, c.stream>>>(g, (const uint4*)x, (const uint4*)x, pooled, pooled, norm, norm, 1, units);
-  else
-    pool_kernel<16><<<blocks, 256, 0, c.stream>>>(g, (const uint4*)x, (const uint4*)x, pooled, pooled, norm, norm, 1, units);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
-}
-
 int launch_select(const HostCtx& c, const void* q, const void* k, int32_t* block_idx, float* pooled_q,
                   float* pooled_k, float* norm_q, float* norm_k) {
   const Geo& g = c.g;
-  if (g.Ukv != g.U) {  // grouped-query attention: Q and K have different head counts, one launch each
-    int rc = launch_pool_one(c, q, pooled_q, norm_q, g.U);
-    if (!rc) rc = launch_pool_one(c, k, pooled_k, norm_k, g.Ukv);
-    if (rc) return rc;
-  } else {
-    const long long threads = 2ll * g.U * g.m * 8;
-    const unsigned blocks = (unsigned)((threads + 255) / 256);
-    if (g.bw == 8)
-      pool_kernel<8><<<blocks, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pooled_q, pooled_k, norm_q,
-                                                   norm_k, 2, g.U);
-    else
-      pool_kernel<16><<<blocks, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pooled_q, pooled_k, norm_q,
-                                                    norm_k, 2, g.U);
-    if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
-  }
+  PoolArgs a = {};
+  a.n = 2;
+  a.job[0] = {q, pooled_q, norm_q, nullptr, g.U};
+  a.job[1] = {k, pooled_k, norm_k, nullptr, g.Ukv};
+  if (const int rc = launch_pool(c, a)) return rc;
   if (g.topk > 0) {
     // the most query blocks per CTA (64, 32, 16) that still gives every SM about two CTAs; small problems are
     // latency-bound and take 8 rows per CTA and 64-key chunks, so that more warps are resident.  The survivors of a

@@ -61,9 +61,8 @@ extern "C" int mosaic_bsa_select_static(const mosaic_bsa_params* p, const void* 
   if ((rc = scratch_address(&base))) return rc;
   c.stream = (cudaStream_t)cuda_stream;
   c.status = reinterpret_cast<int*>(base);
-  // the array keeps what the previous call left: the status block must start at zero; the pooled sums and
-  // norm bounds are fully rewritten by the pooling kernel before the ranking kernel reads them
-  if (cudaMemsetAsync(base, 0, kStatusBytes, c.stream) != cudaSuccess) return MOSAIC_E_CUDA;
+  // the array keeps what the previous call left: the pooling kernel rewrites the status block, the pooled sums and the
+  // norm bounds before the ranking kernel reads them
   return launch_select(c, q, k, block_idx, reinterpret_cast<float*>(base + w.pq), reinterpret_cast<float*>(base + w.pk),
                        reinterpret_cast<float*>(base + w.nq), reinterpret_cast<float*>(base + w.nk));
 }

@@ -663,8 +663,4 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 bool make_map(CUtensorMap* map, const void* base, const Geo& g, int units);
 // [units, nlat, nlon] fp32 view (one value per token), box = the 64 tokens of one chunk {bw, 64/bw, 1}, no swizzle.
 bool make_map_rows(CUtensorMap* map, const void* base, const Geo& g, int units);
-// Current device, its SM count (cached), and the opt-in to `smem` bytes of dynamic shared memory for `func`
-// (set once per device; `done` is the caller's per-kernel bit set of devices already configured).
-int launch_setup(const void* func, size_t smem, unsigned long long* done, int* sms);
-
 }  // namespace mosaic
