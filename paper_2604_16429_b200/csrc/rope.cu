@@ -37,29 +37,53 @@ __device__ __forceinline__ uint4 rotate8(const uint4& v, const double (&c)[4], c
   constexpr double kUnscale = F16 ? 0x1p-1008 : 0x1p-896;
   const uint32_t x[4] = {v.x, v.y, v.z, v.w};
   uint32_t r[4];
+  if ((((x[0] & kExp) + kOne) | ((x[1] & kExp) + kOne) | ((x[2] & kExp) + kOne) | ((x[3] & kExp) + kOne)) & 0x80008000u) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float y0, y1;
-    if (((x[i] & kExp) + kOne) & 0x80008000u) {  // an infinity or a NaN in the pair
+    for (int i = 0; i < 4; ++i) {  // an infinity or a NaN among them
       float lo, hi;
       unpack16x2(x[i], F16, lo, hi);
       const double cc = c[i] * kUnscale, ss = s[i] * kUnscale;
-      y0 = __double2float_rn((double)lo * cc - (double)hi * ss);
-      y1 = __double2float_rn((double)lo * ss + (double)hi * cc);
-    } else {
-      const double x0 = scaled_lo<F16>(x[i]), x1 = scaled_hi<F16>(x[i]);
-      y0 = __double2float_rn(x0 * c[i] - x1 * s[i]);
-      y1 = __double2float_rn(x0 * s[i] + x1 * c[i]);
+      r[i] = pack16x2(__double2float_rn((double)lo * cc - (double)hi * ss), __double2float_rn((double)lo * ss + (double)hi * cc), F16);
     }
-    r[i] = pack16x2(y0, y1, F16);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double x0 = scaled_lo<F16>(x[i]), x1 = scaled_hi<F16>(x[i]);
+      r[i] = pack16x2(__double2float_rn(x0 * c[i] - x1 * s[i]), __double2float_rn(x0 * s[i] + x1 * c[i]), F16);
+    }
   }
   return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
+// Units u0 .. u1 of one tensor, this lane's 16 bytes of each: four at a time, the next four fetched before these are turned.
+template <bool F16>
+__device__ __forceinline__ void turn_units(const uint4* __restrict__ src, uint4* __restrict__ dst, int u0, int u1,
+                                           long long step, const double (&c)[4], const double (&s)[4]) {
+  src += u0 * step;
+  dst += u0 * step;
+  uint4 v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (u0 + i < u1) v[i] = __ldg(src + i * step);
+  for (int u = u0; u < u1; u += 4) {
+    src += 4 * step;
+    uint4 n[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (u + 4 + i < u1) n[i] = __ldg(src + i * step);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (u + i < u1) dst[i * step] = rotate8<F16>(v[i], c, s);
+      v[i] = n[i];
+    }
+    dst += 4 * step;
+  }
 }
 
 constexpr int kFreqs = kD / 4;  // frequencies of a half
 
 template <bool F16>
-__global__ void __launch_bounds__(256) rope_kernel(Geo g, const uint4* __restrict__ q, const uint4* __restrict__ k,
+__global__ void __launch_bounds__(256, 4) rope_kernel(Geo g, const uint4* __restrict__ q, const uint4* __restrict__ k,
                                                    const float* __restrict__ pos, double theta,
                                                    uint4* __restrict__ q_out, uint4* __restrict__ k_out) {
   __shared__ double freq[kFreqs];
@@ -76,19 +100,12 @@ __global__ void __launch_bounds__(256) rope_kernel(Geo g, const uint4* __restric
     s[j] *= F16 ? 0x1p1008 : 0x1p896;
     c[j] *= F16 ? 0x1p1008 : 0x1p896;
   }
-  // this block's share of the units of Q, then of K
+  // this block's share of the units (Q's, then K's)
   const int total = g.U + g.Ukv, per = (total + (int)gridDim.y - 1) / (int)gridDim.y;
   const int u0 = (int)blockIdx.y * per, u1 = min(total, u0 + per);
-#pragma unroll 4
-  for (int u = u0; u < min(u1, g.U); ++u) {
-    const long long at = ((long long)u * g.N + x) * 8 + part;
-    q_out[at] = rotate8<F16>(__ldg(q + at), c, s);
-  }
-#pragma unroll 4
-  for (int u = max(u0, g.U) - g.U; u < u1 - g.U; ++u) {
-    const long long at = ((long long)u * g.N + x) * 8 + part;
-    k_out[at] = rotate8<F16>(__ldg(k + at), c, s);
-  }
+  const long long row = x * 8 + part, step = g.N * 8;
+  turn_units<F16>(q + row, q_out + row, u0, min(u1, g.U), step, c, s);
+  turn_units<F16>(k + row, k_out + row, max(u0, g.U) - g.U, u1 - g.U, step, c, s);
 }
 
 }  // namespace

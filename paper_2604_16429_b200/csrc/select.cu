@@ -14,26 +14,28 @@
 namespace mosaic {
 
 // ------------------------------------------------------------------------------------------
-// topk_kernel<NW, RI, CAP>: ranking of the key blocks of NW * RI query blocks of one unit (warp w owns RI
-// rows; a lane owns the keys lane, lane + 32, ... of every 128-key chunk that streams through shared memory).
+// topk_kernel<TI, CAP>: ranking of the key blocks of TI query blocks of one unit by a CTA of eight warps.
 //
 // The ids must be those of the exact fp64 scores, but almost all of the m scores of a row are irrelevant,
-// so the kernel screens in fp32 and scores exactly only what survives:
-//   1. screening score  s~ = fp32 FMA chain over the channels.  |s~ - s| <= gamma_64 * sum|a_c||b_c|
-//      <= 2^-18 (1 + 1e-5) |a||b|  (standard bound of a length-64 dot product, any order, FMA or not;
-//      Cauchy-Schwarz).  The kernel uses eps = 2^-16 * na * nb + 1e-37 with the norm bounds of the pooling
-//      kernel: four times the bound, which also covers the rounding of s~ -+ eps and subnormal products.
-//      A non-finite s~ or eps makes the candidate's interval (-inf, +inf).
-//   2. every lane tracks the two largest lower bounds s~ - eps among its own keys; the k-th largest of
-//      those 64 values is a lower bound thr of the row's k-th best exact score (they belong to k distinct
-//      candidates).  A candidate with s~ + eps < thr is worse than k others whatever the ties: dropped.
-//      Chunks are visited from the CTA's own neighbourhood outwards (on smooth fields the best keys are
-//      near, so the threshold is tight at once); the first chunk is screened twice, first for a threshold only.
-//   3. survivors (id and upper bound) collect in shared memory, pruned when thr has risen; a row whose
-//      survivors overflow (massive ties) falls back to scoring every key exactly.
-//   4. exact phase: the fp64 chain of the selection's definition for every survivor of the warp's rows
-//      (lanes take survivors, two chains in flight each), then each row ranks its survivors by
-//      (score descending, id ascending) by counting, and ranks 0..k-1 are written.
+// so the kernel screens with tensor cores and scores exactly only what survives:
+//   1. screening score  s~: the fp32 vectors are split into two bf16 parts each (a = ah + al + ea, |al| <= 2^-9 |a|,
+//      |ea| <= 2^-18 |a| per channel) and s~ = ah.bh + ah.bl + al.bh by mma.sync with fp32 accumulation.  What is left
+//      out (al.bl and the ea, eb terms) is at most 3 * 2^-18 (1 + 2^-8) |a||b| by Cauchy-Schwarz; twelve accumulation steps of
+//      sixteen exact products, each step off by at most 17 * 2^-23 |a||b| even if it truncates, add 2^-15.3 |a||b|.
+//      The kernel uses eps = 2^-14 * na * nb + 1e-37 with the norm bounds of the pooling kernel, 1.8 times the sum.  A
+//      non-finite s~, and vectors so short that their parts may be subnormal, make the candidate's interval (-inf, +inf).
+//   2. first pass: every lane keeps the largest lower bounds s~ - eps of its share of a row's keys; the k-th largest of
+//      the row's 64 kept values is a lower bound thr of the row's k-th best exact score (they belong to k distinct
+//      candidates).
+//   3. second pass, the same products again: a candidate with s~ + eps < thr is worse than k others whatever the ties;
+//      the rest (about 1.2 k of them) collect in shared memory.  A row whose survivors overflow (massive ties) falls back
+//      to scoring every key exactly.
+//   4. exact phase: the fp64 chain of the selection's definition for every survivor of the warp's rows (lanes take
+//      survivors, two chains in flight each), then each row ranks its survivors by (score descending, id ascending) by
+//      counting, and ranks 0..k-1 are written.
+// Screening twice costs less than keeping a threshold current during one pass did: with FMAs on the CUDA cores, their
+// operand loads (6 words per 8 FMAs) and the running thresholds a warp spent 1770 instructions on 4 rows x 64 keys; now
+// about 200 per pass on 16 rows x 16 keys.
 // ------------------------------------------------------------------------------------------
 
 // Total-order key: larger key = better score.  0 = not a candidate, 1 = NaN.
@@ -60,31 +62,44 @@ __device__ __forceinline__ float from_ordered_bits(unsigned o) {
 
 constexpr int kKStr = kD + 4;   // padded row of the staged vectors (floats): 16-byte reads of one row per lane hit every bank once
 
-template <int NW, int RI, int CAP, int JT>
+constexpr int kTW = 8;           // warps of a ranking CTA
+constexpr int kTJ = 64;          // keys of a chunk
+constexpr int kHStr = kD + 8;    // padded row of the split keys (16-bit elements): ldmatrix reads hit every bank once
+constexpr int kTracked = 64;     // lower bounds kept per row
+
+template <int TI, int CAP>
 struct TopkSmem {
   union {
     struct {
-      float ks[2][JT][kKStr];  // pooled keys of two chunks (one being read, one in flight)
-      float nk[2][JT];         // their norm bounds
+      __nv_bfloat16 kh[2][2][kTJ][kHStr];  // [buffer][high part, low part][key][channel]
+      float nk[2][kTJ];                    // norm bounds of the keys times 2^-14
     } scr;
-    unsigned long long ekey[NW * RI][CAP];  // exact phase: score keys of the rows' survivors (every row that did not overflow)
+    float tracked[TI][kTracked];           // between the passes
+    unsigned long long ekey[TI][CAP];      // exact phase: score keys of the rows' survivors (rows that did not overflow)
   };
-  float qs[NW * RI][kKStr];     // pooled queries of this CTA
-  int surv[NW * RI][CAP];       // surviving key ids per row ...
-  float surv_ub[NW * RI][CAP];  // ... and the upper bound of their score
+  float qs[TI][kKStr];   // pooled queries of this CTA
+  float nq[TI], thr[TI];
+  int cnt[TI];
+  int surv[TI][CAP];     // surviving key ids per row
 };
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
-  const unsigned n = valid ? 16u : 0u;  // 0 source bytes: the destination is filled with zeros
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(n)
+// a = high + low + rest: two floats into packed bf16 high parts and packed low parts
+__device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(x - __low2float(h), y - __high2float(h));
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(p))
                : "memory");
 }
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
-  const unsigned n = valid ? 4u : 0u;
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(n)
-               : "memory");
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // The warp's sorted list of the best candidates so far holds one entry per lane (lane r = rank r).  Offers this
@@ -135,14 +150,26 @@ __device__ __forceinline__ unsigned long long exact_key(const float* qrow, const
   return score_key(s);
 }
 
-template <int NW, int RI, int CAP, int JT, int MB>
-__global__ void __launch_bounds__(NW * 32, MB) topk_kernel(Geo g, const float* __restrict__ pq,
-                                                       const float* __restrict__ pk, const float* __restrict__ nq,
-                                                       const float* __restrict__ nk, int32_t* __restrict__ block_idx) {
+// a / b for 0 <= a < 2^24 and inv = 1.0f / b: the rounded quotient is off by at most one
+__device__ __forceinline__ int quick_div(int a, int b, float inv) {
+  int q = __float2int_rz((float)a * inv);
+  const int r = a - q * b;
+  q += r >= b ? 1 : r < 0 ? -1 : 0;
+  return q;
+}
+
+template <int TI, int CAP>
+__global__ void __launch_bounds__(kTW * 32, 2) topk_kernel(Geo g, const float* __restrict__ pq, const float* __restrict__ pk,
+                                                           const float* __restrict__ nq, const float* __restrict__ nk,
+                                                           int32_t* __restrict__ block_idx) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  using SM = TopkSmem<NW, RI, CAP, JT>;
+  using SM = TopkSmem<TI, CAP>;
   SM& sm = *reinterpret_cast<SM*>(smem_raw);
-  constexpr int TI = NW * RI, NT = NW * 32, KB = JT / 32;  // KB: keys of a chunk per lane
+  constexpr int RT = TI / 16;              // 16-row tiles of the products
+  constexpr int NT8 = RT;                  // 8-key tiles per warp and chunk: the eight warps share RT x 8 of them
+  constexpr int kDepth = kTracked * RT / 32;  // lower bounds a lane keeps per row (32 / RT lanes share a row)
+  constexpr int RI = TI / kTW;             // rows per warp in the exact phase
+  constexpr int NT = kTW * 32;
   const float kInf = __int_as_float(0x7f800000);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles = (g.m + TI - 1) / TI;
@@ -150,215 +177,210 @@ __global__ void __launch_bounds__(NW * 32, MB) topk_kernel(Geo g, const float* _
   const float* pq_u = pq + (long long)u * g.m * kD;
   const float* pk_u = pk + (long long)kv_unit(g, u) * g.m * kD;   // grouped-query attention: the group's key head
   const float* nk_u = nk + (long long)kv_unit(g, u) * g.m;
-  const int nchunks = (g.m + JT - 1) / JT;
+  const int nchunks = (g.m + kTJ - 1) / kTJ;
 
-  auto load_chunk = [&](int ch, int buf) {
-    const int j0 = ch * JT;
-    for (int e = tid; e < JT * (kD / 4); e += NT) {
-      const int jj = e / (kD / 4), c4 = e - jj * (kD / 4);
-      const bool valid = j0 + jj < g.m;
-      cp_async16(&sm.scr.ks[buf][jj][4 * c4], pk_u + (long long)(valid ? j0 + jj : 0) * kD + 4 * c4, valid);
-    }
-    for (int jj = tid; jj < JT; jj += NT) {
-      const bool valid = j0 + jj < g.m;
-      cp_async4(&sm.scr.nk[buf][jj], nk_u + (valid ? j0 + jj : 0), valid);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  // a chunk's keys: four threads per key, sixteen channels each, fetched into registers one chunk ahead
+  float4 stage[4];
+  float stage_n = 0.f;
+  const int sj = tid >> 2, sc = 16 * (tid & 3);
+  auto fetch = [&](int ch) {
+    const int j = ch * kTJ + sj;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      stage[x] = j < g.m ? __ldg(reinterpret_cast<const float4*>(pk_u + (long long)j * kD + sc) + x) : make_float4(0.f, 0.f, 0.f, 0.f);
+    stage_n = j < g.m ? __ldg(nk_u + j) : 0.f;
   };
-  // visiting order: the chunk that holds the middle of this CTA's rows, then alternately the next one above and
-  // below (every chunk once).  seq_next() hands out that sequence.
-  const int c_home = min((i0 + TI / 2) / JT, nchunks - 1);
-  int seq_lo = c_home - 1, seq_hi = c_home + 1, seq_n = 0;
-  auto seq_next = [&]() {
-    int c;
-    if (seq_n == 0) c = c_home;
-    else if (seq_hi < nchunks && (seq_lo < 0 || (seq_n & 1))) c = seq_hi++;
-    else c = seq_lo--;
-    ++seq_n;
-    return c;
+  auto deposit = [&](int buf) {
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      split2(stage[x].x, stage[x].y, hi[2 * x], lo[2 * x]);
+      split2(stage[x].z, stage[x].w, hi[2 * x + 1], lo[2 * x + 1]);
+    }
+    uint4* h = reinterpret_cast<uint4*>(&sm.scr.kh[buf][0][sj][sc]);
+    uint4* l = reinterpret_cast<uint4*>(&sm.scr.kh[buf][1][sj][sc]);
+    h[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    h[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
+    l[0] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    l[1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+    // a vector too short to be split safely (its parts may be subnormal) gets an infinite bound
+    if ((tid & 3) == 0) sm.scr.nk[buf][sj] = stage_n < 1e-30f ? kInf : stage_n * 6.103515625e-5f;
   };
-
-  int ch_cur = seq_next();  // visit 0 (threshold only) and visit 1 both take the home chunk
-  load_chunk(ch_cur, 0);
+  fetch(0);
   for (int e = tid; e < TI * (kD / 4); e += NT) {
     const int r = e / (kD / 4), c4 = e - r * (kD / 4);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i0 + r < g.m) v = __ldg(reinterpret_cast<const float4*>(pq_u + (long long)(i0 + r) * kD + 4 * c4));
     *reinterpret_cast<float4*>(&sm.qs[r][4 * c4]) = v;
   }
+  if (tid < TI) {
+    const float n = i0 + tid < g.m ? __ldg(nq + (long long)u * g.m + i0 + tid) : 1.f;
+    sm.nq[tid] = n < 1e-30f ? kInf : n;
+    sm.cnt[tid] = 0;
+  }
+  deposit(0);
+  __syncthreads();
 
-  // per row of this warp: block coordinates, norm bound, the lane's two best lower bounds, threshold, survivors
-  int iy[RI], ix[RI], cnt[RI], cnt_upd[RI];
-  float nqv[RI], m1[RI], m2[RI], thr[RI];
+  // this warp's part of the products: rows of one 16-row tile, NT8 groups of eight keys
+  const int rt = warp % RT, n0 = (warp / RT) * NT8;
+  const int rr[2] = {16 * rt + (lane >> 2), 16 * rt + (lane >> 2) + 8};  // the lane's two rows
+  uint32_t ah[4][4], al[4][4];
 #pragma unroll
-  for (int a = 0; a < RI; ++a) {
-    const int i = min(i0 + warp * RI + a, g.m - 1);
+  for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const float2 v = *reinterpret_cast<const float2*>(&sm.qs[rr[x & 1]][16 * ks + 8 * (x >> 1) + 2 * (lane & 3)]);
+      split2(v.x, v.y, ah[ks][x], al[ks][x]);
+    }
+  const float nqv[2] = {sm.nq[rr[0]], sm.nq[rr[1]]};
+  // block coordinates of the rows (group mode: of their groups)
+  const float inv_nbw = 1.0f / (float)g.nbw, inv_rlat = 1.0f / (float)max(g.rlat, 1), inv_rlon = 1.0f / (float)max(g.rlon, 1);
+  int iy[2], ix[2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int i = min(i0 + rr[a], g.m - 1);
     iy[a] = i / g.nbw;
     ix[a] = i - iy[a] * g.nbw;
-    nqv[a] = __ldg(nq + (long long)u * g.m + i);
-    m1[a] = -kInf; m2[a] = -kInf; thr[a] = -kInf;
-    cnt[a] = 0; cnt_upd[a] = 0;
+    if (g.local_groups) { iy[a] /= g.rlat; ix[a] /= g.rlon; }
   }
-  const unsigned lower = (1u << lane) - 1u;
+  // block rows (group mode: group rows) that hold keys local to a row of the 16-row tile
+  int iy_lo = (i0 + 16 * rt) / g.nbw, iy_hi = (i0 + 16 * rt + 15) / g.nbw;
+  if (g.local_groups) { iy_lo /= g.rlat; iy_hi /= g.rlat; }
+  else { iy_lo -= g.rlat; iy_hi += g.rlat; }
+  float best[2][kDepth], thr[2] = {0.f, 0.f};
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int d = 0; d < kDepth; ++d) best[a][d] = -kInf;
 
-  // thr <- k-th largest of the warp's tracked lower bounds, for the rows in `rows` (bit a = row a), all of them in
-  // lockstep so that the latencies of their warp-wide steps overlap.  A pop takes the largest out of its lane's pair.
-  auto update_thresholds = [&](unsigned rows) {
-    float t1[RI], t2[RI];
+  int buf = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int ch = 0; ch < nchunks; ++ch) {
+      const bool more = ch + 1 < nchunks || pass == 0;
+      if (more) fetch(ch + 1 < nchunks ? ch + 1 : 0);  // the next chunk streams in while this one is screened
+      const int j0 = ch * kTJ;
+      float c[NT8][4];
 #pragma unroll
-    for (int a = 0; a < RI; ++a) { t1[a] = m1[a]; t2[a] = m2[a]; }
-    for (int r = 0; r + 1 < g.topk; ++r) {
+      for (int n = 0; n < NT8; ++n) {
 #pragma unroll
-      for (int a = 0; a < RI; ++a) {
-        if (!((rows >> a) & 1u)) continue;  // warp-uniform
-        const unsigned o = ordered_bits(t1[a]);
-        const unsigned best = __reduce_max_sync(0xffffffffu, o);
-        const unsigned who = __ballot_sync(0xffffffffu, o == best);
-        if (lane == __ffs(who) - 1) { t1[a] = t2[a]; t2[a] = -kInf; }
-      }
-    }
+        for (int x = 0; x < 4; ++x) c[n][x] = 0.f;
+        // eight keys: per part two loads of four 8 x 8 matrices (channels 0-31, 32-63)
+        uint32_t bh[2][4], bl[2][4];
+        const int key = 8 * (n0 + n) + (lane & 7), col = 8 * (lane >> 3);
 #pragma unroll
-    for (int a = 0; a < RI; ++a)
-      if ((rows >> a) & 1u) thr[a] = from_ordered_bits(__reduce_max_sync(0xffffffffu, ordered_bits(t1[a])));
-  };
-  // drop the survivors of row a that the current threshold rules out (order kept)
-  auto prune = [&](int a) {
-    const int row = warp * RI + a, n = min(cnt[a], CAP);
-    if (cnt[a] > CAP) return;  // overflowed: the row is rescored in full anyway
-    int kept = 0;
-    for (int e0 = 0; e0 < n; e0 += 32) {
-      const int e = e0 + lane;
-      const int j = e < n ? sm.surv[row][e] : 0;
-      const float ub = e < n ? sm.surv_ub[row][e] : 0.f;
-      const bool keep = e < n && !(ub < thr[a]);
-      const unsigned km = __ballot_sync(0xffffffffu, keep);
-      __syncwarp();
-      if (keep) {
-        const int at = kept + __popc(km & lower);
-        sm.surv[row][at] = j;
-        sm.surv_ub[row][at] = ub;
-      }
-      kept += __popc(km);
-      __syncwarp();
-    }
-    cnt[a] = kept;
-  };
-
-  // visit 0 screens the home chunk for a threshold only; visits 1 .. nchunks screen every chunk, the home chunk first
-  for (int v = 0; v <= nchunks; ++v) {
-    const int ch = ch_cur, buf = v & 1;
-    if (v < nchunks) {  // the next visit's chunk streams in while this one is screened
-      ch_cur = v == 0 ? ch : seq_next();
-      load_chunk(ch_cur, buf ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const int j0 = ch * JT;
-    float acc[RI][KB];
-#pragma unroll
-    for (int a = 0; a < RI; ++a)
-#pragma unroll
-      for (int b = 0; b < KB; ++b) acc[a][b] = 0.f;
-#pragma unroll 4
-    for (int c4 = 0; c4 < kD / 4; ++c4) {
-      float4 kv[KB];
-#pragma unroll
-      for (int b = 0; b < KB; ++b) kv[b] = *reinterpret_cast<const float4*>(&sm.scr.ks[buf][lane + 32 * b][4 * c4]);
-#pragma unroll
-      for (int a = 0; a < RI; ++a) {
-        const float4 qv = *reinterpret_cast<const float4*>(&sm.qs[warp * RI + a][4 * c4]);
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-          acc[a][b] = fmaf(qv.x, kv[b].x, acc[a][b]);
-          acc[a][b] = fmaf(qv.y, kv[b].y, acc[a][b]);
-          acc[a][b] = fmaf(qv.z, kv[b].z, acc[a][b]);
-          acc[a][b] = fmaf(qv.w, kv[b].w, acc[a][b]);
+        for (int x = 0; x < 2; ++x) {
+          ldmatrix4(bh[x], &sm.scr.kh[buf][0][key][32 * x + col]);
+          ldmatrix4(bl[x], &sm.scr.kh[buf][1][key][32 * x + col]);
         }
-      }
-    }
-    float nkc[KB];  // norm bound of the lane's keys times 2^-16
 #pragma unroll
-    for (int b = 0; b < KB; ++b) nkc[b] = sm.scr.nk[buf][lane + 32 * b] * 1.52587890625e-5f;
-    unsigned stale = 0;  // rows whose threshold should be recomputed
-    // One candidate: bounds of its exact score, filter against the row's threshold, tracking of the lower bounds.
-    // A non-finite screening score gives the interval (-inf, +inf); a non-finite eps does so by itself (s + eps is
-    // then +inf or NaN, which the filter keeps, and s - eps is -inf or NaN, which the tracking ignores).
-    auto candidate = [&](int a, int b, bool cand) {
-      const float sc = acc[a][b], eps = fmaf(nqv[a], nkc[b], 1e-37f);
-      const bool fin = fabsf(sc) <= 1e38f;
-      const float lb = fin ? sc - eps : -kInf, ub = fin ? sc + eps : kInf;
-      if (v >= 1) {
-        const bool keep = cand && !(ub < thr[a]);
-        const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (km) {  // warp-uniform
-          if (keep) {
-            const int at = cnt[a] + __popc(km & lower);
-            if (at < CAP) { sm.surv[warp * RI + a][at] = j0 + lane + 32 * b; sm.surv_ub[warp * RI + a][at] = ub; }
+        for (int ks = 0; ks < 4; ++ks) {
+          mma_bf16(c[n], al[ks], bh[ks >> 1][2 * (ks & 1)], bh[ks >> 1][2 * (ks & 1) + 1]);
+          mma_bf16(c[n], ah[ks], bl[ks >> 1][2 * (ks & 1)], bl[ks >> 1][2 * (ks & 1) + 1]);
+        }
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          mma_bf16(c[n], ah[ks], bh[ks >> 1][2 * (ks & 1)], bh[ks >> 1][2 * (ks & 1) + 1]);
+      }
+      // Plain chunk for this warp (the common case): wholly inside the grid, every row of the tile exists, and no key of
+      // the chunk can be local to any of the rows, so every (row, key) pair is a candidate.
+      bool plain = j0 + kTJ <= g.m && i0 + 16 * rt + 15 < g.m;
+      if (plain) {
+        int jy_lo = quick_div(j0, g.nbw, inv_nbw), jy_hi = quick_div(j0 + kTJ - 1, g.nbw, inv_nbw);
+        if (g.local_groups) {
+          jy_lo = quick_div(jy_lo, g.rlat, inv_rlat);
+          jy_hi = quick_div(jy_hi, g.rlat, inv_rlat);
+        }
+        plain = jy_lo > iy_hi || jy_hi < iy_lo;
+      }
+#pragma unroll
+      for (int n = 0; n < NT8; ++n) {
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          const int jj = 8 * (n0 + n) + 2 * (lane & 3) + y, j = j0 + jj;
+          const float nkc = sm.scr.nk[buf][jj];
+          bool cand[2] = {true, true};
+          if (!plain) {
+            int jy = quick_div(j, g.nbw, inv_nbw), jx = j - jy * g.nbw;
+            if (g.local_groups) {
+              jy = quick_div(jy, g.rlat, inv_rlat);
+              jx = quick_div(jx, g.rlon, inv_rlon);
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+              int dx = jx - ix[a];
+              dx += dx < 0 ? g.nbw : 0;  // (jx - ix) mod nbw
+              const bool local = g.local_groups ? (jy == iy[a] && jx == ix[a])
+                                                : (abs(jy - iy[a]) <= g.rlat && (dx <= g.rlon || g.nbw - dx <= g.rlon));
+              cand[a] = j < g.m && !local && i0 + rr[a] < g.m;
+            }
           }
-          cnt[a] += __popc(km);
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            const float s = c[n][2 * a + y], eps = fmaf(nqv[a], nkc, 1e-37f);
+            const bool fin = fabsf(s) <= 1e38f;  // (an infinite eps gives the bounds -inf and +inf by itself)
+            if (pass == 0) {
+              float x = fin && cand[a] ? s - eps : -kInf;
+#pragma unroll
+              for (int d = 0; d < kDepth; ++d) {  // insertion into the lane's sorted list
+                const float top = fmaxf(best[a][d], x);
+                x = fminf(best[a][d], x);
+                best[a][d] = top;
+              }
+            } else if (cand[a] && !(fin && s + eps < thr[a])) {
+              const int at = atomicAdd(&sm.cnt[rr[a]], 1);
+              if (at < CAP) sm.surv[rr[a]][at] = j;
+            }
+          }
         }
       }
-      if (v != 1 && cand) {  // the home chunk's bounds were tracked in the threshold-only visit
-        if (lb > m1[a]) { m2[a] = m1[a]; m1[a] = lb; }
-        else m2[a] = fmaxf(m2[a], lb);
+      if (ch + 1 < nchunks) {
+        deposit(buf ^ 1);
+        buf ^= 1;
+        __syncthreads();
       }
-    };
-    // Plain chunk for this warp (the common case): wholly inside the grid, every row of the warp exists, and no key of
-    // the chunk can be local to any of the warp's rows, so every (row, key) pair is a candidate.
-    const int i_lo = i0 + warp * RI, i_hi = i_lo + RI - 1;
-    bool plain = j0 + JT <= g.m && i_hi < g.m;
-    if (plain) {
-      const int jy_lo = j0 / g.nbw, jy_hi = (j0 + JT - 1) / g.nbw, iy_lo = i_lo / g.nbw, iy_hi = i_hi / g.nbw;
-      plain = g.local_groups ? (jy_lo / g.rlat > iy_hi / g.rlat || jy_hi / g.rlat < iy_lo / g.rlat)
-                             : (jy_lo > iy_hi + g.rlat || jy_hi < iy_lo - g.rlat);
     }
-    if (plain) {
+    if (pass == 0) {
+      // thr <- k-th largest of a row's kept lower bounds, two per lane; the rows of a warp in lockstep so that the
+      // latencies of the warp-wide steps overlap.  A pop takes the largest out of its lane's pair.
+      __syncthreads();
 #pragma unroll
-      for (int a = 0; a < RI; ++a)
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < KB; ++b) candidate(a, b, true);
-    } else {
-      int jy[KB], jx[KB];
+        for (int d = 0; d < kDepth; ++d) sm.tracked[rr[a]][((warp / RT) * 4 + (lane & 3)) * kDepth + d] = best[a][d];
+      __syncthreads();
+      float t1[RI], t2[RI];
 #pragma unroll
-      for (int b = 0; b < KB; ++b) {
-        const int j = min(j0 + lane + 32 * b, g.m - 1);
-        jy[b] = j / g.nbw;
-        jx[b] = j - jy[b] * g.nbw;
+      for (int a = 0; a < RI; ++a) {
+        const float x = sm.tracked[warp * RI + a][lane], y = sm.tracked[warp * RI + a][lane + 32];
+        t1[a] = fmaxf(x, y);
+        t2[a] = fminf(x, y);
+      }
+      for (int r = 0; r + 1 < g.topk; ++r) {
+#pragma unroll
+        for (int a = 0; a < RI; ++a) {
+          const unsigned o = ordered_bits(t1[a]);
+          const unsigned top = __reduce_max_sync(0xffffffffu, o);
+          const unsigned who = __ballot_sync(0xffffffffu, o == top);
+          if (lane == __ffs(who) - 1) { t1[a] = t2[a]; t2[a] = -kInf; }
+        }
       }
 #pragma unroll
       for (int a = 0; a < RI; ++a) {
-        const bool row_ok = i_lo + a < g.m;  // warp-uniform
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-          int dx = jx[b] - ix[a];
-          dx += dx < 0 ? g.nbw : 0;  // (jx - ix) mod nbw
-          const bool local = g.local_groups ? (jy[b] / g.rlat == iy[a] / g.rlat && jx[b] / g.rlon == ix[a] / g.rlon)
-                                            : (abs(jy[b] - iy[a]) <= g.rlat && (dx <= g.rlon || g.nbw - dx <= g.rlon));
-          candidate(a, b, row_ok && j0 + lane + 32 * b < g.m && !local);
-        }
+        const float t = from_ordered_bits(__reduce_max_sync(0xffffffffu, ordered_bits(t1[a])));
+        if (lane == 0) sm.thr[warp * RI + a] = t;
       }
+      __syncthreads();  // the kept values are consumed: the first chunk may land in their place
+      buf = 0;
+      deposit(0);
+      __syncthreads();
+      thr[0] = sm.thr[rr[0]];
+      thr[1] = sm.thr[rr[1]];
     }
-#pragma unroll
-    for (int a = 0; a < RI; ++a) {
-      // recompute when the row has no threshold yet, gathered enough new survivors to suggest it is stale, fills
-      // up, or is about to be scored
-      const bool due = v <= 1 || v == nchunks || cnt[a] - cnt_upd[a] >= g.topk / 2 + 4 || cnt[a] > CAP / 2;
-      if (i_lo + a < g.m && due && cnt[a] <= CAP) stale |= 1u << a;
-    }
-    if (stale) {  // warp-uniform
-      __syncwarp();
-      update_thresholds(stale);
-#pragma unroll
-      for (int a = 0; a < RI; ++a)
-        if ((stale >> a) & 1u) {
-          if (v >= 1) prune(a);
-          cnt_upd[a] = cnt[a];
-        }
-    }
-    __syncthreads();  // everyone is done with this buffer before the chunk after next lands in it
   }
+  __syncthreads();  // the survivors are complete, the staging buffers are free
+  int cnt[RI];
+#pragma unroll
+  for (int a = 0; a < RI; ++a) cnt[a] = sm.cnt[warp * RI + a];
 
   // ---- exact phase (the staging buffers are free now and hold the survivors' score keys)
   // rows whose survivors fit the counting rank: flatten (row, entry) pairs over the lanes, two chains in flight
@@ -418,11 +440,7 @@ __global__ void __launch_bounds__(NW * 32, MB) topk_kernel(Geo g, const float* _
         const int j = jb + lane;
         bool cand = j < g.m;
         if (cand) {
-          const int jy = j / g.nbw, jx = j - jy * g.nbw;
-          int dx = jx - ix[a];
-          dx += dx < 0 ? g.nbw : 0;
-          cand = g.local_groups ? !(jy / g.rlat == iy[a] / g.rlat && jx / g.rlon == ix[a] / g.rlon)
-                                : !(abs(jy - iy[a]) <= g.rlat && (dx <= g.rlon || g.nbw - dx <= g.rlon));
+          cand = !is_local(g, i, j);
         }
         insert_batch(cand ? exact_key(sm.qs[row], pk_u, j) : 0ull, j, lkey, lid, g.topk, lane);
       }
@@ -431,24 +449,17 @@ __global__ void __launch_bounds__(NW * 32, MB) topk_kernel(Geo g, const float* _
   }
 }
 
-template <int NW, int RI, int CAP, int JT, int MB>
-int launch_topk(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* norm_q,
-                const float* norm_k, int32_t* block_idx) {
+template <int TI, int CAP>
+int launch_topk(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* norm_q, const float* norm_k,
+                int32_t* block_idx) {
   const Geo& g = c.g;
-  const size_t smem = sizeof(TopkSmem<NW, RI, CAP, JT>);
+  const size_t smem = sizeof(TopkSmem<TI, CAP>);
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return MOSAIC_E_CUDA;
-  if (dev < 0 || dev >= 64) return MOSAIC_E_UNSUPPORTED;
-  if (!((configured >> dev) & 1ull)) {
-    if (cudaFuncSetAttribute(topk_kernel<NW, RI, CAP, JT, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return MOSAIC_E_CUDA;
-    configured |= 1ull << dev;
-  }
-  const int tiles = (g.m + NW * RI - 1) / (NW * RI);
-  topk_kernel<NW, RI, CAP, JT, MB><<<(unsigned)(g.U * tiles), NW * 32, smem, c.stream>>>(g, pooled_q, pooled_k, norm_q,
-                                                                                norm_k, block_idx);
+  int sms = 0;
+  if (const int rc = launch_setup(reinterpret_cast<const void*>(topk_kernel<TI, CAP>), smem, &configured, &sms)) return rc;
+  const long long ctas = (long long)g.U * ((g.m + TI - 1) / TI);
+  if (ctas > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
+  topk_kernel<TI, CAP><<<(unsigned)ctas, kTW * 32, smem, c.stream>>>(g, pooled_q, pooled_k, norm_q, norm_k, block_idx);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 
@@ -461,20 +472,14 @@ int launch_select(const HostCtx& c, const void* q, const void* k, int32_t* block
   a.job[1] = {k, pooled_k, norm_k, nullptr, g.Ukv};
   if (const int rc = launch_pool(c, a)) return rc;
   if (g.topk > 0) {
-    // the most query blocks per CTA (64, 32, 16) that still gives every SM about two CTAs; small problems are
-    // latency-bound and take 8 rows per CTA and 64-key chunks, so that more warps are resident.  The survivors of a
-    // row grow with top-k (the threshold is the k-th best of 64 tracked bounds), and a row whose survivors overflow
-    // scores every key exactly: beyond top-k 16 only the configurations with room for 192 survivors are used.
-    auto ctas = [&](int ti) { return (long long)g.U * ((g.m + ti - 1) / ti); };
-    int rc;
-    if (g.topk > 16)
-      rc = ctas(16) >= 296 ? launch_topk<4, 4, 192, 128, 2>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
-                           : launch_topk<4, 2, 192, 64, 4>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx);
-    else
-      rc = ctas(64) >= 296   ? launch_topk<8, 4, 96, 64, 3>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
-           : ctas(32) >= 296 ? launch_topk<4, 8, 128, 128, 1>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
-           : ctas(16) >= 296 ? launch_topk<4, 4, 192, 128, 2>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
-                             : launch_topk<4, 2, 192, 64, 4>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx);
+    // 32 query blocks per CTA where that still gives every SM about two CTAs, 16 below.  The survivors of a row grow with
+    // top-k (the threshold is the k-th best of 64 kept bounds), and a row whose survivors overflow scores every key
+    // exactly: beyond top-k 16 there is room for 192 of them.
+    const bool wide = (long long)g.U * ((g.m + 31) / 32) >= 296;
+    const int rc = g.topk > 16 ? (wide ? launch_topk<32, 192>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
+                                       : launch_topk<16, 192>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx))
+                               : (wide ? launch_topk<32, 96>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx)
+                                       : launch_topk<16, 96>(c, pooled_q, pooled_k, norm_q, norm_k, block_idx));
     if (rc) return rc;
   }
   return MOSAIC_OK;
