@@ -71,7 +71,7 @@ BranchWs branch_layout(const Geo& g) {
 
 namespace {
 
-struct BwdWs { size_t neg_d, neg_lse2, gate, off, q, order, total; };
+struct BwdWs { size_t neg_d, neg_lse2, gate, gated_do, off, q, order, total; };
 // `planes`: sets of row statistics (two, and the gates, in the three-branch form)
 BwdWs bwd_layout(const Geo& g, int planes, size_t at) {
   BwdWs w;
@@ -79,6 +79,7 @@ BwdWs bwd_layout(const Geo& g, int planes, size_t at) {
   w.neg_d = at; at += rows;
   w.neg_lse2 = at; at += rows;
   w.gate = at; at += planes > 1 ? rows : 0;
+  w.gated_do = at; at += planes > 1 ? align256(2 * (size_t)planes * g.U * g.N * kD) : 0;
   w.off = at; at = align256(at + sizeof(int32_t) * (size_t)g.U * (g.m + 1));
   w.q = at; at = align256(at + sizeof(int32_t) * (size_t)g.U * g.m * (g.topk > 0 ? g.topk : 1));
   // dK/dV items (two 128-row tiles per 256-row item of a key/value unit), longest first, and their cost classes
@@ -283,6 +284,7 @@ int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   out.neg_lse2 = F(w.b.neg_lse2);
   out.neg_d = F(w.b.neg_d);
   out.gate = F(w.b.gate);
+  out.gated_do = base + w.b.gated_do;
   if ((rc = launch_fwd_tc(c, kFwdStats, q, k, v, block_idx, out, c.status + 1))) return rc;
   // compression branch on the block level
   const CompressBwd cb = {pq, pk, pv, F(w.dob), ocg, F(w.lse_cg), F(w.dqm), F(w.dkm), F(w.dvm)};
@@ -292,6 +294,7 @@ int mosaic_bsa_bwd_branches(const mosaic_bsa_params* p, const void* q, const voi
   st.neg_lse2 = out.neg_lse2;
   st.neg_d = out.neg_d;
   st.gate = out.gate;
+  st.gated_do = out.gated_do;
   st.dqm = F(w.dqm);
   st.dkm = F(w.dkm);
   st.dvm = F(w.dvm);

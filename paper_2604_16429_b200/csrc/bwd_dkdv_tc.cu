@@ -38,27 +38,21 @@ constexpr uint32_t kTmemCols = 512;
 // dK, dV accumulators; per chunk of a pair S^T and dP^T (fp32, 64 columns) and P^T and dS^T (bf16 pairs, 32 columns)
 constexpr uint32_t kColDK = 0, kColDV = 64, kColS = 128, kColDP = 256, kColP = 384, kColDS = 448;
 // BR: backward of the three-branch form.  The local and the selected blocks have a softmax of their own, so a query row has
-// two sets of statistics, and its dO is scaled by the branch's gate: P enters dV as gate P, dS = P (gate dP - gate <dO, O>).
-// Statistics of a query row: -LSE*log2e, -D (and the gate, for the local, then for the selected blocks).
-template <bool BR>
-constexpr int kStats = BR ? 6 : 2;
-template <bool BR>
-constexpr uint32_t kChunkBytes = 2 * kTile + kStats<BR> * 64 * 4;
+// two sets of statistics, and its dO is scaled by the branch's gate beforehand: dO and the statistics come in two planes, of
+// which a list entry takes one.
+constexpr uint32_t kChunkBytes = 2 * kTile + 2 * 64 * 4;
 
-template <bool BR>
 struct Slot {
   unsigned char q[2][kTile];     // per chunk 64 query rows x 128 B, swizzled; the two tiles form one 128-row operand
   unsigned char d_o[2][kTile];
-  float stat[kStats<BR>][2][64]; // statistics of the chunks' query rows
+  float stat[2][2][64];          // -LSE * log2(e) and -D of the chunks' query rows
 };
-static_assert(sizeof(Slot<false>) % 1024 == 0 && sizeof(Slot<true>) % 1024 == 0,
-              "slots keep the 1024-byte alignment of the swizzled tiles");
+static_assert(sizeof(Slot) % 1024 == 0, "slots keep the 1024-byte alignment of the swizzled tiles");
 
-template <bool BR>
 struct Smem {
   unsigned char k[2 * kTile];              // 128 key rows x 128 B
   unsigned char v[2 * kTile];
-  Slot<BR> ring[kSlots];
+  Slot ring[kSlots];
   unsigned long long ring_full[kSlots], ring_empty[kSlots];
   unsigned long long kv_full, kv_empty, s_full, sdp_free, p_full[2], pv_done, acc_done, acc_free;
   unsigned long long mma_drain_bar[2];  // abort path: completion of each issuer's outstanding products
@@ -73,7 +67,7 @@ struct Smem {
 // Planner of the key-stationary kernel: per item (tile), the merged local neighbourhoods of its key blocks,
 // then each block's list of selecting query blocks, cut into list buffers.
 template <bool BR>
-__device__ __forceinline__ void planner_kv_loop(Smem<BR>& sm, const Geo& g, const int32_t* __restrict__ csr_off,
+__device__ __forceinline__ void planner_kv_loop(Smem& sm, const Geo& g, const int32_t* __restrict__ csr_off,
                                                 const int32_t* __restrict__ csr_q,
                                                 const int32_t* __restrict__ order, int* work_counter, int ipu,
                                                 int total_items, int lane, volatile int* abort, int* status) {
@@ -224,19 +218,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     dkdv_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                    const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    const __grid_constant__ CUtensorMap map_nlse, const __grid_constant__ CUtensorMap map_nd,
-                   const __grid_constant__ CUtensorMap map_gate, const int32_t* __restrict__ csr_off,
-                   const int32_t* __restrict__ csr_q, const int32_t* __restrict__ order, __nv_bfloat16* __restrict__ dk,
+                   const int32_t* __restrict__ csr_off, const int32_t* __restrict__ csr_q, const int32_t* __restrict__ order, __nv_bfloat16* __restrict__ dk,
                    __nv_bfloat16* __restrict__ dv, const float* __restrict__ dkm, const float* __restrict__ dvm,
                    int* status, int* work_counter, int ipu, int total_items) {
   extern __shared__ unsigned char smem_raw[];
-  Smem<BR>& sm = *reinterpret_cast<Smem<BR>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s) { mbar_init(s32(&sm.ring_full[s]), 1); mbar_init(s32(&sm.ring_empty[s]), 1); }
     mbar_init(s32(&sm.kv_full), 1);
     mbar_init(s32(&sm.kv_empty), 1);
-    mbar_init(s32(&sm.s_full), 1);
+    mbar_init(s32(&sm.s_full), 2);  // the products' completion, and the issuing warp itself
     mbar_init(s32(&sm.sdp_free), 32 * kRowWarps);
     mbar_init(s32(&sm.p_full[0]), 32 * kGroupWarps);
     mbar_init(s32(&sm.p_full[1]), 32 * kGroupWarps);
@@ -258,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // Every role walks the same sequence: list buffers, and inside a buffer its n * cpb chunks two at a time.
   // `pr` counts pairs (ring slot pr % kSlots, phase of the per-pair barriers).
   if (warp == kWPlan) {
-    planner_kv_loop(sm, g, csr_off, csr_q, order, work_counter, ipu, total_items, lane, abort, status);
+    planner_kv_loop<BR>(sm, g, csr_off, csr_q, order, work_counter, ipu, total_items, lane, abort, status);
   } else if (warp == kWProd) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -292,21 +285,18 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int slot = (int)(pr % kSlots), np = min(2, chunks - p0);
           ok = mbar_wait(s32(&sm.ring_empty[slot]), (uint32_t)((pr / kSlots) & 1) ^ 1, abort, status);
           if (!ok) break;
-          Slot<BR>& sl = sm.ring[slot];
+          Slot& sl = sm.ring[slot];
           const uint32_t bar = s32(&sm.ring_full[slot]);
-          mbar_expect_tx(bar, np * kChunkBytes<BR>);
+          mbar_expect_tx(bar, np * kChunkBytes);
           for (int h = 0; h < np; ++h) {
             const int e = (p0 + h) / g.cpb, c = (p0 + h) - e * g.cpb;
             const int i = sm.ids[buf][e], by = i / g.nbw, bx = i - by * g.nbw;
             const int x0 = bx * g.bw, y0 = by * g.bh + c * g.crows;
             tma_load_4d(s32(sl.q[h]), &map_q, bar, 0, x0, y0, u);
-            tma_load_4d(s32(sl.d_o[h]), &map_do, bar, 0, x0, y0, u);
-#pragma unroll
-            for (int pl = 0; pl < (BR ? 2 : 1); ++pl) {  // planes of the statistics: local, selected
-              tma_load_3d(s32(sl.stat[3 * pl][h]), &map_nlse, bar, x0, y0, u + pl * g.U);
-              tma_load_3d(s32(sl.stat[3 * pl + 1][h]), &map_nd, bar, x0, y0, u + pl * g.U);
-              if constexpr (BR) tma_load_3d(s32(sl.stat[3 * pl + 2][h]), &map_gate, bar, x0, y0, u + pl * g.U);
-            }
+            const int uo = BR && sm.mask[buf][e] > 15 ? u + g.U : u;  // plane 0: local, plane 1: selected
+            tma_load_4d(s32(sl.d_o[h]), &map_do, bar, 0, x0, y0, uo);
+            tma_load_3d(s32(sl.stat[0][h]), &map_nlse, bar, x0, y0, uo);
+            tma_load_3d(s32(sl.stat[1][h]), &map_nd, bar, x0, y0, uo);
           }
         }
         if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
@@ -358,6 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) umma_ss(tmem + kColDP, vdesc + 2 * kk, dodesc + 2 * kk, idesc, kk > 0);
           tc_commit(s32(&sm.s_full));
+          mbar_arrive(s32(&sm.s_full));  // what this warp has seen land (the slot), the row threads see through this barrier
         }
         __syncwarp();
       }
@@ -388,8 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int p0 = 0; p0 < chunks && ok; p0 += 2, ++pr) {
         const uint32_t slot = pr % kSlots;
         const bool two = chunks - p0 >= 2;
-        // the slot landed before S^T could be produced; this wait makes the copied Q and dO visible here too
-        ok = warp_wait(s32(&sm.ring_full[slot]), (pr / kSlots) & 1u, abort, status);
+        // (the slot has landed: p_full passes on what the row threads saw through s_full)
         // a new accumulation overwrites dK and dV: every row thread must have read the previous item's
         if (ok && first && items > 0) ok = warp_wait(s32(&sm.acc_free), (items - 1) & 1, abort, status);
 #pragma unroll
@@ -478,13 +468,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool connected = ((BR ? mk | (mk >> 4) : mk) & hbit) != 0;
         uint32_t pp[16], ds[16];
         if (connected) {
-          const uint32_t slot = pr % kSlots;
-          // the slot landed before the MMA warp could produce this S^T; waiting on its barrier here as well
-          // makes the copied -LSE and -D visible to this thread
-          ok = warp_wait(s32(&sm.ring_full[slot]), (pr / kSlots) & 1u, abort, status);
-          if (!ok) break;
-          // statistics of the chunk's query columns for this half's kind of connection
-          const float(*stat)[2][64] = &sm.ring[slot].stat[BR && ((mk >> 4) & hbit) ? 3 : 0];
+          // (the slot has landed: s_full passes on what the issuing warp saw; a wait on the slot's own barrier here cost 8 %)
+          const float(*stat)[2][64] = sm.ring[pr % kSlots].stat;
           uint32_t sv[32], dp[32];
           tmem_ld32(tb + col_s, sv);
           tmem_ld32(tb + col_dp, dp);
@@ -496,25 +481,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             // -LSE*log2(e) and -D of four query columns (the same for every thread: broadcast loads)
             const float4 nl = *reinterpret_cast<const float4*>(&stat[0][grp][32 * ch + i]);
             const float4 nd = *reinterpret_cast<const float4*>(&stat[1][grp][32 * ch + i]);
-            const float4 gt = BR ? *reinterpret_cast<const float4*>(&stat[2][grp][32 * ch + i]) : nd;
             float x0, x1, x2, x3, d0, d1, d2, d3;
             unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), scale2, pack2(nl.x, nl.y)), x0, x1);
             unpack2(fma2(pack2(__uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3])), scale2, pack2(nl.z, nl.w)), x2, x3);
             const float e0 = ex2(x0), e1 = ex2(x1), e2 = ex2(x2), e3 = ex2(x3);
             const uint64_t dp01 = pack2(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1]));
             const uint64_t dp23 = pack2(__uint_as_float(dp[i + 2]), __uint_as_float(dp[i + 3]));
-            const uint64_t g01 = pack2(gt.x, gt.y), g23 = pack2(gt.z, gt.w);
-            const uint64_t t01 = BR ? fma2(dp01, g01, pack2(nd.x, nd.y)) : add2(dp01, pack2(nd.x, nd.y));
-            const uint64_t t23 = BR ? fma2(dp23, g23, pack2(nd.z, nd.w)) : add2(dp23, pack2(nd.z, nd.w));
+            const uint64_t t01 = add2(dp01, pack2(nd.x, nd.y)), t23 = add2(dp23, pack2(nd.z, nd.w));
             unpack2(mul2(pack2(e0, e1), t01), d0, d1);
             unpack2(mul2(pack2(e2, e3), t23), d2, d3);
-            float w0 = e0, w1 = e1, w2 = e2, w3 = e3;
-            if (BR) {
-              unpack2(mul2(pack2(e0, e1), g01), w0, w1);
-              unpack2(mul2(pack2(e2, e3), g23), w2, w3);
-            }
-            pp[i >> 1] = pack2<F16>(w0, w1);
-            pp[(i >> 1) + 1] = pack2<F16>(w2, w3);
+            pp[i >> 1] = pack2<F16>(e0, e1);
+            pp[(i >> 1) + 1] = pack2<F16>(e2, e3);
             ds[i >> 1] = pack2<F16>(d0, d1);
             ds[(i >> 1) + 1] = pack2<F16>(d2, d3);
           }
@@ -591,13 +568,12 @@ static int launch_dkdv_tc_t(const HostCtx& c, const void* q, const void* k, cons
                    const RowStats& st, const int32_t* csr_off, const int32_t* csr_q, void* dk,
                    void* dv, int* work_counter, int32_t* order) {
   const Geo& g = c.g;
-  CUtensorMap mq, mdo, mk, mv, mnl, mnd, mgt;
+  CUtensorMap mq, mdo, mk, mv, mnl, mnd;
   const int planes = BR ? 2 : 1;
-  if (!make_map(&mq, q, g, g.U) || !make_map(&mdo, d_o, g, g.U) || !make_map(&mk, k, g, g.Ukv) || !make_map(&mv, v, g, g.Ukv) ||
-      !make_map_rows(&mnl, st.neg_lse2, g, planes * g.U) || !make_map_rows(&mnd, st.neg_d, g, planes * g.U) ||
-      !make_map_rows(&mgt, BR ? st.gate : st.neg_d, g, planes * g.U))
+  if (!make_map(&mq, q, g, g.U) || !make_map(&mdo, BR ? st.gated_do : d_o, g, planes * g.U) || !make_map(&mk, k, g, g.Ukv) || !make_map(&mv, v, g, g.Ukv) ||
+      !make_map_rows(&mnl, st.neg_lse2, g, planes * g.U) || !make_map_rows(&mnd, st.neg_d, g, planes * g.U))
     return MOSAIC_E_CUDA;
-  const size_t smem = sizeof(Smem<BR>) + 1024;
+  const size_t smem = sizeof(Smem) + 1024;
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
   int sms = 0;
   if (const int rc = launch_setup(reinterpret_cast<const void*>(dkdv_tc_kernel<F16, BR>), smem, &configured, &sms)) return rc;
@@ -616,7 +592,7 @@ static int launch_dkdv_tc_t(const HostCtx& c, const void* q, const void* k, cons
       g, csr_off, ipu, (int)total, (int)win_items, order, order + total);
   if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
   dkdv_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
-      g, mq, mdo, mk, mv, mnl, mnd, mgt, csr_off, csr_q, order, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, st.dkm, st.dvm,
+      g, mq, mdo, mk, mv, mnl, mnd, csr_off, csr_q, order, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, st.dkm, st.dvm,
       c.status, work_counter, ipu, (int)total);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }

@@ -12,7 +12,7 @@
 // the tensor-core work; two groups of four warps (thread = query row = TMEM lane) turn S and dP into dS.
 // Per product and tile: S = Q K^T and dP = dO V^T (eight MMAs into two 64-column TMEM buffers); the row
 // threads pull both into registers and hand the buffers back at once, so the next product's S and dP are
-// computed while they form dS (bf16, its own 32 TMEM columns); then dQ += dS K (dS is the TMEM A operand,
+// computed while they form dS (bf16, two buffers of 32 TMEM columns in turn); then dQ += dS K (dS is the TMEM A operand,
 // the K chunk in shared memory is read as the MN-major B operand), issued one product behind.
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
 #include "tc_common.cuh"
@@ -24,7 +24,7 @@ namespace {
 constexpr int kStages = 6;       // key/value ring depth (K + V chunk per stage)
 constexpr int kThreads = 384;
 constexpr uint32_t kTmemCols = 512;
-// dQ of tile t at 64 t; S of tile t at 128 + 128 t, dP right after it; dS (bf16) of tile t at 384 + 32 t
+// dQ of tile t at 64 t; S of tile t at 128 + 128 t, dP right after it; dS buffer b (bf16) of tile t at 384 + 64 t + 32 b
 constexpr uint32_t kColDQ = 0, kColS = 128, kColDS = 384;
 
 struct Smem {
@@ -32,7 +32,8 @@ struct Smem {
   unsigned char d_o[2][2 * kTile];         // [tile][128 rows x 128 B]
   unsigned char kv[kStages][2][kTile];     // [stage][K, V]
   unsigned long long kv_full[kStages], kv_empty[kStages];
-  unsigned long long q_full[2], q_empty[2], s_full[2], sdp_free[2], p_full[2], pv_done[2];  // [tile]
+  unsigned long long q_full[2], q_empty[2], s_full[2], sdp_free[2];  // [tile]
+  unsigned long long p_full[2][2], pv_done[2][2];  // [tile][dS buffer]
   unsigned long long mma_drain_bar[2];  // abort path: completion of each issuer's outstanding products
   unsigned long long list_full[kLists], list_empty[kLists];
   uint32_t tmem_base;
@@ -68,8 +69,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(s32(&sm.mma_drain_bar[t]), 1);
       mbar_init(s32(&sm.s_full[t]), 1);
       mbar_init(s32(&sm.sdp_free[t]), 128);
-      mbar_init(s32(&sm.p_full[t]), 128);
-      mbar_init(s32(&sm.pv_done[t]), 1);
+      mbar_init(s32(&sm.p_full[t][0]), 128);
+      mbar_init(s32(&sm.p_full[t][1]), 128);
+      mbar_init(s32(&sm.pv_done[t][0]), 1);
+      mbar_init(s32(&sm.pv_done[t][1]), 1);
     }
     for (int i = 0; i < kLists; ++i) {
       mbar_init(s32(&sm.list_full[i]), 1);
@@ -146,22 +149,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t idesc_nt = make_idesc(false, 64u, F16), idesc_nn = make_idesc(true, 64u, F16);
     const uint64_t qdesc = smem_desc(s32(sm.q[t])), dodesc = smem_desc(s32(sm.d_o[t]));
     const uint32_t tcol_dq = tmem + kColDQ + 64 * t, tcol_s = tmem + kColS + 128 * t, tcol_dp = tcol_s + 64;
-    const uint32_t tcol_ds = tmem + kColDS + 32 * t;
+    const uint32_t tcol_ds = tmem + kColDS + 64 * t;
     uint32_t base = 0;    // ring position of the item's first chunk
     uint32_t nt = 0;      // products started by this tile so far (phase of the per-product barriers)
     bool ok = true;
     // dQ += dS K of the product whose K chunk sits in ring stage `pst` (the previous product of this tile)
     auto issue_dq = [&](int pst, bool pfirst) {
-      ok = warp_wait(s32(&sm.p_full[t]), (nt - 1) & 1, abort, status);
+      ok = warp_wait(s32(&sm.p_full[t][(nt - 1) & 1]), ((nt - 1) >> 1) & 1, abort, status);
       if (!ok) return;
       tc_fence_after();
       const uint64_t kmn = smem_desc(s32(sm.kv[pst][0]));
+      const uint32_t dscol = tcol_ds + 32 * ((nt - 1) & 1);
       if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          umma_ts(tcol_dq, tcol_ds + 8 * kk, kmn + (uint64_t)((2048 * kk) >> 4), idesc_nn, (!pfirst || kk > 0));
+          umma_ts(tcol_dq, dscol + 8 * kk, kmn + (uint64_t)((2048 * kk) >> 4), idesc_nn, (!pfirst || kk > 0));
         tc_commit(s32(&sm.kv_empty[pst]));
-        tc_commit(s32(&sm.pv_done[t]));
+        tc_commit(s32(&sm.pv_done[t][(nt - 1) & 1]));
       }
       __syncwarp();
     };
@@ -230,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int h = 2 * t + hh;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t ts = tmem + lane_off + kColS + 128 * t, tdp = ts + 64, tdq = tmem + lane_off + kColDQ + 64 * t;
-    const uint32_t tds = tmem + lane_off + kColDS + 32 * t;
+    const uint32_t tds = tmem + lane_off + kColDS + 64 * t;
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
     uint32_t nt = 0;
     bool ok = true;
@@ -295,22 +299,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int i = 0; i < 32; ++i) pk[i] = 0u;
           }
-          // dS has one buffer: the previous product's dQ += dS K must have consumed it
-          if (i0 + c > 0) {
-            ok = warp_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
-            if (!ok) break;
-            tc_fence_after();
-          }
-          tmem_st32(tds, pk);
+          // dS buffer nt & 1 was read by dQ += dS K of product nt - 2, issued before this product's S by the same warp, whose
+          // commit for S therefore covers it: no wait
+          tmem_st32(tds + 32 * (nt & 1), pk);
           tmem_wait_st();
           tc_fence_before();
-          mbar_arrive(s32(&sm.p_full[t]));
+          mbar_arrive(s32(&sm.p_full[t][nt & 1]));
           ++nt;
         }
       }
       if (!ok) break;
       if (cnt > 0) {
-        ok = warp_wait(s32(&sm.pv_done[t]), (nt - 1) & 1, abort, status);
+        ok = warp_wait(s32(&sm.pv_done[t][(nt - 1) & 1]), ((nt - 1) >> 1) & 1, abort, status);
         if (!ok) break;
         tc_fence_after();
         if (valid) {

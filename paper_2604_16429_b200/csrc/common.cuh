@@ -119,7 +119,7 @@ int launch_select(const HostCtx& c, const void* q, const void* k, int32_t* block
 // What the attention kernel computes: kFwdUnion one softmax over local and selected blocks (o, lse); kFwdBranches the
 // gated sum of the three branches (o, lse of the selection branch, lse_l of the local one; reads gates and the block-level
 // output ocg); kFwdStats only what the three-branch backward needs of the forward: the gate gradients and, in two planes
-// of [U, N] (local, selected), the negated base-2 log-sum-exp, -gate * <dO, O> and the gate.
+// of [U, N] (local, selected), the negated base-2 log-sum-exp, -gate * <dO, O>, the gate and gate * dO.
 enum { kFwdUnion = 0, kFwdBranches = 1, kFwdStats = 2 };
 struct FwdOut {
   __nv_bfloat16* o;
@@ -127,6 +127,7 @@ struct FwdOut {
   const float *gates, *ocg;
   const __nv_bfloat16* d_o;
   float *dgates, *neg_lse2, *neg_d, *gate;
+  void* gated_do;
 };
 int launch_fwd_tc(const HostCtx& c, int mode, const void* q, const void* k, const void* v, const int32_t* block_idx,
                   const FwdOut& out, int* work_counter);
@@ -161,9 +162,10 @@ int launch_compress_bwd(const HostCtx& c, const CompressBwd& a);
 int launch_rope(const HostCtx& c, const void* q, const void* k, const float* pos, double theta, void* q_out, void* k_out);
 // What the attention backward reads per query row, [U, N] fp32: the negated base-2 log-sum-exp and -<dO, O>.  Three-branch
 // form (gate set): two planes of each (local blocks, selected blocks), the second of them scaled by the gate, the gates
-// themselves, and what the compression branch gives every token of a block: dqm [U, m, d], dkm, dvm [Ukv, m, d].
+// themselves, dO scaled by each gate ([U, N, d] 16-bit, two planes), and what the compression branch gives every token of a block: dqm [U, m, d], dkm, dvm [Ukv, m, d].
 struct RowStats {
   const float *neg_lse2, *neg_d, *gate, *dqm, *dkm, *dvm;
+  const void* gated_do;
 };
 int launch_rowdot(const HostCtx& c, const void* o, const void* d_o, const float* lse, float* neg_d, float* neg_lse2);
 int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,

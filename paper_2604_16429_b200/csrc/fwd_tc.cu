@@ -96,13 +96,15 @@ __device__ __forceinline__ void store_row(uint4* dst, const uint32_t* a, float f
     dst[x] = make_uint4(pack2<F16>(v[0], v[1]), pack2<F16>(v[2], v[3]), pack2<F16>(v[4], v[5]), pack2<F16>(v[6], v[7]));
   }
 }
-// 32 channels of <dO, O> and of <dO, block-level vector>
+// 32 channels of <dO, O> and of <dO, block-level vector>; gate * dO is stored
 template <bool F16>
-__device__ __forceinline__ void dot_row(const uint4* d_o, const uint32_t* a, const float* cg, float& dot, float& dotc) {
+__device__ __forceinline__ void dot_row(const uint4* d_o, const uint32_t* a, const float* cg, float gate, uint4* gated, float& dot,
+                                        float& dotc) {
 #pragma unroll
   for (int x = 0; x < 4; ++x) {
     const uint4 w = __ldg(d_o + x);
     const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+    uint32_t gw[4];
     const float4 c0 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x), c1 = __ldg(reinterpret_cast<const float4*>(cg) + 2 * x + 1);
     const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
@@ -111,7 +113,9 @@ __device__ __forceinline__ void dot_row(const uint4* d_o, const uint32_t* a, con
       unpack16x2(ww[y], F16, lo, hi);
       dot = fmaf(lo, __uint_as_float(a[8 * x + 2 * y]), fmaf(hi, __uint_as_float(a[8 * x + 2 * y + 1]), dot));
       dotc = fmaf(lo, cv[2 * y], fmaf(hi, cv[2 * y + 1], dotc));
+      gw[y] = pack2<F16>(gate * lo, gate * hi);
     }
+    gated[x] = make_uint4(gw[0], gw[1], gw[2], gw[3]);
   }
 }
 
@@ -457,6 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float gx = MODE == kFwdUnion ? 1.f : __ldg(out.gates + 3 * tok + 1 + branch);
         const float gc = MODE == kFwdBranches && branch ? __ldg(out.gates + 3 * tok) : 0.f;
         float dot = 0.f, dotc = 0.f;
+        const long long at = (branch ? 0 : (long long)g.U * g.N) + tok;  // statistics: plane 0 local, plane 1 selected
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
           uint32_t ov[32];
@@ -468,7 +473,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int x = 0; x < 32; ++x) ov[x] = 0u;
           }
           if (MODE == kFwdStats)
-            dot_row<F16>(reinterpret_cast<const uint4*>(out.d_o + tok * kD) + 4 * part, ov, cg + 32 * part, dot, dotc);
+            dot_row<F16>(reinterpret_cast<const uint4*>(out.d_o + tok * kD) + 4 * part, ov, cg + 32 * part, gx,
+                         static_cast<uint4*>(out.gated_do) + at * 8 + 4 * part, dot, dotc);
           else
             store_row<F16>(reinterpret_cast<uint4*>(out.o + tok * kD) + 4 * part, ov, inv * gx,
                            MODE == kFwdBranches && branch == 1, gc, cg + 32 * part);
@@ -481,7 +487,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           dot *= inv;
           out.dgates[3 * tok + 1 + branch] = dot;
           if (branch) out.dgates[3 * tok] = dotc;
-          const long long at = (branch ? 0 : (long long)g.U * g.N) + tok;  // plane 0: local, plane 1: selected
           out.neg_lse2[at] = -lse2;
           out.neg_d[at] = -gx * dot;
           out.gate[at] = gx;
