@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     dq_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                  const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const int32_t* __restrict__ block_idx, const RowStats st, __nv_bfloat16* __restrict__ dq, int* status,
-                 int* work_counter, int ipu, int total_items) {
+                 int* work_counter, int ipu, const Queue queue) {
   extern __shared__ unsigned char smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort = &sm.abort;
 
   if (warp == 11) {
-    planner_loop<BR ? kPlanTagged : kPlanUnion>(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
+    planner_loop<BR ? kPlanTagged : kPlanUnion>(sm, g, block_idx, work_counter, ipu, queue, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -362,9 +362,10 @@ static int launch_dq_tc_t(const HostCtx& c, const void* q, const void* k, const 
   const int ipu = items_per_unit(g);
   const long long total = (long long)g.U * ipu;
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
-  const long long grid = total < (long long)sms ? total : (long long)sms;
+  const Queue queue = make_queue(total, sms);
+  const int grid = queue.positions < sms ? queue.positions : sms;
   dq_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
-      g, mq, mdo, mk, mv, block_idx, st, (__nv_bfloat16*)dq, c.status, work_counter, ipu, (int)total);
+      g, mq, mdo, mk, mv, block_idx, st, (__nv_bfloat16*)dq, c.status, work_counter, ipu, queue);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 

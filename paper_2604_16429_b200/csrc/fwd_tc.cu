@@ -125,7 +125,7 @@ template <bool F16, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_tc_kernel(const Geo g, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ block_idx,
-                  const __grid_constant__ FwdOut out, int* status, int* work_counter, int ipu, int total_items) {
+                  const __grid_constant__ FwdOut out, int* status, int* work_counter, int ipu, const Queue queue) {
   extern __shared__ unsigned char smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort = &sm.abort;
 
   if (warp == 11) {
-    planner_loop<MODE == kFwdUnion ? kPlanUnion : kPlanSplit>(sm, g, block_idx, work_counter, ipu, total_items, lane, abort, status);
+    planner_loop<MODE == kFwdUnion ? kPlanUnion : kPlanSplit>(sm, g, block_idx, work_counter, ipu, queue, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -514,9 +514,10 @@ int launch_fwd_tc_t(const HostCtx& c, const CUtensorMap& mq, const CUtensorMap& 
   const int ipu = items_per_unit(g);
   const long long total = (long long)g.U * ipu;
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
-  const long long grid = total < (long long)sms ? total : (long long)sms;
+  const Queue queue = make_queue(total, sms);
+  const int grid = queue.positions < sms ? queue.positions : sms;
   fwd_tc_kernel<F16, MODE><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mk, mv, block_idx, out, c.status,
-                                                                        work_counter, ipu, (int)total);
+                                                                        work_counter, ipu, queue);
   return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
 }
 }  // namespace
