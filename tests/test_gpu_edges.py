@@ -1,0 +1,185 @@
+"""GPU parity at the edges of the kernels' tiles and of their launch rules, against the oracle, through the C ABI: the
+sizes on both sides of every line at which a kernel changes its width, its split or its work queue.  Tolerances are those
+of the full tests: ids and rotated values exact (one 16-bit step at rounding ties), outputs and gradients the bounds of
+the shared helpers."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2604_16429_b200 import binding as mb
+from paper_2604_16429_b200 import synth
+from tests import gpu_util as G
+from tests import test_gpu_rope as R
+from tests import test_gpu_three_branch as T
+
+pytestmark = pytest.mark.gpu
+
+
+def _name(w):
+    return f"m{w.m}_k{w.topk}_U{w.U}" if hasattr(w, "m") else str(w)
+
+
+# Ranking: 16 query blocks per CTA, 32 from 296 CTAs of 32 on (148 units of 33 blocks), 64 keys per chunk; room for 96
+# survivors per row, 192 beyond top-k 16.  Pooling: 2, 4 or 8 channels per lane from 75000 / 16 and 75000 / 8 pooled
+# blocks on (Q and K together).
+RANK = [synth.small_case(8 * a, 8 * b, 8, 8, k, H=h, seed=300 + i) for i, (a, b, k, h) in enumerate([
+    (3, 5, 16, 1), (4, 4, 4, 2), (17, 1, 17, 1), (3, 21, 16, 1), (8, 8, 17, 1), (5, 13, 32, 2), (3, 43, 31, 1),
+    (3, 11, 16, 147), (3, 11, 16, 148), (3, 11, 17, 148), (3, 11, 32, 71), (1, 11, 8, 213), (1, 11, 8, 214), (1, 11, 8, 426),
+    (1, 11, 8, 427)])] + [synth.small_case(24, 176, 8, 16, 5, H=h, seed=320 + h) for h in (1, 100, 148)]
+
+
+@pytest.mark.parametrize("w", RANK, ids=_name)
+def test_ranking_and_pooling_at_tile_and_rule_edges(w):
+    x = synth.make_inputs(w)
+    got = G.gpu_select(w, G.device_inputs(x)).cpu().numpy()
+    want = G.oracle_select_all(w, x)
+    assert np.array_equal(got, want), f"{(got != want).sum()} of {want.size} ids differ"
+
+
+# Work queue of the row-stationary kernels on 148 SMs: the items left over after full waves are cut into four parts up to
+# 37 of them, into two up to 74; none are cut after one to three full waves.  One item per unit here (2 x 2 blocks, and
+# three blocks in a row, whose fourth part is empty).
+QUEUE = [(16, 16, h) for h in (1, 37, 38, 74, 75, 148, 149, 593, 630)] + [(8, 24, h) for h in (1, 38, 75, 594, 631)]
+
+
+@pytest.mark.parametrize("nlat,nlon,heads", QUEUE)
+def test_left_over_items_in_parts(nlat, nlon, heads):
+    w = synth.small_case(nlat, nlon, 8, 8, 2, H=heads, seed=340 + heads, rlat=0, rlon=0, backward=True)
+    x = synth.make_inputs(w)
+    dx = G.device_inputs(x)
+    idx = G.gpu_select(w, dx)
+    o, lse = G.gpu_fwd(w, dx, idx)
+    grads = G.gpu_bwd(w, dx, o, lse, idx)
+    gates = np.random.default_rng(heads).standard_normal((1, heads, w.N, 3))
+    three = T._run(w, x, idx, gates)
+    assert all(bool(torch.isfinite(t.float()).all()) for t in (o, lse, *grads)) and np.isfinite(three[0]).all()
+    idx_h = idx.cpu().numpy()
+    units = range(heads) if heads <= 12 else [0, 1, heads // 2, *range(heads - 4, heads)]
+    for h in units:
+        G.compare_fwd_unit(w, x, 0, h, idx_h[0, h], o, lse)
+        ref = oracle.bwd(G.geom_of(w), x["q"][0, h], x["k"][0, h], x["v"][0, h], x["do"][0, h], idx_h[0, h])
+        for name, got, want in zip(("dQ", "dK", "dV"), grads, ref):
+            G.assert_bwd_close(f"{name} unit {h}", got[0, h], want)
+    _compare3_units(w, x, idx_h, gates, three, units, T._compare)
+
+
+def _compare3_units(w, x, idx_h, gates, got, units, compare):
+    """A three-branch comparison of some units only (one key/value head per query head)."""
+    one = dataclasses.replace(w, H=1, Hkv=0)
+    for h in units:
+        s = slice(h, h + 1)
+        compare(one, {k: v[:, s] for k, v in x.items()}, idx_h[:, s], gates[:, s], [t[:, s] for t in got])
+
+
+# Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2, 4 or 8 CTAs (as many as
+# give every SM two, at most one per chunk; on the key side the chunks of all query heads of a group count).
+COMPRESS = [synth.small_case(8 * m, 8, 8, 8, 2, H=h, Hkv=kv, seed=360 + i, backward=True) for i, (m, h, kv) in enumerate([
+    (63, 1, 0), (64, 1, 0), (65, 1, 0), (129, 1, 0), (193, 1, 0), (449, 1, 0), (65, 4, 1), (65, 6, 2)])]
+
+
+@pytest.mark.parametrize("w", COMPRESS, ids=_name)
+def test_block_level_tiles_and_cluster_sizes(w):
+    x = synth.make_inputs(w)
+    idx = G.gpu_select(w, G.device_inputs(x))
+    gates = np.random.default_rng(w.cfg).standard_normal((w.B, w.H, w.N, 3))
+    if not w.Hkv:
+        T._compare(w, x, idx.cpu().numpy(), gates, T._run(w, x, idx, gates))
+    T._compare_bwd3(w, x, idx.cpu().numpy(), gates, T._run_bwd3(w, x, idx, gates))
+
+
+@pytest.mark.parametrize("heads", [16, 40, 148])
+def test_block_level_many_units(heads):
+    """Gated pooling with 2, 4 and 8 channels per lane (4 * heads * 65 pooled blocks), and with 148 units a block level
+    that needs no clusters."""
+    w = synth.small_case(40, 104, 8, 8, 3, H=heads, seed=380 + heads, backward=True)
+    x = synth.make_inputs(w)
+    idx = G.gpu_select(w, G.device_inputs(x))
+    gates = np.random.default_rng(w.cfg).standard_normal((w.B, w.H, w.N, 3))
+    got = T._run_bwd3(w, x, idx, gates)
+    assert all(np.isfinite(t).all() for t in got)
+    _compare3_units(w, x, idx.cpu().numpy(), gates, got, (0, heads - 1), T._compare_bwd3)
+
+
+@pytest.mark.parametrize("topk", [1, 3, 7, 17, 32])
+def test_transposed_lists_for_any_topk(topk):
+    """A warp of the transposed-pattern kernel takes 32 / topk rows at a time; rows of repeated, local and absent ids."""
+    w = synth.small_case(40, 56, 8, 8, topk, H=1, seed=400 + topk, backward=True)
+    x = synth.make_inputs(w)
+    dx = G.device_inputs(x)
+    idx = G.gpu_select(w, dx)
+    idx[0, 0, 9, :] = -1
+    clean = idx.clone()
+    if topk > 2:                                            # the oracle gets the rows without the ids that are to be skipped
+        idx[0, 0, 12, 1] = idx[0, 0, 12, 0]                 # a repeat
+        idx[0, 0, 13, 2] = 13                               # the block itself, local already
+        clean[0, 0, 12, 1] = clean[0, 0, 13, 2] = -1
+    idx_h = clean.cpu().numpy()
+    p = mb.Params.from_workload(w)
+    ws = mb.alloc_workspace(p, mb.OP_FWD)
+    o, lse = mb.mosaic_bsa_fwd(p, dx["q"], dx["k"], dx["v"], idx, ws=ws)
+    ws = mb.alloc_workspace(p, mb.OP_BWD)
+    grads = mb.mosaic_bsa_bwd(p, dx["q"], dx["k"], dx["v"], o, lse, dx["do"], idx, ws=ws)
+    ref = oracle.bwd(G.geom_of(w), x["q"][0, 0], x["k"][0, 0], x["v"][0, 0], x["do"][0, 0], idx_h[0, 0])
+    for name, got, want in zip(("dQ", "dK", "dV"), grads, ref):
+        G.assert_bwd_close(name, got[0, 0], want)
+
+
+@pytest.mark.parametrize("bh,bw,nlat,nlon", [(8, 8, 64, 64), (8, 16, 64, 128)])
+def test_a_tile_that_skips_most_of_its_items_list(bh, bw, nlat, nlon):
+    """The two tiles of an item walk their own entries of the merged list; here a tile attends only the first and the last
+    of 60 blocks that the other one attends in between, many more than the key ring holds."""
+    w = synth.small_case(nlat, nlon, bh, bw, 30, H=1, seed=420 + bw, rlat=0, rlon=0, backward=True)
+    x = synth.make_inputs(w)
+    dx = G.device_inputs(x)
+    nbw = nlon // bw
+    idx_h = np.full((1, 1, w.m, 30), -1, np.int32)
+    for y in range(0, nlat // bh, 2):
+        for c in range(0, nbw, 2):
+            far = [j for j in range(w.m) if j not in (y * nbw + c, y * nbw + c + 1, (y + 1) * nbw + c, (y + 1) * nbw + c + 1)]
+            idx_h[0, 0, y * nbw + c] = far[:30]
+            idx_h[0, 0, y * nbw + c + 1] = far[30:60]
+            idx_h[0, 0, (y + 1) * nbw + c, :2] = [far[0], far[59]]
+            idx_h[0, 0, (y + 1) * nbw + c + 1, :1] = [far[59]]
+    idx_h[0, 0, -1, :] = -1
+    idx = torch.from_numpy(idx_h).cuda()
+    o, lse = G.gpu_fwd(w, dx, idx)
+    G.compare_fwd_unit(w, x, 0, 0, idx_h[0, 0], o, lse)
+    grads = G.gpu_bwd(w, dx, o, lse, idx)
+    ref = oracle.bwd(G.geom_of(w), x["q"][0, 0], x["k"][0, 0], x["v"][0, 0], x["do"][0, 0], idx_h[0, 0])
+    for name, got, want in zip(("dQ", "dK", "dV"), grads, ref):
+        G.assert_bwd_close(name, got[0, 0], want)
+    gates = np.random.default_rng(w.cfg).standard_normal((1, 1, w.N, 3))
+    T._compare(w, x, idx_h, gates, T._run(w, x, idx, gates))
+    T._compare_bwd3(w, x, idx_h, gates, T._run_bwd3(w, x, idx, gates))
+
+
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("heads,kv", [(1, 1), (6, 1), (7, 1), (6, 6), (24, 1), (15, 15)])
+def test_rope_unit_shares_and_non_finite_values(heads, kv, f16):
+    """Short sequences split the units over blocks from eight units on (shares that end inside Q's or K's units, or run
+    over their border); infinities and NaNs take the plain conversion, subnormals and zeros the exact scaled one."""
+    w = synth.small_case(24, 40, 8, 8, 2, H=heads, Hkv=kv, seed=440 + heads, f16=f16)
+    x = synth.make_inputs(w)
+    inf = 0x7C00 if f16 else 0x7F80
+    for a in (x["q"], x["k"]):
+        a[0, :, 5, :8] = [inf, inf | 0x8000, inf | 1, 0, 0x8000, 1, 0x8001, inf - 1]
+    pos = R._positions(w, np.random.default_rng(w.cfg))
+    p = mb.Params.from_workload(w)
+    dx = G.device_inputs(x, f16=f16)
+    out = mb.mosaic_bsa_rope(p, dx["q"], dx["k"], torch.from_numpy(pos).cuda())
+    g = G.geom_of(w)
+    total = same = 0
+    for got, src in zip(out, (x["q"], x["k"])):
+        bits = got.view(torch.int16).cpu().numpy().view(np.uint16)
+        for h in range(src.shape[1]):
+            _, want = oracle.rope(g, src[0, h], pos.astype(np.float64))
+            nan = (want & 0x7FFF) > inf
+            assert np.array_equal(nan, (bits[0, h] & 0x7FFF) > inf)
+            dist = np.abs(R._ordered(bits[0, h]) - R._ordered(want))[~nan]
+            assert dist.max() <= 1
+            total += dist.size
+            same += int((dist == 0).sum())
+    assert same >= 0.9999 * total
