@@ -144,8 +144,7 @@ int mosaic_bsa_fwd(const mosaic_bsa_params *p, const void *q, const void *k, con
  *   gates      in   [B,H,N,3] fp32, order (compression, selection, local)
  *   o          out  [B,H,N,d] bf16
  *   lse_fg, lse_l  out  [B,H,N] fp32, natural-log sum-exp of the selection and local branches
- * Workspace: mosaic_bsa_workspace_bytes(p, MOSAIC_OP_FWD_BRANCHES) (pooled sums, the block-level output
- * and the two branch outputs in bf16).
+ * Workspace: mosaic_bsa_workspace_bytes(p, MOSAIC_OP_FWD_BRANCHES) (pooled sums and the block-level output).
  */
 int mosaic_bsa_fwd_branches(const mosaic_bsa_params *p, const void *q, const void *k, const void *v,
                             const int32_t *block_idx, const float *gates, void *o, float *lse_fg,
@@ -176,7 +175,7 @@ int mosaic_bsa_bwd(const mosaic_bsa_params *p, const void *q, const void *k, con
  *   d_o              in   [B,H,N,d] bf16, gradient of the forward's o
  *   dq               out  [B,H,N,d] bf16;  dk, dv out [B,Hkv,N,d] bf16
  *   dgates           out  [B,H,N,3] fp32, dgates[l][x] = <d_o_l, branch output x of token l>
- * Workspace: mosaic_bsa_workspace_bytes(p, MOSAIC_OP_BWD_BRANCHES) (about ten tensors of the size of q).
+ * Workspace: mosaic_bsa_workspace_bytes(p, MOSAIC_OP_BWD_BRANCHES) (about three tensors of the size of q).
  * Results are deterministic.  Errors as for mosaic_bsa_bwd.
  */
 int mosaic_bsa_bwd_branches(const mosaic_bsa_params *p, const void *q, const void *k, const void *v,

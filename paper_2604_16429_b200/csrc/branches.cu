@@ -15,6 +15,9 @@
 // owns 64 stationary blocks of one unit and streams the other side in chunks of 64; a thread computes a 4 x 4 tile of a
 // 64 x 64 product from shared memory.  The chunks of a tile are split over a cluster of up to 8 CTAs, which add their partial sums over
 // distributed shared memory in rank order, so results do not depend on timing.
+// Bound by shared-memory operand loads (2 reads of 4 words per 16 FMAs) and, for few tiles, by the length of a stream.  us,
+// before -> after: forward of 8 units of 450 blocks twice 77 -> 53, backward of both sides 110 -> 81; backward of 12 units of
+// 384 blocks 212 -> 92; of 20 units of 24 blocks 27 -> 16.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -96,7 +99,7 @@ __global__ void __launch_bounds__(kThr) compress_kernel(Geo g, const float* __re
   const cgs::cluster_group cluster = cgs::this_cluster();
   const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int tiles = (g.m + kT - 1) / kT, tile = (int)blockIdx.x / ranks;
+  const int tiles = (g.m + kT - 1) / kT, tile = (int)blockIdx.x / ranks + await_stream();
   const int u = tile / tiles, i0 = (tile - u * tiles) * kT;
   const float* pk_u = pk + (long long)kv_unit(g, u) * g.m * kD;   // grouped-query attention: the group's key/value head
   const float* pv_u = pv + (long long)kv_unit(g, u) * g.m * kD;
@@ -295,8 +298,9 @@ __global__ void __launch_bounds__(kThr) compress_bwd_kernel(Geo g, const Compres
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& sm = *reinterpret_cast<BwdSmem*>(smem_raw);
   const int ranks = (int)cgs::this_cluster().num_blocks();
-  if ((int)blockIdx.x < query_ctas) compress_bwd_tile<false>(g, sm, (int)blockIdx.x / ranks, a);
-  else compress_bwd_tile<true>(g, sm, ((int)blockIdx.x - query_ctas) / ranks, a);
+  const int cta = (int)blockIdx.x + await_stream();
+  if (cta < query_ctas) compress_bwd_tile<false>(g, sm, cta / ranks, a);
+  else compress_bwd_tile<true>(g, sm, (cta - query_ctas) / ranks, a);
 }
 
 // CTAs per tile: enough of them that every SM gets about two, at most one per chunk (and 8, the portable cluster size)
@@ -312,18 +316,7 @@ int launch_clustered(const HostCtx& c, Kernel kernel, size_t smem, unsigned long
   int sms = 0;
   if (const int rc = launch_setup(reinterpret_cast<const void*>(kernel), smem, configured, &sms)) return rc;
   if (ctas > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)ctas);
-  cfg.blockDim = dim3(kThr);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = c.stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cluster;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(kernel, dim3((unsigned)ctas), kThr, smem, c.stream, false, cluster, args...);
 }
 
 }  // namespace

@@ -26,8 +26,9 @@ __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uin
                                                      const uint4* __restrict__ d_o, const float* __restrict__ lse,
                                                      float* __restrict__ neg_d, float* __restrict__ neg_lse2, bool f16,
                                                      int* status) {
-  if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0;  // the op's first kernel
-  long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int tid = (int)threadIdx.x + await_stream();
+  if (blockIdx.x == 0 && tid < kStatusBytes / 4) status[tid] = 0;  // the op's first kernel
+  long long t = ((long long)blockIdx.x * blockDim.x + tid) >> 3;
   int part = threadIdx.x & 7;
   float acc = 0.f;
   if (t < tokens) {
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(256) rowdot_kernel(long long tokens, const uin
 //      fixes the dK/dV summation order).
 // Shared memory: (nseg + 1) * m counters + m * topk bits.
 // ------------------------------------------------------------------------------------------
-// Latency-bound (one CTA per unit): with a thread per row and eight segments 9216 entries took 66 us.
+// Latency-bound (one CTA per unit): with a thread per row and eight segments 9216 entries took 66 us, now 43.
 constexpr int kCsrThreads = 512;
 __global__ void __launch_bounds__(kCsrThreads) csr_kernel(Geo g, const int32_t* __restrict__ block_idx,
                                                   int32_t* __restrict__ csr_off, int32_t* __restrict__ csr_q, int nseg) {
@@ -71,13 +72,14 @@ __global__ void __launch_bounds__(kCsrThreads) csr_kernel(Geo g, const int32_t* 
   int* tot = csr_sm;                        // [m] list lengths, then list starts
   int* seg = csr_sm + g.m;                  // [nseg][m] counts, then cursors
   unsigned* bits = reinterpret_cast<unsigned*>(seg + (long long)nseg * g.m);  // [ceil(m * topk / 32)] valid entries
-  const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int32_t* idx = block_idx + (long long)u * g.m * g.topk;
-  int32_t* off = csr_off + (long long)u * (g.m + 1);
-  int32_t* outq = csr_q + (long long)u * g.m * g.topk;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int E = g.m * g.topk, rps = (g.m + nseg - 1) / nseg;  // rows per segment
   for (int x = tid; x < (nseg + 1) * g.m; x += blockDim.x) csr_sm[x] = 0;
   for (int x = tid; x < (E + 31) / 32; x += blockDim.x) bits[x] = 0u;
+  const int u = (int)blockIdx.x + await_stream();
+  const int32_t* idx = block_idx + (long long)u * g.m * g.topk;
+  int32_t* off = csr_off + (long long)u * (g.m + 1);
+  int32_t* outq = csr_q + (long long)u * g.m * g.topk;
   __syncthreads();
   int lanes = 1;  // lanes of a row: the power of two that holds topk
   while (lanes < g.topk) lanes *= 2;
@@ -166,9 +168,8 @@ static int csr_segments(const Geo& g, size_t* smem) {
 
 int launch_rowdot(const HostCtx& c, const void* o, const void* d_o, const float* lse, float* neg_d, float* neg_lse2) {
   const long long tokens = (long long)c.g.U * c.g.N, threads = tokens * 8;
-  rowdot_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c.stream>>>(tokens, (const uint4*)o, (const uint4*)d_o, lse,
-                                                                         neg_d, neg_lse2, c.g.f16 != 0, c.status);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(rowdot_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, c.stream, true, 0, tokens, (const uint4*)o,
+                       (const uint4*)d_o, lse, neg_d, neg_lse2, c.g.f16 != 0, c.status);
 }
 
 int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, const RowStats& st, const void* d_o,
@@ -187,12 +188,13 @@ int launch_bwd(const HostCtx& c, const void* q, const void* k, const void* v, co
         return MOSAIC_E_CUDA;
       configured |= 1ull << dev;
     }
-    csr_kernel<<<g.U, kCsrThreads, smem, c.stream>>>(g, block_idx, csr_off, csr_q, nseg);
+    if (const int rc = launch_kernel(csr_kernel, dim3((unsigned)g.U), kCsrThreads, smem, c.stream, true, 0, g, block_idx, csr_off,
+                                     csr_q, nseg))
+      return rc;
   } else {
     if (cudaMemsetAsync(csr_off, 0, sizeof(int32_t) * (size_t)g.U * (g.m + 1), c.stream) != cudaSuccess)
       return MOSAIC_E_CUDA;
   }
-  if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
   // the work queues count in words of the status block (zeroed when the op started)
   const int rc = launch_dq_tc(c, q, k, v, d_o, st, block_idx, dq, counters);
   if (rc) return rc;

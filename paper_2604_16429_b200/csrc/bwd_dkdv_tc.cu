@@ -22,6 +22,10 @@
 // halves they are connected to) and appends each block's CSR list; a list longer than a list buffer
 // continues in the next buffer (ItemInfo::more).  The order of a list is a function of the pattern alone,
 // so the summation order, and with it the result, is deterministic.
+// Bound like dQ by the row threads' instruction queue, about 2600 cycles per pair of products.  Issuers that walk their loops
+// as whole warps, no divisions and no wait on the ring in the row threads: 64 units of 28800 tokens 2405 -> 1802 us, 32 units
+// of 12288 tokens 743 -> 565.  One launch for both branches of the three-branch form, with dO scaled by either gate
+// beforehand: 12 units of 49152 tokens 1742 -> 1320.
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
 #include "tc_common.cuh"
 
@@ -173,6 +177,7 @@ __global__ void __launch_bounds__(1024) dkdv_order_kernel(const Geo g, const int
   const int first_item = (int)blockIdx.x * window_items;
   const int end_item = min(total_items, first_item + window_items);
   for (int i = tid; i < kCostBins; i += (int)blockDim.x) hist[i] = 0;
+  csr_off += await_stream();
   __syncthreads();
   const int ratio = g.H / g.Hkv;
   for (int item = first_item + tid; item < end_item; item += (int)blockDim.x) {
@@ -245,6 +250,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     sm.abort = 0;
     cta_publish_barriers();
   }
+  const int zero = await_stream();  // before the TMEM is taken: a kernel ahead may still need it
+  csr_off += zero;
+  csr_q += zero;
+  order += zero;
   const uint32_t tmem = cta_tmem_alloc(warp == kWMma0, &sm.tmem_base, kTmemCols);
   volatile int* abort = &sm.abort;
 
@@ -588,13 +597,12 @@ static int launch_dkdv_tc_t(const HostCtx& c, const void* q, const void* k, cons
   const long long min_units = (16ll * sms + 2 * ipu - 1) / (2 * ipu);
   if (win_units < min_units) win_units = min_units;
   const long long win_items = win_units * 2 * ipu;
-  dkdv_order_kernel<<<(unsigned)((total + win_items - 1) / win_items), 1024, 0, c.stream>>>(
-      g, csr_off, ipu, (int)total, (int)win_items, order, order + total);
-  if (cudaGetLastError() != cudaSuccess) return MOSAIC_E_CUDA;
-  dkdv_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
-      g, mq, mdo, mk, mv, mnl, mnd, csr_off, csr_q, order, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, st.dkm, st.dvm,
-      c.status, work_counter, ipu, (int)total);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  if (const int rc = launch_kernel(dkdv_order_kernel, dim3((unsigned)((total + win_items - 1) / win_items)), 1024, 0, c.stream,
+                                   true, 0, g, csr_off, ipu, (int)total, (int)win_items, order, order + total))
+    return rc;
+  return launch_kernel(dkdv_tc_kernel<F16, BR>, dim3((unsigned)grid), kThreads, smem, c.stream, true, 0, g, mq, mdo, mk, mv, mnl, mnd,
+                       csr_off, csr_q, order, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, st.dkm, st.dvm, c.status,
+                       work_counter, ipu, (int)total);
 }
 
 int launch_dkdv_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,

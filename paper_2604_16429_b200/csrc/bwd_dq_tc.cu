@@ -14,6 +14,11 @@
 // threads pull both into registers and hand the buffers back at once, so the next product's S and dP are
 // computed while they form dS (bf16, two buffers of 32 TMEM columns in turn); then dQ += dS K (dS is the TMEM A operand,
 // the K chunk in shared memory is read as the MN-major B operand), issued one product behind.
+// BR, the three-branch form: a list entry carries a mask of the halves that attend it locally and one of those that selected
+// it; the row threads take the matching statistics, gate and dO share, so one launch serves both branches, and the epilogue adds the
+// block level's share (with two launches, their sum in a third: 254 + 20 us at 8 units of 28800 tokens, now 188).
+// Bound by the row threads' queue of MUFU, shared-memory and TMEM instructions, in which a wait on a completed barrier takes
+// 150 to 250 cycles: a second dS buffer, which saves one, and cheaper polls took 64 units of 28800 tokens from 1401 to 1151 us.
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
 #include "tc_common.cuh"
 
@@ -81,6 +86,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     sm.abort = 0;
     cta_publish_barriers();
   }
+  block_idx += await_stream();  // before the TMEM is taken: a kernel ahead may still need it
   const uint32_t tmem = cta_tmem_alloc(warp == 9, &sm.tmem_base, kTmemCols);
   volatile int* abort = &sm.abort;
 
@@ -364,9 +370,8 @@ static int launch_dq_tc_t(const HostCtx& c, const void* q, const void* k, const 
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
   const Queue queue = make_queue(total, sms);
   const int grid = queue.positions < sms ? queue.positions : sms;
-  dq_tc_kernel<F16, BR><<<(unsigned)grid, kThreads, smem, c.stream>>>(
-      g, mq, mdo, mk, mv, block_idx, st, (__nv_bfloat16*)dq, c.status, work_counter, ipu, queue);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(dq_tc_kernel<F16, BR>, dim3((unsigned)grid), kThreads, smem, c.stream, true, 0, g, mq, mdo, mk, mv, block_idx,
+                       st, (__nv_bfloat16*)dq, c.status, work_counter, ipu, queue);
 }
 
 int launch_dq_tc(const HostCtx& c, const void* q, const void* k, const void* v, const void* d_o, const RowStats& st,

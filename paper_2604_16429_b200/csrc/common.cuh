@@ -96,7 +96,41 @@ __host__ __device__ inline int items_per_unit(const Geo& g) {
   return g.m * ((g.cpb + 3) >> 2);
 }
 
+// Every kernel is launched before the one ahead of it in the stream has finished (launch_kernel below): it sets up what
+// touches no global memory, then calls this.  It returns when everything ahead is complete and visible, and lets the next
+// kernel's CTAs in as SMs run empty (not earlier: the chain of waits makes "the kernel before me is complete" mean "all
+// before it are").  The result is zero, opaque to the compiler: an address that it takes part in cannot be read earlier.
+__device__ __forceinline__ int await_stream() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
+  return zero;
+}
+
 // ---- host side ---------------------------------------------------------------------------
+// Launches a kernel that calls await_stream; with `overlap` its launch and set-up overlap the kernel ahead of it.  A pass
+// of ten kernels over 3072 tokens takes 434 us without any overlap and 411 with it.  Not for kernels whose CTAs share SMs
+// and are few (pooling and ranking beyond one CTA per SM, the block level): they land where the kernel ahead runs empty
+// first and not evenly (pass over 8 units of 450 blocks: pooling 202.0 against 197.4 us, ranking 208.7 against 206.8; its
+// three-branch training: block level 1088 against 1082).
+template <class... P, class... A>
+inline int launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool overlap,
+                         int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...) == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+}
+
 struct HostCtx {
   Geo g;
   cudaStream_t stream;

@@ -33,6 +33,12 @@
 // more than 2^8 (then O is rescaled, between two P V products), packed two-lane fp32 arithmetic, and a
 // quarter of the exponentials evaluated by a cubic on the FMA pipe because at d = 64 the MUFU pipe
 // (16 ex2 per clock per SM against 8192 tensor FLOP per clock) is the limiter, not the tensor core.
+// Bound by the softmax warps: 730 cycles per product against 384 of MUFU time; one more satisfied wait per product costs
+// them 3 %, one more in the MMA issuers nothing (8 units of 28800 tokens 162 -> 155 us with cheaper polls and the queue's parts).
+// Three-branch form (kFwdBranches, kFwdStats): the planner hands out an item twice in a row, with its selected list and with
+// its local list; the first epilogue leaves the gated part in o, the second adds its own and the block level's.  kFwdStats
+// writes what the backward needs instead of an output.  Two launches and the gated sum took 204 us
+// at 8 units of 28800 tokens, one launch 182.
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
 
 
@@ -152,6 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     sm.abort = 0;
     cta_publish_barriers();
   }
+  block_idx += await_stream();  // before the TMEM is taken: a kernel ahead may still need it
   const uint32_t tmem = cta_tmem_alloc(warp == 9, &sm.tmem_base, kTmemCols);
   volatile int* abort = &sm.abort;
 
@@ -516,9 +523,8 @@ int launch_fwd_tc_t(const HostCtx& c, const CUtensorMap& mq, const CUtensorMap& 
   if (total > 0x7fffff00ll) return MOSAIC_E_UNSUPPORTED;
   const Queue queue = make_queue(total, sms);
   const int grid = queue.positions < sms ? queue.positions : sms;
-  fwd_tc_kernel<F16, MODE><<<(unsigned)grid, kThreads, smem, c.stream>>>(g, mq, mk, mv, block_idx, out, c.status,
-                                                                        work_counter, ipu, queue);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(fwd_tc_kernel<F16, MODE>, dim3((unsigned)grid), kThreads, smem, c.stream, true, 0, g, mq, mk, mv, block_idx,
+                       out, c.status, work_counter, ipu, queue);
 }
 }  // namespace
 

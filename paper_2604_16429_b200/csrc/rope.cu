@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256, 4) rope_kernel(Geo g, const uint4* __rest
   __shared__ double freq[kFreqs];
   if (threadIdx.x < kFreqs) freq[threadIdx.x] = pow(theta, -2.0 * threadIdx.x / (kD / 2));
   __syncthreads();
-  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // token of the grid
+  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x + await_stream()) >> 3;  // token of the grid
   const int part = threadIdx.x & 7;
   if (x >= g.N) return;
   const double p = (double)__ldg(pos + 2 * x + (part >> 2));  // longitude for channels 0..31, latitude for 32..63
@@ -118,11 +118,8 @@ int launch_rope(const HostCtx& c, const void* q, const void* k, const float* pos
   int split = 1;
   while (blocks * split < 1184 && split * 8 <= g.U + g.Ukv) split *= 2;
   const dim3 grid((unsigned)blocks, (unsigned)split);
-  if (g.f16)
-    rope_kernel<true><<<grid, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pos, theta, (uint4*)q_out, (uint4*)k_out);
-  else
-    rope_kernel<false><<<grid, 256, 0, c.stream>>>(g, (const uint4*)q, (const uint4*)k, pos, theta, (uint4*)q_out, (uint4*)k_out);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(g.f16 ? rope_kernel<true> : rope_kernel<false>, grid, 256, 0, c.stream, true, 0, g, (const uint4*)q,
+                       (const uint4*)k, pos, theta, (uint4*)q_out, (uint4*)k_out);
 }
 
 }  // namespace mosaic

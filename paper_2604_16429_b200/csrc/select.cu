@@ -36,6 +36,9 @@ namespace mosaic {
 // Screening twice costs less than keeping a threshold current during one pass did: with FMAs on the CUDA cores, their
 // operand loads (6 words per 8 FMAs) and the running thresholds a warp spent 1770 instructions on 4 rows x 64 keys; now
 // about 200 per pass on 16 rows x 16 keys.
+// What bounds it now is the split of the keys into parts and, for few rows, the chain of phases.  us, before -> after: 8 units
+// of 450 blocks 38.7 -> 26.2, 192 units 528 -> 384, 8 units of 4050 blocks 1382 -> 798, 24 units of 384 blocks with top-k 24
+// 136 -> 62.
 // ------------------------------------------------------------------------------------------
 
 // Total-order key: larger key = better score.  0 = not a candidate, 1 = NaN.
@@ -173,7 +176,8 @@ __global__ void __launch_bounds__(kTW * 32, 2) topk_kernel(Geo g, const float* _
   const float kInf = __int_as_float(0x7f800000);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles = (g.m + TI - 1) / TI;
-  const int u = blockIdx.x / tiles, i0 = (blockIdx.x - u * tiles) * TI;
+  const int cta = (int)blockIdx.x + await_stream();
+  const int u = cta / tiles, i0 = (cta - u * tiles) * TI;
   const float* pq_u = pq + (long long)u * g.m * kD;
   const float* pk_u = pk + (long long)kv_unit(g, u) * g.m * kD;   // grouped-query attention: the group's key head
   const float* nk_u = nk + (long long)kv_unit(g, u) * g.m;
@@ -459,8 +463,8 @@ int launch_topk(const HostCtx& c, const float* pooled_q, const float* pooled_k, 
   if (const int rc = launch_setup(reinterpret_cast<const void*>(topk_kernel<TI, CAP>), smem, &configured, &sms)) return rc;
   const long long ctas = (long long)g.U * ((g.m + TI - 1) / TI);
   if (ctas > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
-  topk_kernel<TI, CAP><<<(unsigned)ctas, kTW * 32, smem, c.stream>>>(g, pooled_q, pooled_k, norm_q, norm_k, block_idx);
-  return cudaGetLastError() == cudaSuccess ? MOSAIC_OK : MOSAIC_E_CUDA;
+  return launch_kernel(topk_kernel<TI, CAP>, dim3((unsigned)ctas), kTW * 32, smem, c.stream, ctas <= sms, 0, g, pooled_q, pooled_k, norm_q,
+                       norm_k, block_idx);
 }
 
 int launch_select(const HostCtx& c, const void* q, const void* k, int32_t* block_idx, float* pooled_q,

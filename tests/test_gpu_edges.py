@@ -183,3 +183,34 @@ def test_rope_unit_shares_and_non_finite_values(heads, kv, f16):
             total += dist.size
             same += int((dist == 0).sum())
     assert same >= 0.9999 * total
+
+
+@pytest.mark.parametrize("nlat,nlon,heads", [(16, 24, 2), (64, 128, 4), (120, 160, 6)])
+def test_passes_back_to_back_on_the_same_buffers(nlat, nlon, heads):
+    """Launches overlap the kernel ahead of them: passes over two inputs in turn, with one workspace and one set of outputs
+    and no synchronisation between them, give the bits of passes that ran alone."""
+    w = synth.small_case(nlat, nlon, 8, 8, 3, H=heads, seed=460 + heads, backward=True)
+    p = mb.Params.from_workload(w)
+    xs = [G.device_inputs(synth.make_inputs(dataclasses.replace(w, cfg=w.cfg + 7 * i))) for i in range(2)]
+    gates = torch.randn((1, heads, w.N, 3), device="cuda", generator=torch.Generator("cuda").manual_seed(heads))
+    ws = torch.empty(max(mb.workspace_bytes(p, op) for op in range(5)), dtype=torch.uint8, device="cuda")
+    idx = torch.empty((1, heads, w.m, 3), dtype=torch.int32, device="cuda")
+    o, lse = torch.empty_like(xs[0]["q"]), torch.empty((1, heads, w.N), device="cuda")
+    grads, three, dg = [[torch.empty_like(o) for _ in range(3)] for _ in range(2)] + [torch.empty_like(gates)]
+
+    def run(x):
+        mb.mosaic_bsa_select(p, x["q"], x["k"], block_idx=idx, ws=ws)
+        mb.mosaic_bsa_fwd(p, x["q"], x["k"], x["v"], idx, o=o, lse=lse, ws=ws)
+        mb.mosaic_bsa_bwd(p, x["q"], x["k"], x["v"], o, lse, x["do"], idx, dq=grads[0], dk=grads[1], dv=grads[2], ws=ws)
+        mb.mosaic_bsa_bwd_branches(p, x["q"], x["k"], x["v"], idx, gates, x["do"], dq=three[0], dk=three[1], dv=three[2],
+                                   dgates=dg, ws=ws)
+        return [t.clone() for t in (idx, o, lse, *grads, *three, dg)]
+
+    alone = []
+    for x in xs:
+        torch.cuda.synchronize()
+        alone.append(run(x))
+    torch.cuda.synchronize()
+    for i, got in enumerate([run(xs[i % 2]) for i in range(6)]):
+        for a, b in zip(got, alone[i % 2]):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), i
