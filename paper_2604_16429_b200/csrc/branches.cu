@@ -303,10 +303,12 @@ __global__ void __launch_bounds__(kThr) compress_bwd_kernel(Geo g, const Compres
   else compress_bwd_tile<true>(g, sm, (cta - query_ctas) / ranks, a);
 }
 
-// CTAs per tile: enough of them that every SM gets about two, at most one per chunk (and 8, the portable cluster size)
+// CTAs per tile: enough of them that every SM gets one, at most one per chunk (and 8, the portable cluster size).  With two
+// per SM the sums over the ranks and the repeated loads cost more than the shorter streams give (8 units of 450 blocks:
+// forward twice 52.8 us against 44.1, backward 80.8 against 69.3; without clusters 84.1 and 89.3).
 int cluster_size(long long tiles_total, int chunks) {
   int s = 1;
-  while (s < 8 && tiles_total * s < 296 && 2 * s <= chunks) s *= 2;
+  while (s < 8 && tiles_total * s < 148 && 2 * s <= chunks) s *= 2;
   return s;
 }
 

@@ -75,7 +75,7 @@ def _compare3_units(w, x, idx_h, gates, got, units, compare):
 
 
 # Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2, 4 or 8 CTAs (as many as
-# give every SM two, at most one per chunk; on the key side the chunks of all query heads of a group count).
+# give every SM one, at most one per chunk; on the key side the chunks of all query heads of a group count).
 COMPRESS = [synth.small_case(8 * m, 8, 8, 8, 2, H=h, Hkv=kv, seed=360 + i, backward=True) for i, (m, h, kv) in enumerate([
     (63, 1, 0), (64, 1, 0), (65, 1, 0), (129, 1, 0), (193, 1, 0), (449, 1, 0), (65, 4, 1), (65, 6, 2)])]
 
