@@ -64,7 +64,7 @@ struct Smem {
   unsigned long long kv_full[kStages], kv_empty[kStages];
   unsigned long long q_full[2][2], q_empty[2][2];  // [item parity][tile]
   unsigned long long mma_drain_bar[2];             // abort path: completion of each issuer's outstanding products
-  unsigned long long q_ready[2];                   // [tile]: the item's query rows are in TMEM
+  unsigned long long q_ready[2];                   // [tile]: the query rows of a list the tile attends are in TMEM
   unsigned long long s_full[2][2], p_full[2][2], pv_done[2][2];  // [tile][S buffer]
   unsigned long long list_full[kLists], list_empty[kLists];
   uint32_t tmem_base;
@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tcol_o = tmem + kColO + 64 * t, tcol_s = tmem + kColS + 128 * t, tcol_q = tmem + kColQ + 32 * t;
     uint32_t base = 0;    // ring position of the item's first chunk
     uint32_t nt = 0;      // products issued by this tile so far: buffer nt & 1, phase (nt >> 1) & 1
+    uint32_t nq = 0;      // lists that this tile attends so far (phase of q_ready)
     bool ok = true;
     // P V of product `pn` (its V chunk sits in ring stage `pst`); `pfirst` starts a new accumulation
     auto issue_pv = [&](uint32_t pn, int pst, bool pfirst) {
@@ -255,13 +256,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       const int n = sm.info[buf].n;
       if (n < 0) break;
-      // the item's query rows are in TMEM (copied there by the softmax threads)
-      ok = warp_wait(s32(&sm.q_ready[t]), it & 1, abort, status);
-      if (!ok) break;
+      const int cnt = sm.info[buf].nsteps[t];
+      // the item's query rows are in TMEM (copied there by the softmax threads).  A list that the tile does not attend has no
+      // such hand-off: nothing would keep the softmax threads from running two phases ahead of this warp.
+      if (cnt > 0) {
+        ok = warp_wait(s32(&sm.q_ready[t]), nq & 1, abort, status);
+        if (!ok) break;
+        ++nq;
+      }
       bool first = true, pend = false, pend_first = false;
       uint32_t pend_n = 0, pend_step = 0;
       int pend_st = 0;
-      const int cnt = sm.info[buf].nsteps[t];
       for (int i = 0; i < cnt && ok; ++i) {
         uint32_t step = base + (sm.steps[buf][t][i] >> 8) * (uint32_t)g.cpb;
         for (int c = 0; c < g.cpb && ok; ++c, ++step) {
@@ -331,10 +336,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint4 v = *reinterpret_cast<const uint4*>(rowp + ((c ^ (r & 7)) << 4));
         qv[4 * c] = v.x; qv[4 * c + 1] = v.y; qv[4 * c + 2] = v.z; qv[4 * c + 3] = v.w;
       }
-      tmem_st32(tq, qv);
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(s32(&sm.q_ready[t]));
+      if (sm.info[buf2].nsteps[t] > 0) {  // (the same for the whole warp)
+        tmem_st32(tq, qv);
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(s32(&sm.q_ready[t]));
+      }
       mbar_arrive(s32(&sm.q_empty[qb2][t]));
       return n2;
     };

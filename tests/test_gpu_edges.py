@@ -74,6 +74,28 @@ def _compare3_units(w, x, idx_h, gates, got, units, compare):
         compare(one, {k: v[:, s] for k, v in x.items()}, idx_h[:, s], gates[:, s], [t[:, s] for t in got])
 
 
+@pytest.mark.parametrize("nlat,nlon,heads,topk", [(16, 16, 37, 0), (16, 16, 74, 0), (16, 16, 80, 0), (16, 16, 444, 0), (8, 24, 38, 3),
+                                                  (16, 16, 37, 4), (64, 64, 5, 4)])
+def test_lists_that_a_tile_does_not_attend(nlat, nlon, heads, topk):
+    """Without selected blocks every list of the selection branch is empty, and a part of an item leaves one tile empty in
+    both of its lists: the roles of a tile that has nothing to do stay in step, pass after pass.  No block is selected here
+    (top-k 0, or rows of -1); on the largest grid every fourth row selects one."""
+    w = synth.small_case(nlat, nlon, 8, 8, topk, H=heads, seed=350 + heads, rlat=0, rlon=0, backward=True)
+    x = synth.make_inputs(w)
+    idx_h = np.full((1, heads, w.m, topk), -1, np.int32)
+    if w.m > 4:
+        idx_h[:, :, ::4, 1] = (np.arange(0, w.m, 4) + 5) % w.m
+    idx = torch.from_numpy(idx_h).cuda()
+    gates = np.random.default_rng(heads).standard_normal((1, heads, w.N, 3))
+    first = T._run(w, x, idx, gates), T._run_bwd3(w, x, idx, gates)
+    units = sorted({0, heads // 2, heads - 1})
+    _compare3_units(w, x, idx_h, gates, first[0], units, T._compare)
+    _compare3_units(w, x, idx_h, gates, first[1], units, T._compare_bwd3)
+    for _ in range(20):
+        for run, want in zip((T._run, T._run_bwd3), first):
+            assert all(np.array_equal(a, b) for a, b in zip(run(w, x, idx, gates), want))
+
+
 # Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2, 4 or 8 CTAs (as many as
 # give every SM one, at most one per chunk; on the key side the chunks of all query heads of a group count).
 COMPRESS = [synth.small_case(8 * m, 8, 8, 8, 2, H=h, Hkv=kv, seed=360 + i, backward=True) for i, (m, h, kv) in enumerate([
