@@ -36,7 +36,7 @@ struct Smem {
   unsigned char q[2][2 * kTile];           // [tile][128 rows x 128 B]
   unsigned char d_o[2][2 * kTile];         // [tile][128 rows x 128 B]
   unsigned char kv[kStages][2][kTile];     // [stage][K, V]
-  unsigned long long kv_full[kStages], kv_empty[kStages];
+  unsigned long long kv_full[kFullBars], kv_empty[kStages];
   unsigned long long q_full[2], q_empty[2], s_full[2], sdp_free[2];  // [tile]
   unsigned long long p_full[2][2], pv_done[2][2];  // [tile][dS buffer]
   unsigned long long mma_drain_bar[2];  // abort path: completion of each issuer's outstanding products
@@ -50,6 +50,8 @@ struct Smem {
   int tmp_ids[kMaxUnion];            // planner scratch: merged list before reordering
   unsigned char tmp_mask[kMaxUnion];
 };
+
+static_assert(kFullBars >= kMaxUnion + kStages && (kFullBars & (kFullBars - 1)) == 0, "a list's chunks land on barriers of their own");
 
 }  // namespace
 
@@ -67,7 +69,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(s32(&sm.kv_full[s]), 1); mbar_init(s32(&sm.kv_empty[s]), 2); }
+    for (int s = 0; s < kStages; ++s) mbar_init(s32(&sm.kv_empty[s]), 2);
     for (int t = 0; t < 2; ++t) {
       mbar_init(s32(&sm.q_full[t]), 1);
       mbar_init(s32(&sm.q_empty[t]), 1);
@@ -84,8 +86,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(s32(&sm.list_empty[i]), 11);  // 8 row-thread warps + 2 MMA warps + TMA producer
     }
     sm.abort = 0;
-    cta_publish_barriers();
   }
+  for (int s = tid; s < kFullBars; s += kThreads) mbar_init(s32(&sm.kv_full[s]), 1);
+  cta_publish_barriers();
   block_idx += await_stream();  // before the TMEM is taken: a kernel ahead may still need it
   const uint32_t tmem = cta_tmem_alloc(warp == 9, &sm.tmem_base, kTmemCols);
   volatile int* abort = &sm.abort;
@@ -95,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      long long step = 0;  // key/value chunks issued so far (ring position)
+      uint32_t step = 0;   // key/value chunks issued so far (ring position)
       int q_armed[2] = {-1, -1};  // phase parity of the last load into each tile's Q / dO buffer
       bool ok = true;
       for (int it = 0; ok; ++it) {
@@ -124,12 +127,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int j = sm.ids[buf][e], by = j / g.nbw, bx = j - by * g.nbw;
           const uint32_t mk = who_attends(sm.mask[buf][e]);
           for (int c = 0; c < g.cpb; ++c, ++step) {
-            const int st = (int)(step % kStages);
-            ok = mbar_wait(s32(&sm.kv_empty[st]), (uint32_t)((step / kStages) & 1) ^ 1, abort, status);
+            const uint32_t st = step % kStages;
+            const uint32_t full = s32(&sm.kv_full[step % kFullBars]);
+            ok = mbar_wait(s32(&sm.kv_empty[st]), ((step / kStages) & 1) ^ 1, abort, status);
             if (!ok) break;
-            mbar_expect_tx(s32(&sm.kv_full[st]), 2 * kTile);
-            tma_load_4d(s32(sm.kv[st][0]), &map_k, s32(&sm.kv_full[st]), 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
-            tma_load_4d(s32(sm.kv[st][1]), &map_v, s32(&sm.kv_full[st]), 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
+            mbar_expect_tx(full, 2 * kTile);
+            tma_load_4d(s32(sm.kv[st][0]), &map_k, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
+            tma_load_4d(s32(sm.kv[st][1]), &map_v, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
             // a tile that does not attend this entry never looks at the stage: its release is given here
             if (!(mk & 3u)) mbar_arrive(s32(&sm.kv_empty[st]));
             if (!(mk & 12u)) mbar_arrive(s32(&sm.kv_empty[st]));
@@ -138,14 +142,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
       }
       if (*abort) {  // copies this thread issued must land before the CTA's memory is released
-        const long long first = step > kStages ? step - kStages : 0;
-        for (long long s = first; s < step; ++s) mbar_drain(s32(&sm.kv_full[s % kStages]), (uint32_t)((s / kStages) & 1));
+        const uint32_t first = step > kStages ? step - kStages : 0;
+        for (uint32_t s = first; s < step; ++s) mbar_drain(s32(&sm.kv_full[s % kFullBars]), (s / kFullBars) & 1);
         for (int t = 0; t < 2; ++t)
           if (q_armed[t] >= 0) mbar_drain(s32(&sm.q_full[t]), (uint32_t)q_armed[t]);
       } else {       // drain: the last uses of every ring stage have been released by both tiles
-        const long long first = step > kStages ? step - kStages : 0;
-        for (long long s = first; s < step; ++s)
-          if (!mbar_wait(s32(&sm.kv_empty[s % kStages]), (uint32_t)((s / kStages) & 1), abort, status)) break;
+        const uint32_t first = step > kStages ? step - kStages : 0;
+        for (uint32_t s = first; s < step; ++s)
+          if (!mbar_wait(s32(&sm.kv_empty[s % kStages]), (s / kStages) & 1, abort, status)) break;
       }
     }
   } else if (warp == 9 || warp == 10) {
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             pend = false;
             if (!ok) break;
           }
-          ok = warp_wait(s32(&sm.kv_full[st]), (step / kStages) & 1u, abort, status);
+          ok = warp_wait(s32(&sm.kv_full[step % kFullBars]), (step / kFullBars) & 1u, abort, status);
           if (!ok) break;
           // S and dP may be overwritten once the row threads hold the previous product's values in registers
           if (nt > 0) {

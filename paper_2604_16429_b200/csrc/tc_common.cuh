@@ -14,6 +14,14 @@ namespace {
 constexpr int kTile = 8192;                      // bytes of one 64 x 64 bf16 chunk
 constexpr int kMaxUnion = 4 * kMaxList;          // most entries of an item's merged key list
 constexpr int kLists = 4;                        // key lists in flight (the planner runs this far ahead)
+// Barriers on which the key/value chunks of the row-stationary kernels land: one per ring position modulo kFullBars, many more
+// than stages of data.  A tile's issuer looks only at the chunks its tile attends (the producer releases the others on its
+// behalf), and a wait on a phase's parity is exact only if the barrier's previous phase has completed: with one barrier per
+// stage the phase two rounds back, of an older chunk, passed for the awaited one.  What the issuer knows when it looks at a
+// chunk: every earlier list is armed (the list's query tile was loaded after them), and in this list everything up to its
+// last chunk.  An armed chunk means that the chunks a ring's length before it have landed, so the barrier's previous phase
+// has completed if kFullBars is at least the longest list plus the stages.
+constexpr int kFullBars = 512;
 #ifdef MOSAIC_TEST_SPIN_CYCLES                   // test build only: a short bound, so that a wait that nothing ends runs out quickly
 constexpr long long kSpinCycles = MOSAIC_TEST_SPIN_CYCLES;
 #else

@@ -178,6 +178,43 @@ def test_a_tile_that_skips_most_of_its_items_list(bh, bw, nlat, nlon):
     T._compare_bwd3(w, x, idx_h, gates, T._run_bwd3(w, x, idx, gates))
 
 
+@pytest.mark.parametrize("bh,bw,nlat,nlon,heads,f16", [(8, 8, 64, 64, 5, False), (8, 16, 64, 128, 3, False), (16, 8, 128, 64, 3, True)])
+def test_lists_of_very_different_lengths(bh, bw, nlat, nlon, heads, f16):
+    """The key ring goes round several times between two entries of a tile: in every other 2 x 2 group the upper two blocks
+    (128-token blocks: the left one of a pair) select 56 blocks of which the lower two (the right one) select none, the first
+    or the last; four common blocks make sure that the two long lists share a tile.  The other groups' rows have 0, 1 or 30
+    entries at random.  80 and 96 items, which the work queue does not cut."""
+    w = synth.small_case(nlat, nlon, bh, bw, 30, H=heads, seed=430 + bw + bh, rlat=0, rlon=0, backward=True, f16=f16)
+    x = synth.make_inputs(w)
+    dx = G.device_inputs(x, f16=f16)
+    nbh, nbw = nlat // bh, nlon // bw
+    rng = np.random.default_rng(w.cfg)
+    idx_h = np.full((1, heads, w.m, 30), -1, np.int32)
+    for n, (h, y, c) in enumerate((h, y, c) for h in range(heads) for y in range(0, nbh, 2) for c in range(0, nbw, 2)):
+        own = [y * nbw + c, y * nbw + c + 1, (y + 1) * nbw + c, (y + 1) * nbw + c + 1]
+        far = [int(j) for j in rng.permutation([j for j in range(w.m) if j not in own])]
+        if n % 2:
+            rows = [list(rng.permutation(far)[:k]) for k in rng.choice([0, 1, 30], size=4)]
+        else:
+            long = [far[:30], far[26:56]]
+            short = [[far[0]] if n & 2 else [], [far[55]] if n & 4 else []]
+            rows = long + short if bh * bw == 64 else [long[0], short[0], long[1], short[1]]
+        for j, r in zip(own, rows):
+            idx_h[0, h, j, :len(r)] = r
+    idx = torch.from_numpy(idx_h).cuda()
+    o, lse = G.gpu_fwd(w, dx, idx)
+    grads = G.gpu_bwd(w, dx, o, lse, idx)
+    for h in range(heads):
+        G.compare_fwd_unit(w, x, 0, h, idx_h[0, h], o, lse)
+        ref = oracle.bwd(G.geom_of(w), x["q"][0, h], x["k"][0, h], x["v"][0, h], x["do"][0, h], idx_h[0, h])
+        for name, got, want in zip(("dQ", "dK", "dV"), grads, ref):
+            G.assert_bwd_close(f"{name} unit {h}", got[0, h], want)
+    if not f16:
+        gates = rng.standard_normal((1, heads, w.N, 3))
+        _compare3_units(w, x, idx_h, gates, T._run(w, x, idx, gates), range(heads), T._compare)
+        _compare3_units(w, x, idx_h, gates, T._run_bwd3(w, x, idx, gates), range(heads), T._compare_bwd3)
+
+
 @pytest.mark.parametrize("f16", [False, True])
 @pytest.mark.parametrize("heads,kv", [(1, 1), (6, 1), (7, 1), (6, 6), (24, 1), (15, 15)])
 def test_rope_unit_shares_and_non_finite_values(heads, kv, f16):
