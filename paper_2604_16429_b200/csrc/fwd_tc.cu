@@ -36,7 +36,8 @@
 // Bound by the softmax warps: 730 cycles per product against 384 of MUFU time; one more satisfied wait per product costs
 // them 3 %, one more in the MMA issuers nothing (8 units of 28800 tokens 162 -> 155 us with cheaper polls and the queue's parts).
 // Three-branch form (kFwdBranches, kFwdStats): the planner hands out an item twice in a row, with its selected list and with
-// its local list; the first epilogue leaves the gated part in o, the second adds its own and the block level's.  kFwdStats
+// its local list; the first epilogue leaves the selected part in o (not gated yet: a weighted mean of values fits their type
+// whatever the gates are), the second weights it and adds its own and the block level's.  kFwdStats
 // writes what the backward needs instead of an output.  Two launches and the gated sum took 204 us
 // at 8 units of 28800 tokens, one launch 182.
 // Every mbarrier wait is bounded; on expiry the CTA records MOSAIC_E_DEVICE_TIMEOUT and drains.
@@ -79,10 +80,10 @@ struct Smem {
 
 static_assert(kFullBars >= kMaxUnion + kStages && (kFullBars & (kFullBars - 1)) == 0, "a list's chunks land on barriers of their own");
 
-// 32 channels of a token's output row (fp32 in `a`) times f, stored in 16 bits; `add`: plus the row that `dst` holds already
-// and gc times the block-level vector cg.
+// 32 channels of a token's output row (fp32 in `a`) times f, stored in 16 bits; `add`: plus gs times the row that `dst` holds
+// already and gc times the block-level vector cg.
 template <bool F16>
-__device__ __forceinline__ void store_row(uint4* dst, const uint32_t* a, float f, bool add, float gc, const float* cg) {
+__device__ __forceinline__ void store_row(uint4* dst, const uint32_t* a, float f, bool add, float gs, float gc, const float* cg) {
 #pragma unroll
   for (int x = 0; x < 4; ++x) {
     float v[8];
@@ -97,8 +98,8 @@ __device__ __forceinline__ void store_row(uint4* dst, const uint32_t* a, float f
       for (int y = 0; y < 4; ++y) {
         float lo, hi;
         unpack16x2(ow[y], F16, lo, hi);
-        v[2 * y] += lo + gc * cv[2 * y];
-        v[2 * y + 1] += hi + gc * cv[2 * y + 1];
+        v[2 * y] += gs * lo + gc * cv[2 * y];
+        v[2 * y + 1] += gs * hi + gc * cv[2 * y + 1];
       }
     }
     dst[x] = make_uint4(pack2<F16>(v[0], v[1]), pack2<F16>(v[2], v[3]), pack2<F16>(v[4], v[5]), pack2<F16>(v[6], v[7]));
@@ -478,6 +479,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float* cg = MODE == kFwdUnion ? nullptr : out.ocg + ((long long)u * g.m + blk) * kD;
         const float gx = MODE == kFwdUnion ? 1.f : __ldg(out.gates + 3 * tok + 1 + branch);
         const float gc = MODE == kFwdBranches && branch ? __ldg(out.gates + 3 * tok) : 0.f;
+        const float gs = MODE == kFwdBranches && branch ? __ldg(out.gates + 3 * tok + 1) : 0.f;
         float dot = 0.f, dotc = 0.f;
         const long long at = (branch ? 0 : (long long)g.U * g.N) + tok;  // statistics: plane 0 local, plane 1 selected
 #pragma unroll
@@ -494,8 +496,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             dot_row<F16>(reinterpret_cast<const uint4*>(out.d_o + tok * kD) + 4 * part, ov, cg + 32 * part, gx,
                          static_cast<uint4*>(out.gated_do) + at * 8 + 4 * part, dot, dotc);
           else
-            store_row<F16>(reinterpret_cast<uint4*>(out.o + tok * kD) + 4 * part, ov, inv * gx,
-                           MODE == kFwdBranches && branch == 1, gc, cg + 32 * part);
+            store_row<F16>(reinterpret_cast<uint4*>(out.o + tok * kD) + 4 * part, ov, MODE == kFwdBranches && !branch ? inv : inv * gx,
+                           MODE == kFwdBranches && branch == 1, gs, gc, cg + 32 * part);
         }
         if (MODE == kFwdUnion) {
           out.lse[tok] = lse2 * 0.6931471805599453f;

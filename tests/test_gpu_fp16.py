@@ -96,3 +96,27 @@ def test_three_branch_forward_backward_and_rope_in_binary16():
             a, b_ = bits[0, h].astype(np.int32), want.astype(np.int32)
             oa, ob = np.where(a & 0x8000, -(a & 0x7FFF), a), np.where(b_ & 0x8000, -(b_ & 0x7FFF), b_)
             assert np.abs(oa - ob).max() <= 1 and (oa == ob).mean() >= 0.9999, name
+
+
+def test_three_branch_forward_in_binary16_with_large_gates_that_cancel():
+    """Gates are any numbers: the gated branches may leave binary16's range (1000 times 100) where their sum does not.
+    Every weight and every 16-bit value on the way to a branch output is off by at most 2^-11 of it, so a branch by 2 * 2^-11
+    of the largest value, times its gate; the sum rounds once more."""
+    w = synth.small_case(32, 64, 8, 8, 4, B=1, H=2, seed=127, f16=True)
+    x = synth.make_inputs(w)
+    rng = np.random.default_rng(127)
+    x["v"] = (100 + rng.standard_normal(x["v"].shape)).astype(np.float16).view(np.uint16)
+    dx = G.device_inputs(x, f16=True)
+    p = mb.Params.from_workload(w)
+    idx = G.gpu_select(w, dx)
+    g = G.geom_of(w)
+    for signs in ((0.0, 1000.0, -995.0), (0.0, -1000.0, 995.0), (-1990.0, 1000.0, 1000.0)):
+        gates = np.float32(signs) + rng.standard_normal((w.B, w.H, w.N, 3)).astype(np.float32)
+        o, _, _ = mb.mosaic_bsa_fwd_branches(p, dx["q"], dx["k"], dx["v"], idx, torch.from_numpy(gates).cuda())
+        for h in range(w.H):
+            gq = gates[0, h].astype(np.float64)
+            ref = oracle.fwd3(g, x["q"][0, h], x["k"][0, h], x["v"][0, h], idx[0, h].cpu().numpy(), gq)["o"]
+            top = np.abs(oracle.widen16(g, x["v"][0, h])).max()
+            bound = 2.0 ** -11 * (2 * top * np.abs(gq).sum(axis=1, keepdims=True) + np.abs(ref))
+            got = o[0, h].float().cpu().numpy()
+            assert np.isfinite(got).all() and (np.abs(got - ref) <= bound).all(), (signs, np.abs(got - ref).max())
