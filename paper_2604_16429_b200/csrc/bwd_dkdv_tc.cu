@@ -64,7 +64,7 @@ struct Smem {
   uint32_t tmem_base;
   int abort;
   ItemInfo info[kLists];             // hb/hc/hvalid entries 0 and 1 describe the tile's two halves
-  int ids[kLists][kMaxUnion];
+  alignas(16) int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
 };
 
@@ -127,9 +127,14 @@ __device__ __forceinline__ void planner_kv_loop(Smem& sm, const Geo& g, const in
         acquire();
         if (!ok) break;
       }
-      // local neighbourhoods (at most 64 entries per block, merged with masks), straight into the list buffer
-      if (use0) n = merge_block(g, true, -1, hb[0], bits0, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
-      if (use1) n = merge_block(g, true, -1, hb[1], bits1, sm.ids[lb % kLists], sm.mask[lb % kLists], n, lane, status);
+      // local neighbourhoods, merged with masks, straight into the list buffer (the window is made anew: kept over the loop it
+      // costs the row threads registers, 64 units of 28800 tokens in training 4700 us against 4675)
+      const Window w = make_window(g, lane);
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh)
+        if (hh == 0 ? use0 : use1)
+          n = merge_list(local_id(g, w, hh == 0 ? hb[0] : hb[1]), hh == 0 ? bits0 : bits1, -1, 0u, sm.ids[lb % kLists],
+                         sm.mask[lb % kLists], n, lane);
       // query blocks that selected the key block (ascending ids), appended 32 at a time
       const int32_t* off = csr_off + (long long)qu * (g.m + 1);
       const int32_t* sel = csr_q + (long long)qu * g.m * g.topk;

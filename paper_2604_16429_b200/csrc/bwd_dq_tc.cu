@@ -44,10 +44,10 @@ struct Smem {
   uint32_t tmem_base;
   int abort;
   ItemInfo info[kLists];
-  int ids[kLists][kMaxUnion];
+  alignas(16) int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
   unsigned short steps[kLists][2][kMaxUnion];  // [list][tile]
-  int tmp_ids[kMaxUnion];            // planner scratch: merged list before reordering
+  alignas(16) int tmp_ids[kMaxUnion];            // planner scratch: merged list before reordering
   unsigned char tmp_mask[kMaxUnion];
 };
 

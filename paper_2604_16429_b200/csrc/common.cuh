@@ -77,6 +77,14 @@ __device__ __forceinline__ bool is_local(const Geo& g, int i, int j) {
   return row_ok && col_ok;
 }
 
+// a / b for 0 <= a < 2^24 and inv = 1.0f / b: the rounded quotient is off by at most one
+__device__ __forceinline__ int quick_div(int a, int b, float inv) {
+  int q = __float2int_rz((float)a * inv);
+  const int r = a - q * b;
+  q += r >= b ? 1 : r < 0 ? -1 : 0;
+  return q;
+}
+
 // First token (row-major grid index inside the unit) of row `r` of chunk `c` of block j.
 __device__ __forceinline__ long long chunk_row_token(const Geo& g, int j, int c, int r) {
   int by = j / g.nbw, bx = j - by * g.nbw;

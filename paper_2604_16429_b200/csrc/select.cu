@@ -153,14 +153,6 @@ __device__ __forceinline__ unsigned long long exact_key(const float* qrow, const
   return score_key(s);
 }
 
-// a / b for 0 <= a < 2^24 and inv = 1.0f / b: the rounded quotient is off by at most one
-__device__ __forceinline__ int quick_div(int a, int b, float inv) {
-  int q = __float2int_rz((float)a * inv);
-  const int r = a - q * b;
-  q += r >= b ? 1 : r < 0 ? -1 : 0;
-  return q;
-}
-
 template <int TI, int CAP>
 __global__ void __launch_bounds__(kTW * 32, 2) topk_kernel(Geo g, const float* __restrict__ pq, const float* __restrict__ pk,
                                                            const float* __restrict__ nq, const float* __restrict__ nk,

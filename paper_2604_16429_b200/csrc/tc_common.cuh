@@ -375,106 +375,128 @@ __device__ __forceinline__ int item_halves(const Geo& g, int it, int (&hb)[4], i
 struct Queue {
   int full, pieces, positions;
 };
-// Halves of queue position `pos`: the item's unit and index inside the unit in u and it, the result and hb, hc as from
-// item_halves; a part's halves come first.
-__device__ __forceinline__ int queue_halves(const Geo& g, const Queue& q, int pos, int ipu, int& u, int (&hb)[4], int (&hc)[4]) {
-  const int cut = max(pos - q.full, 0), item = min(pos, q.full) + cut / q.pieces, part = cut % q.pieces;
+// The item of queue position `pos`: its unit and index inside the unit in u and it; the position covers the item's halves
+// first .. first + width - 1.
+__device__ __forceinline__ void queue_item(const Queue& q, int pos, int ipu, int& u, int& it, int& first, int& width) {
+  const int cut = max(pos - q.full, 0), item = min(pos, q.full) + cut / q.pieces;
   u = item / ipu;
-  int valid = item_halves(g, item - u * ipu, hb, hc);
-  if (pos >= q.full && q.pieces > 1) {
-    const int first = q.pieces == 2 ? 2 * part : part;
-    valid = (valid >> first) & (q.pieces == 2 ? 3 : 1);
-    const int b0 = hb[first], c0 = hc[first], b1 = hb[q.pieces == 2 ? first + 1 : first], c1 = hc[q.pieces == 2 ? first + 1 : first];
-    hb[0] = hb[2] = hb[3] = b0;
-    hc[0] = hc[2] = hc[3] = c0;
-    hb[1] = b1;
-    hc[1] = c1;
+  it = item - u * ipu;
+  width = pos >= q.full ? 4 / q.pieces : 4;
+  first = cut % q.pieces * width;
+}
+// Mask of an entry in the list of the halves first .. first + width - 1 (which come first there)
+__device__ __forceinline__ unsigned part_mask(unsigned m, int first, int width) {
+  const unsigned keep = (1u << width) - 1u;
+  return ((m & 15u) >> first & keep) | ((m >> 4 >> first & keep) << 4);
+}
+// Drops the entries that none of the halves first .. first + width - 1 attends; returns the number of entries left.
+__device__ __forceinline__ int keep_part(int* ids, unsigned char* mask, int n, int first, int width, int lane) {
+  int kept = 0;
+  for (int e0 = 0; e0 < n; e0 += 32) {
+    const int e = e0 + lane, id = e < n ? ids[e] : 0;
+    const unsigned m = e < n ? part_mask(mask[e], first, width) : 0u, act = __ballot_sync(0xffffffffu, m != 0u);
+    __syncwarp();
+    if (m) {
+      const int at = kept + __popc(act & ((1u << lane) - 1u));
+      ids[at] = id;
+      mask[at] = (unsigned char)m;
+    }
+    kept += __popc(act);
+    __syncwarp();
   }
-  return valid;
+  return kept;
 }
 
-// Warp-cooperative attended list of query block i (local set if with_local, then valid selected ids) written to
-// ids[n0..); returns the new count.  `j` is this lane's entry of the block's row of block_idx (-1 beyond top-k).
-__device__ __forceinline__ int warp_attended(const Geo& g, bool with_local, int j, int i, int* ids, int n0, int lane,
-                                             int* status) {
-  const int by = i / g.nbw, bx = i - by * g.nbw;
-  int id = -1 - lane;  // lanes without a block hold distinct negative values
-  int nl;
-  if (g.local_groups) {   // the aligned group of rlat x rlon blocks that holds block i (ragged at the grid's edge)
-    nl = with_local ? g.rlat * g.rlon : 0;
-    if (lane < nl) {
-      const int dy = lane / g.rlon, dx = lane - dy * g.rlon;
-      const int y = (by / g.rlat) * g.rlat + dy, x = (bx / g.rlon) * g.rlon + dx;
-      if (y < g.nbh && x < g.nbw) id = y * g.nbw + x;
-    }
-  } else {
-    const int wl = 2 * g.rlon + 1;
-    nl = with_local ? (2 * g.rlat + 1) * wl : 0;
-    if (lane < nl) {
-      const int dy = lane / wl - g.rlat, dx = lane - (lane / wl) * wl - g.rlon;
-      const int y = min(max(by + dy, 0), g.nbh - 1);
-      int x = (bx + dx) % g.nbw;
-      x += x < 0 ? g.nbw : 0;
-      id = y * g.nbw + x;
-    }
+// What a planner's lane needs of the geometry for every block it lists: its place in the local set (row and column offset; in
+// group mode inside the group) and reciprocals for quick_div.  A list takes the planner 10000 cycles and more, about as long as
+// a short item: with integer divisions a selection and forward of 8 units of 28800 tokens took 188.3 us, now 185.8.
+struct Window {
+  int dy, dx;
+  bool in;  // the lane holds a place of the local set (columns that come round again in a narrow grid excluded)
+  float inv_nbw, inv_rlat, inv_rlon;
+};
+__device__ __forceinline__ Window make_window(const Geo& g, int lane) {
+  Window w;
+  const int wide = g.local_groups ? g.rlon : 2 * g.rlon + 1, high = g.local_groups ? g.rlat : 2 * g.rlat + 1;
+  w.dy = lane / wide;
+  w.dx = lane - w.dy * wide;
+  w.in = lane < high * wide && w.dx < g.nbw;
+  if (!g.local_groups) { w.dy -= g.rlat; w.dx -= g.rlon; }
+  w.inv_nbw = 1.0f / (float)g.nbw;
+  w.inv_rlat = 1.0f / (float)max(g.rlat, 1);
+  w.inv_rlon = 1.0f / (float)max(g.rlon, 1);
+  return w;
+}
+
+// This lane's block of query block i's local set (-1: none); the lanes hold the set in list order.  In group mode the set is
+// the aligned group of rlat x rlon blocks that holds block i (ragged at the grid's edge), else the window, whose rows beyond the
+// grid fold onto rows that it holds anyway.
+__device__ __forceinline__ int local_id(const Geo& g, const Window& w, int i) {
+  const int by = quick_div(i, g.nbw, w.inv_nbw), bx = i - by * g.nbw;
+  const int y = (g.local_groups ? quick_div(by, g.rlat, w.inv_rlat) * g.rlat : by) + w.dy;
+  int x = (g.local_groups ? quick_div(bx, g.rlon, w.inv_rlon) * g.rlon : bx) + w.dx;
+  const bool keep = w.in && y >= 0 && y < g.nbh && !(g.local_groups && x >= g.nbw);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {  // longitude is periodic (offsets of at most two, a grid may be one column wide)
+    x += x < 0 ? g.nbw : 0;
+    x -= x >= g.nbw ? g.nbw : 0;
   }
-  const unsigned same = __match_any_sync(0xffffffffu, id);
-  const bool keep = id >= 0 && (__ffs(same) - 1) == lane;  // first occurrence of a block
-  const unsigned km = __ballot_sync(0xffffffffu, keep);
-  if (keep) ids[n0 + __popc(km & ((1u << lane) - 1u))] = id;
-  int n = n0 + __popc(km);
-  // selected ids outside [-1, m), inside the local set (attended already) or repeated in the row: skipped, reported
+  return keep ? y * g.nbw + x : -1;
+}
+// This lane's entry j of query block i's row of block_idx, -1 if it is none or one that is skipped and reported: an id outside
+// [-1, m), inside the local set (attended already) or repeated in the row.
+__device__ __forceinline__ int selected_id(const Geo& g, const Window& w, int i, int j, int lane, int* status) {
   const unsigned twins = __match_any_sync(0xffffffffu, j);
-  if (j != -1 && (j < 0 || j >= g.m || is_local(g, i, j) || (__ffs(twins) - 1) != lane)) {
-    set_status(status, MOSAIC_E_DEVICE_BAD_INDEX);
-    j = -1;
+  if (j == -1) return -1;
+  bool bad = j < 0 || j >= g.m || (__ffs(twins) - 1) != lane;
+  if (!bad) {
+    const int by = quick_div(i, g.nbw, w.inv_nbw), bx = i - by * g.nbw, jy = quick_div(j, g.nbw, w.inv_nbw), jx = j - jy * g.nbw;
+    if (g.local_groups) {
+      bad = quick_div(jy, g.rlat, w.inv_rlat) == quick_div(by, g.rlat, w.inv_rlat) &&
+            quick_div(jx, g.rlon, w.inv_rlon) == quick_div(bx, g.rlon, w.inv_rlon);
+    } else {
+      int dx = jx - bx;
+      dx += dx < 0 ? g.nbw : 0;  // (jx - bx) mod nbw in [0, nbw)
+      bad = abs(jy - by) <= g.rlat && (dx <= g.rlon || g.nbw - dx <= g.rlon);
+    }
   }
-  const unsigned sm_ = __ballot_sync(0xffffffffu, j >= 0);
-  if (j >= 0) ids[n + __popc(sm_ & ((1u << lane) - 1u))] = j;
-  return n + __popc(sm_);
+  if (bad) set_status(status, MOSAIC_E_DEVICE_BAD_INDEX);
+  return bad ? -1 : j;
 }
 
-// Merge the attended list of query block `blk` into the item's list (ids/mask, n entries so far):
-// entries already present get `bits` OR-ed into their mask, new ones are appended.  Returns the new n.
-// `jsel` is this lane's entry of the block's row of block_idx (-1 beyond top-k, or where only the local set is wanted).
-__device__ __forceinline__ int merge_block(const Geo& g, bool with_local, int jsel, int blk, unsigned char bits, int* ids,
-                                           unsigned char* mask, int n, int lane, int* status) {
+// Merges the list of a query block into the item's list (ids/mask, n entries so far): the blocks id0 of all lanes, then the
+// blocks id1 (-1: none; no block twice).  Entries already present get the bits OR-ed into their mask, new ones are appended.
+// Returns the new n.
+__device__ __forceinline__ int merge_list(int id0, unsigned bits0, int id1, unsigned bits1, int* ids, unsigned char* mask, int n,
+                                          int lane) {
   const int n0 = n;
-  const int nb = warp_attended(g, with_local, jsel, blk, ids, n0, lane, status) - n0;  // staged behind the list
-  __syncwarp();
-  if (n0 == 0) {
-    for (int e = lane; e < nb; e += 32) mask[e] = bits;
-    __syncwarp();
-    return nb;
-  }
-  int mine[2], pos[2];  // at most 64 entries per block: two per lane
+  int pos0 = -1, pos1 = -1;
+#pragma unroll 4
+  for (int a = 0; a < n0; a += 4) {
+    const int4 v = *reinterpret_cast<const int4*>(ids + a);
+    const int id[4] = {v.x, a + 1 < n0 ? v.y : -2, a + 2 < n0 ? v.z : -2, a + 3 < n0 ? v.w : -2};
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int e = lane + 32 * r;
-    mine[r] = e < nb ? ids[n0 + e] : -1;
-    pos[r] = -1;
-  }
-#pragma unroll 8
-  for (int a = 0; a < n0; ++a) {
-    const int id = ids[a];
-    pos[0] = id == mine[0] ? a : pos[0];
-    pos[1] = id == mine[1] ? a : pos[1];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const bool have = mine[r] >= 0, fresh = have && pos[r] < 0;
-    if (have && pos[r] >= 0) mask[pos[r]] |= bits;
-    const unsigned fm = __ballot_sync(0xffffffffu, fresh);
-    if (fresh) {
-      const int at = n + __popc(fm & ((1u << lane) - 1u));
-      ids[at] = mine[r];
-      mask[at] = bits;
+    for (int x = 0; x < 4; ++x) {
+      pos0 = id[x] == id0 ? a + x : pos0;
+      pos1 = id[x] == id1 ? a + x : pos1;
     }
-    n += __popc(fm);
-    __syncwarp();
   }
-  return n;
+  __syncwarp();
+  const bool new0 = id0 >= 0 && pos0 < 0, new1 = id1 >= 0 && pos1 < 0;
+  const unsigned m0 = __ballot_sync(0xffffffffu, new0), m1 = __ballot_sync(0xffffffffu, new1), lower = (1u << lane) - 1u;
+  if (id0 >= 0) {
+    const int at = new0 ? n + __popc(m0 & lower) : pos0;
+    mask[at] = (unsigned char)(new0 ? bits0 : mask[at] | bits0);
+    if (new0) ids[at] = id0;
+  }
+  n += __popc(m0);
+  if (id1 >= 0) {
+    const int at = new1 ? n + __popc(m1 & lower) : pos1;
+    mask[at] = (unsigned char)(new1 ? bits1 : mask[at] | bits1);
+    if (new1) ids[at] = id1;
+  }
+  __syncwarp();
+  return n + __popc(m1);
 }
 
 // One lane of a converged warp (the same lane every time).
@@ -527,16 +549,19 @@ __device__ __forceinline__ void interleave_tiles(const int* sid, const unsigned 
     }
     if (e < n) {
       int pos = k;
+      const int step = 8 * nx;
+      const float inv = 1.0f / (float)step;
 #pragma unroll
       for (int y = 0; y < NC; ++y) {
         const int ny = cnt[y];
-        if (y == cls || ny == 0) continue;
-        // entries j of class y that come first: (8j + y) nx < (8k + cls) ny, ties to the lower class
-        const int R = (8 * k + cls) * ny - y * nx;
-        int c = 0;
-        if (y < cls) c = R >= 0 ? R / (8 * nx) + 1 : 0;
-        else c = R > 0 ? (R + 8 * nx - 1) / (8 * nx) : 0;
-        pos += min(c, ny);
+        // entries j of class y that come first: (8j + y) nx < (8k + cls) ny, ties to the lower class: one more than the
+        // quotient, if there is one (all below 2^20, where the rounded quotient is off by at most one; 191.3 us with divisions, 188.9
+        // without, in the pass named at Window)
+        const int R = (8 * k + cls) * ny - y * nx - (y > cls ? 1 : 0);
+        int q = __float2int_rz((float)R * inv);
+        const int r = R - q * step;
+        q += r >= step ? 1 : r < 0 ? -1 : 0;
+        if (y != cls && R >= 0) pos += min(q + 1, ny);
       }
       did[pos] = sid[e];
       dmask[pos] = (unsigned char)m;
@@ -579,6 +604,7 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
                                              volatile int* abort, int* status) {
   int lb = 0;  // list buffers handed out so far
   bool ok = true;
+  const Window w = make_window(g, lane);
   auto acquire = [&]() {  // wait until list buffer lb % kLists is free
     if (lane == 0) ok = mbar_wait(s32(&sm.list_empty[lb % kLists]), ((lb / kLists) & 1) ^ 1, abort, status);
     ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -594,8 +620,9 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
       if (lane == 0) { sm.info[lb % kLists].n = -1; mbar_arrive(s32(&sm.list_full[lb % kLists])); }
       break;
     }
-    int u, hb[4], hc[4];
-    const int valid = queue_halves(g, queue, item, ipu, u, hb, hc);
+    int u, in_unit, first, width, hb[4], hc[4];
+    queue_item(queue, item, ipu, u, in_unit, first, width);
+    const int valid = item_halves(g, in_unit, hb, hc);
     int jsel[4];  // the four rows of block_idx, fetched together
 #pragma unroll
     for (int h = 0; h < 4; ++h)
@@ -606,26 +633,17 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
         if (!ok) break;
       }
       int n = 0;
+#pragma unroll 1
+      for (int h = 0; h < 4; ++h) {  // (one copy of the code: with four, 186.0 us instead of 183.0 in the pass named at Window)
+        const int blk = h == 0 ? hb[0] : h == 1 ? hb[1] : h == 2 ? hb[2] : hb[3];
+        const int j = h == 0 ? jsel[0] : h == 1 ? jsel[1] : h == 2 ? jsel[2] : jsel[3];
+        unsigned bits = 0;  // the halves of this block
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        if (!((valid >> h) & 1)) continue;
-        bool first = true;  // first half of its block: merge the block's list once, for all its halves
-        unsigned char bits = 0;
-#pragma unroll
-        for (int h2 = 0; h2 < 4; ++h2) {
-          if (((valid >> h2) & 1) && hb[h2] == hb[h]) {
-            if (h2 < h) first = false;
-            bits |= (unsigned char)(1 << h2);
-          }
-        }
-        if (!first) continue;
-        if (PLAN == kPlanTagged) {
-          n = merge_block(g, true, -1, hb[h], bits, sm.tmp_ids, sm.tmp_mask, n, lane, status);
-          n = merge_block(g, false, jsel[h], hb[h], (unsigned char)(bits << 4), sm.tmp_ids, sm.tmp_mask, n, lane, status);
-        } else {
-          n = merge_block(g, PLAN == kPlanUnion || part == 1, part == 1 ? -1 : jsel[h], hb[h], bits, sm.tmp_ids,
-                          sm.tmp_mask, n, lane, status);
-        }
+        for (int h2 = 0; h2 < 4; ++h2) bits |= ((valid >> h2) & 1) && hb[h2] == blk ? 1u << h2 : 0u;
+        if (!((valid >> h) & 1) || (bits & ((1u << h) - 1u))) continue;  // missing, or listed with the block's first half
+        const int loc = PLAN != kPlanSplit || part == 1 ? local_id(g, w, blk) : -1;
+        const int sel = PLAN != kPlanSplit || part == 0 ? selected_id(g, w, blk, j, lane, status) : -1;
+        n = merge_list(loc, bits, sel, PLAN == kPlanTagged ? bits << 4 : bits, sm.tmp_ids, sm.tmp_mask, n, lane);
       }
       if (g.cpb == 1 && valid == 0xF && part == 0) {
         // Four different query blocks: which two share a 128-row tile is free.  Take the pairing whose tiles have
@@ -659,12 +677,20 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
       }
       const int buf = lb % kLists;
       interleave_tiles(sm.tmp_ids, sm.tmp_mask, n, sm.ids[buf], sm.mask[buf], lane);
+      // A part keeps the order of the whole item's list: a row's result must not depend on where the queue cuts, which
+      // depends on the number of units and of SMs.  (A 32 x 64 grid, all of which is cut: 30.4 us a pass with lists of the
+      // parts' own blocks, 32.0 so.)
+      if (width < 4) n = keep_part(sm.ids[buf], sm.mask[buf], n, first, width, lane);
       tile_steps(sm.mask[buf], n, sm.steps[buf], sm.info[buf].nsteps, lane);
       if (lane == 0) {
         ItemInfo& inf = sm.info[buf];
-        inf.n = n; inf.unit = u; inf.hvalid = valid; inf.more = 0; inf.branch = part;
+        inf.n = n; inf.unit = u; inf.hvalid = (int)part_mask((unsigned)valid, first, width); inf.more = 0; inf.branch = part;
 #pragma unroll
-        for (int h = 0; h < 4; ++h) { inf.hb[h] = hb[h]; inf.hc[h] = hc[h]; }
+        for (int h = 0; h < 4; ++h) {
+          const int from = first + (h < width ? h : 0);
+          inf.hb[h] = from == 0 ? hb[0] : from == 1 ? hb[1] : from == 2 ? hb[2] : hb[3];
+          inf.hc[h] = from == 0 ? hc[0] : from == 1 ? hc[1] : from == 2 ? hc[2] : hc[3];
+        }
       }
       __syncwarp();
       ++lb;

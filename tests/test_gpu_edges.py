@@ -96,6 +96,35 @@ def test_lists_that_a_tile_does_not_attend(nlat, nlon, heads, topk):
             assert all(np.array_equal(a, b) for a, b in zip(run(w, x, idx, gates), want))
 
 
+# A unit's bits depend on its own inputs only: not on its place in the batch, nor on how many units there are, by which the
+# work queue cuts items into parts (every number on 148 SMs: 8 units of 113 items leave 16, cut into four; one unit is not cut;
+# 2 leave 78, not cut, 3 leave 43, cut into two; 7 items are cut into four, 70 into two, 77 not).
+ALONE = [(synth.small_case(120, 240, 8, 8, 8, kind="smooth", seed=501, backward=True), (1, 3, 8)),
+         (synth.small_case(24, 56, 8, 8, 5, seed=502, backward=True), (1, 7, 10, 11)),                 # ragged groups
+         (synth.small_case(192, 16, 8, 16, 4, seed=503, rlat=8, rlon=1, local_groups=True, backward=True), (1, 6, 8, 13)),
+         (synth.small_case(24, 80, 8, 16, 3, seed=504, backward=True), (1, 6, 12)),
+         (synth.small_case(32, 64, 16, 16, 3, seed=505, backward=True), (1, 8, 10))]
+
+
+@pytest.mark.parametrize("w,counts", ALONE, ids=_name)
+def test_a_units_bits_do_not_depend_on_the_other_units(w, counts):
+    gen = torch.Generator("cuda").manual_seed(w.cfg)
+    one = G.device_inputs(synth.make_inputs(w))
+    gates = torch.randn((1, 1, w.N, 3), device="cuda", generator=gen)
+    want = None
+    for n in counts:
+        wn = dataclasses.replace(w, H=n)
+        dx = {k: torch.cat([v] + [torch.randn(v.shape, device="cuda", generator=gen).to(v.dtype)] * (n - 2) + [v] * (n > 1), dim=1)
+              for k, v in one.items()}
+        idx = G.gpu_select(wn, dx)
+        o, lse = G.gpu_fwd(wn, dx, idx)
+        p, gt = mb.Params.from_workload(wn), gates.expand(1, n, w.N, 3).contiguous()
+        got = [idx, o, lse, *G.gpu_bwd(wn, dx, o, lse, idx), *mb.mosaic_bsa_fwd_branches(p, dx["q"], dx["k"], dx["v"], idx, gt)[1:]]
+        want = [t[:, 0].clone() for t in got] if want is None else want
+        for i, (t, ref) in enumerate(zip(got, want)):
+            assert torch.equal(t[:, 0], ref) and torch.equal(t[:, -1], ref), (n, i)
+
+
 # Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2, 4 or 8 CTAs (as many as
 # give every SM one, at most one per chunk; on the key side the chunks of all query heads of a group count).
 COMPRESS = [synth.small_case(8 * m, 8, 8, 8, 2, H=h, Hkv=kv, seed=360 + i, backward=True) for i, (m, h, kv) in enumerate([
