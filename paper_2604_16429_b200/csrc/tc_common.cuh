@@ -712,14 +712,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 }
 }  // namespace
 
-// Cuts the last, partly filled round of items (one item per SM and round) into parts, as finely as they still fit one
-// round.  A part walks a shorter list, alone on its SM: 128-row parts take about 0.6 of the time of a
-// 256-row item and 64-row parts 0.45: worth it where SMs would be idle (32 items of a 32 x 64 grid: forward 26.0 -> 17.4 us;
-// 904 items: 155 -> 154) but not after one to three full rounds, whose SMs finish far apart and pick the rest up anyway
-// (330 items: 63.9 -> 71.0 us).
+// Cuts the last, partly filled round of items (one item per SM and round) into parts, as finely as they still fit one round: a
+// part walks a shorter list, alone on its SM.  Forward in us, uncut and cut, at items = full rounds x 148 + rest (one unit of
+// 2 x 2 groups of 64-token blocks, top-k 8; 128-token blocks alike): 20 items 27.8 / 20.2, 37 (the most for quarters) 29.1 /
+// 20.7, 38 (halves) 28.6 / 23.8, 74 (the most for halves) 29.5 / 24.3, 148 + 2 48.0 / 39.5, 148 + 42 48.7 / 43.6, 296 + 34
+// 67.8 / 59.7, 444 + 6 86.5 / 78.0, 592 + 38 105.7 / 101.0, 888 + 16 142.9 / 134.9; a rest that is not cut changes nothing.
 inline Queue make_queue(long long items, int sms) {
-  const int rem = (int)(items % sms), few = items >= sms && items < 4ll * sms;
-  const int pieces = few ? 1 : rem * 4 <= sms ? 4 : rem * 2 <= sms ? 2 : 1;
+  const int rem = (int)(items % sms), pieces = rem * 4 <= sms ? 4 : rem * 2 <= sms ? 2 : 1;
   Queue q;
   q.full = (int)items - rem;
   q.pieces = pieces;

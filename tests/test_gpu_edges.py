@@ -40,8 +40,7 @@ def test_ranking_and_pooling_at_tile_and_rule_edges(w):
 
 
 # Work queue of the row-stationary kernels on 148 SMs: the items left over after full waves are cut into four parts up to
-# 37 of them, into two up to 74; none are cut after one to three full waves.  One item per unit here (2 x 2 blocks, and
-# three blocks in a row, whose fourth part is empty).
+# 37 of them, into two up to 74.  One item per unit here (2 x 2 blocks, and three blocks in a row, whose fourth part is empty).
 QUEUE = [(16, 16, h) for h in (1, 37, 38, 74, 75, 148, 149, 593, 630)] + [(8, 24, h) for h in (1, 38, 75, 594, 631)]
 
 
