@@ -13,7 +13,7 @@
 //
 // Everything here is fp32 on the CUDA cores (4 to 8 m^2 d FLOP per unit; the inputs are fp32 sums).  A CTA of 256 threads
 // owns 64 stationary blocks of one unit and streams the other side in chunks of 64; a thread computes a 4 x 4 tile of a
-// 64 x 64 product from shared memory.  The chunks of a tile are split over a cluster of up to 8 CTAs, which add their partial sums over
+// 64 x 64 product from shared memory.  The chunks of a tile are split over a cluster of up to 4 CTAs, which add their partial sums over
 // distributed shared memory in rank order, so results do not depend on timing.
 // Bound by shared-memory operand loads (2 reads of 4 words per 16 FMAs) and, for few tiles, by the length of a stream.  us,
 // before -> after: forward of 8 units of 450 blocks twice 77 -> 53, backward of both sides 110 -> 81; backward of 12 units of
@@ -303,12 +303,13 @@ __global__ void __launch_bounds__(kThr) compress_bwd_kernel(Geo g, const Compres
   else compress_bwd_tile<true>(g, sm, (cta - query_ctas) / ranks, a);
 }
 
-// CTAs per tile: enough of them that every SM gets one, at most one per chunk (and 8, the portable cluster size).  With two
-// per SM the sums over the ranks and the repeated loads cost more than the shorter streams give (8 units of 450 blocks:
-// forward twice 52.8 us against 44.1, backward 80.8 against 69.3; without clusters 84.1 and 89.3).
-int cluster_size(long long tiles_total, int chunks) {
+// CTAs per tile: at most four, at most one per chunk.  Not by how many units there are, because the sums are formed per CTA:
+// a unit's bits must not depend on the others.  us of a pass over units of 450 blocks with a cluster of two, four, eight: training
+// 1 unit 314, 274, 260, 4 units 614, 586, 586, 8 units 999, 1001, 1021, 16 units 1850, 1875, 1914, 64 units 6831, 6883, 7034,
+// inference of 192 units 4843, 4881, 4993.
+int cluster_size(int chunks) {
   int s = 1;
-  while (s < 8 && tiles_total * s < 148 && 2 * s <= chunks) s *= 2;
+  while (s < 4 && 2 * s <= chunks) s *= 2;
   return s;
 }
 
@@ -326,7 +327,8 @@ int launch_clustered(const HostCtx& c, Kernel kernel, size_t smem, unsigned long
 int launch_compress(const HostCtx& c, const float* pooled_q, const float* pooled_k, const float* pooled_v, float* ocg,
                     float* lse2) {
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
-  const int tiles = (c.g.m + kT - 1) / kT, s = cluster_size((long long)c.g.U * tiles, tiles);
+  const int tiles = (c.g.m + kT - 1) / kT, s = cluster_size(tiles);
+  if ((long long)c.g.U * tiles * s > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
   return launch_clustered(c, compress_kernel, sizeof(FwdSmem), &configured, (long long)c.g.U * tiles * s, s, c.g, pooled_q,
                           pooled_k, pooled_v, ocg, lse2);
 }
@@ -335,7 +337,7 @@ int launch_compress_bwd(const HostCtx& c, const CompressBwd& a) {
   static unsigned long long configured = 0;  // devices on which the kernel's shared-memory opt-in is set
   const int tiles = (c.g.m + kT - 1) / kT;
   const long long q_tiles = (long long)c.g.U * tiles, kv_tiles = (long long)c.g.Ukv * tiles;
-  const int s = cluster_size(kv_tiles, tiles * (c.g.H / c.g.Hkv));  // the key side has the longer streams
+  const int s = cluster_size(tiles * (c.g.H / c.g.Hkv));  // the key side has the longer streams
   if (q_tiles * s > 0x7fffffffll) return MOSAIC_E_UNSUPPORTED;
   return launch_clustered(c, compress_bwd_kernel, sizeof(BwdSmem), &configured, (q_tiles + kv_tiles) * s, s, c.g, a,
                           (int)(q_tiles * s));

@@ -97,7 +97,8 @@ def test_lists_that_a_tile_does_not_attend(nlat, nlon, heads, topk):
 
 # A unit's bits depend on its own inputs only: not on its place in the batch, nor on how many units there are, by which the
 # work queue cuts items into parts (every number on 148 SMs: 8 units of 113 items leave 16, cut into four; one unit is not cut;
-# 2 leave 78, not cut, 3 leave 43, cut into two; 7 items are cut into four, 70 into two, 77 not).
+# 2 leave 78, not cut, 3 leave 43, cut into two; 7 items are cut into four, 70 into two, 77 not).  The block level sums
+# 450, 21, 24, 15 and 8 blocks in four, one, one, one and one parts.
 ALONE = [(synth.small_case(120, 240, 8, 8, 8, kind="smooth", seed=501, backward=True), (1, 3, 8)),
          (synth.small_case(24, 56, 8, 8, 5, seed=502, backward=True), (1, 7, 10, 11)),                 # ragged groups
          (synth.small_case(192, 16, 8, 16, 4, seed=503, rlat=8, rlon=1, local_groups=True, backward=True), (1, 6, 8, 13)),
@@ -118,14 +119,16 @@ def test_a_units_bits_do_not_depend_on_the_other_units(w, counts):
         idx = G.gpu_select(wn, dx)
         o, lse = G.gpu_fwd(wn, dx, idx)
         p, gt = mb.Params.from_workload(wn), gates.expand(1, n, w.N, 3).contiguous()
-        got = [idx, o, lse, *G.gpu_bwd(wn, dx, o, lse, idx), *mb.mosaic_bsa_fwd_branches(p, dx["q"], dx["k"], dx["v"], idx, gt)[1:]]
+        three = mb.mosaic_bsa_fwd_branches(p, dx["q"], dx["k"], dx["v"], idx, gt)
+        three += mb.mosaic_bsa_bwd_branches(p, dx["q"], dx["k"], dx["v"], idx, gt, dx["do"])
+        got = [idx, o, lse, *G.gpu_bwd(wn, dx, o, lse, idx), *three]
         want = [t[:, 0].clone() for t in got] if want is None else want
         for i, (t, ref) in enumerate(zip(got, want)):
             assert torch.equal(t[:, 0], ref) and torch.equal(t[:, -1], ref), (n, i)
 
 
-# Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2, 4 or 8 CTAs (as many as
-# give every SM one, at most one per chunk; on the key side the chunks of all query heads of a group count).
+# Block level of the three-branch form: 64 x 64 tiles, a tile's streams over a cluster of 1, 2 or 4 CTAs (at most one per
+# chunk; on the key side the chunks of all query heads of a group count).
 COMPRESS = [synth.small_case(8 * m, 8, 8, 8, 2, H=h, Hkv=kv, seed=360 + i, backward=True) for i, (m, h, kv) in enumerate([
     (63, 1, 0), (64, 1, 0), (65, 1, 0), (129, 1, 0), (193, 1, 0), (449, 1, 0), (65, 4, 1), (65, 6, 2)])]
 
@@ -142,8 +145,8 @@ def test_block_level_tiles_and_cluster_sizes(w):
 
 @pytest.mark.parametrize("heads", [16, 40, 148])
 def test_block_level_many_units(heads):
-    """Gated pooling with 2, 4 and 8 channels per lane (4 * heads * 65 pooled blocks), and with 148 units a block level
-    that needs no clusters."""
+    """Gated pooling with 2, 4 and 8 channels per lane (4 * heads * 65 pooled blocks), and with 148 units a block level of
+    many CTAs per SM."""
     w = synth.small_case(40, 104, 8, 8, 3, H=heads, seed=380 + heads, backward=True)
     x = synth.make_inputs(w)
     idx = G.gpu_select(w, G.device_inputs(x))
