@@ -19,6 +19,8 @@
  *     attention (Hkv < H; paper: "Overall architecture" paragraph, GQA ratio 4) K, V, dK, dV
  *     are [B, Hkv, N, d] and query head h reads key/value head h / (H / Hkv); the selection
  *     stays per query head, dK and dV sum over the query heads of a group.
+ *   - A unit's results do not depend on the other units of the call, nor on its place among them, bit for bit.
+ *   - Outputs and the workspace must not overlap inputs or one another, except where an entry point says so.
  *   - block_idx is contiguous [B, H, m, topk] int32, m = (nlat/bh)*(nlon/bw), block id
  *     j = by*(nlon/bw) + bx.  Row i holds the selected non-local block ids of query
  *     block i, best first, padded with -1.  The local set is implicit.

@@ -16,7 +16,7 @@
 // 64 x 64 product from shared memory.  The chunks of a tile are split over a cluster of up to 4 CTAs, which add their partial sums over
 // distributed shared memory in rank order, so results do not depend on timing.
 // Bound by shared-memory operand loads (2 reads of 4 words per 16 FMAs) and, for few tiles, by the length of a stream.  us,
-// before -> after: forward of 8 units of 450 blocks twice 77 -> 53, backward of both sides 110 -> 81; backward of 12 units of
+// before -> after: forward of 8 units of 450 blocks twice 77 -> 47, backward of both sides 110 -> 72; backward of 12 units of
 // 384 blocks 212 -> 92; of 20 units of 24 blocks 27 -> 16.
 #include <cooperative_groups.h>
 

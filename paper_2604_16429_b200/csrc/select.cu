@@ -22,7 +22,7 @@ namespace mosaic {
 //      |ea| <= 2^-18 |a| per channel) and s~ = ah.bh + ah.bl + al.bh by mma.sync with fp32 accumulation.  What is left
 //      out (al.bl and the ea, eb terms) is at most 3 * 2^-18 (1 + 2^-8) |a||b| by Cauchy-Schwarz; twelve accumulation steps of
 //      sixteen exact products, each step off by at most 17 * 2^-23 |a||b| even if it truncates, add 2^-15.3 |a||b|.
-//      The kernel uses eps = 2^-14 * na * nb + 1e-37 with the norm bounds of the pooling kernel, 1.8 times the sum.  A
+//      The kernel uses eps = 2^-14 * na * nb + 1e-37 with the norm bounds of the pooling kernel, 1.7 times the sum.  A
 //      non-finite s~, and vectors so short that their parts may be subnormal, make the candidate's interval (-inf, +inf).
 //   2. first pass: every lane keeps the largest lower bounds s~ - eps of its share of a row's keys; the k-th largest of
 //      the row's 64 kept values is a lower bound thr of the row's k-th best exact score (they belong to k distinct

@@ -63,16 +63,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Non-blocking test of a phase.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // Bounded wait.  Returns false after the limit (status recorded) or once another thread aborted.
 // The clock and the abort flag are looked at only every 64 polls to keep the poll loop light.
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
@@ -95,6 +85,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return mbar_wait_slow(bar, parity, abort, status);
 }
 
+// A bounded wait of a converged warp whose lanes all wait for the same phase: the outcome is the same in every lane, and the
+// usual case is one poll and one vote.
+__device__ __noinline__ bool warp_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort, status));
+}
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return warp_wait_slow(bar, parity, abort, status);
+}
+
 // Abort path only: a bounded wait for phase `parity` of `bar` that records nothing.  After a failed wait the roles
 // leave their loops with copies and tensor-core work possibly still in flight; the producer waits on the barriers it
 // armed and each MMA issuer commits and waits once more, so that shared memory and TMEM are released only after
@@ -105,15 +105,6 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
   while (!mbar_try_wait(bar, parity))
     if (clock64() - t0 > kDrainCycles) return false;
   return true;
-}
-// The same for a converged warp whose lanes all wait for the same phase: the outcome is the same in every lane, and the
-// usual case is one poll and one vote.
-__device__ __noinline__ bool warp_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
-  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort, status));
-}
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-  return warp_wait_slow(bar, parity, abort, status);
 }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
@@ -223,12 +214,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       "%15, %16};" ::"r"(taddr),
       MOSAIC_W16(r, 0)
       : "memory");
-}
-
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
-               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
 }
 
 __device__ __forceinline__ float ex2(float x) {

@@ -39,6 +39,19 @@ def test_ranking_and_pooling_at_tile_and_rule_edges(w):
     assert np.array_equal(got, want), f"{(got != want).sum()} of {want.size} ids differ"
 
 
+@pytest.mark.parametrize("offset", [1.0, 16.0, 64.0])
+def test_ranking_of_vectors_with_a_large_common_part(offset):
+    """A constant on every channel of Q and K: all scores of a row are alike in their leading bits, down to below the width
+    of the screening's bounds, so that from few to all rows keep more candidates than there is room for and score every key."""
+    w = synth.small_case(3072, 16, 8, 16, 24, H=2, kind="smooth", seed=335)
+    x = synth.make_inputs(w)
+    for n in ("q", "k"):
+        x[n] = synth.to_bf16_bits(synth.bf16_bits_to_f32(x[n]) + np.float32(offset))
+    got = G.gpu_select(w, G.device_inputs(x)).cpu().numpy()
+    want = G.oracle_select_all(w, x)
+    assert np.array_equal(got, want), f"{(got != want).sum()} of {want.size} ids differ"
+
+
 # Work queue of the row-stationary kernels on 148 SMs: the items left over after full waves are cut into four parts up to
 # 37 of them, into two up to 74.  One item per unit here (2 x 2 blocks, and three blocks in a row, whose fourth part is empty).
 QUEUE = [(16, 16, h) for h in (1, 37, 38, 74, 75, 148, 149, 593, 630)] + [(8, 24, h) for h in (1, 38, 75, 594, 631)]
@@ -182,8 +195,9 @@ def test_transposed_lists_for_any_topk(topk):
 
 @pytest.mark.parametrize("bh,bw,nlat,nlon", [(8, 8, 64, 64), (8, 16, 64, 128)])
 def test_a_tile_that_skips_most_of_its_items_list(bh, bw, nlat, nlon):
-    """The two tiles of an item walk their own entries of the merged list; here a tile attends only the first and the last
-    of 60 blocks that the other one attends in between, many more than the key ring holds."""
+    """The two tiles of an item walk their own entries of a merged list of 64, and rows without entries stand beside full ones.
+    (The planner pairs the blocks that have most in common, so the two tiles take turns; with one unit every item is cut into
+    parts.  Lists whose tiles wait for one another over the whole key ring: test_lists_of_very_different_lengths.)"""
     w = synth.small_case(nlat, nlon, bh, bw, 30, H=1, seed=420 + bw, rlat=0, rlon=0, backward=True)
     x = synth.make_inputs(w)
     dx = G.device_inputs(x)
@@ -287,14 +301,18 @@ def test_passes_back_to_back_on_the_same_buffers(nlat, nlon, heads):
     idx = torch.empty((1, heads, w.m, 3), dtype=torch.int32, device="cuda")
     o, lse = torch.empty_like(xs[0]["q"]), torch.empty((1, heads, w.N), device="cuda")
     grads, three, dg = [[torch.empty_like(o) for _ in range(3)] for _ in range(2)] + [torch.empty_like(gates)]
+    pos = torch.rand((w.N, 2), device="cuda", generator=torch.Generator("cuda").manual_seed(heads + 1))
+    qr, kr, o3, lse3 = torch.empty_like(o), torch.empty_like(o), torch.empty_like(o), [torch.empty_like(lse) for _ in range(2)]
 
     def run(x):
-        mb.mosaic_bsa_select(p, x["q"], x["k"], block_idx=idx, ws=ws)
+        mb.mosaic_bsa_rope(p, x["q"], x["k"], pos, q_out=qr, k_out=kr)
+        mb.mosaic_bsa_select(p, qr, kr, block_idx=idx, ws=ws)
+        mb.mosaic_bsa_fwd_branches(p, qr, kr, x["v"], idx, gates, o=o3, lse_fg=lse3[0], lse_l=lse3[1], ws=ws)
         mb.mosaic_bsa_fwd(p, x["q"], x["k"], x["v"], idx, o=o, lse=lse, ws=ws)
         mb.mosaic_bsa_bwd(p, x["q"], x["k"], x["v"], o, lse, x["do"], idx, dq=grads[0], dk=grads[1], dv=grads[2], ws=ws)
         mb.mosaic_bsa_bwd_branches(p, x["q"], x["k"], x["v"], idx, gates, x["do"], dq=three[0], dk=three[1], dv=three[2],
                                    dgates=dg, ws=ws)
-        return [t.clone() for t in (idx, o, lse, *grads, *three, dg)]
+        return [t.clone() for t in (qr, kr, idx, o3, *lse3, o, lse, *grads, *three, dg)]
 
     alone = []
     for x in xs:
