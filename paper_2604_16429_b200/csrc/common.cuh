@@ -105,9 +105,10 @@ __host__ __device__ inline int items_per_unit(const Geo& g) {
 }
 
 // A kernel may be launched before the one ahead of it in the stream has finished (launch_kernel below says which are): every
-// kernel sets up what touches no global memory, then calls this.  It returns when everything ahead is complete and visible, and lets the next
-// kernel's CTAs in as SMs run empty (not earlier: the chain of waits makes "the kernel before me is complete" mean "all
-// before it are").  The result is zero, opaque to the compiler: an address that it takes part in cannot be read earlier.
+// kernel sets up what touches no global memory, then calls this.  It returns when everything ahead is complete and visible,
+// and lets the next kernel's CTAs in as SMs run empty (not earlier: the chain of waits makes "the kernel before me is
+// complete" mean "all before it are").  The result is zero, opaque to the compiler: an address that it takes part in cannot
+// be read earlier.
 __device__ __forceinline__ int await_stream() {
   int zero;
   asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");

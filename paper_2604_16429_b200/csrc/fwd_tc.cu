@@ -34,8 +34,9 @@
 // quarter of the exponentials evaluated by a cubic on the FMA pipe because at d = 64 the MUFU pipe
 // (16 ex2 per clock per SM against 8192 tensor FLOP per clock) is the limiter, not the tensor core.
 // Bound by the softmax warps: 730 cycles per product against 384 of MUFU time; one more satisfied wait per product costs
-// them 3 %, one more in the MMA issuers nothing (8 units of 28800 tokens 162 -> 155 us with cheaper polls and the queue's parts).  With
-// 64-token blocks the planner is the next: since it builds its lists without integer divisions the same takes 146 us (159, L2 flushed).
+// them 3 %, one more in the MMA issuers nothing (8 units of 28800 tokens 162 -> 155 us with cheaper polls and the queue's
+// parts).  With 64-token blocks the planner is next: without integer divisions in its lists the same input takes 146 us
+// instead of 159 (L2 flushed).
 // Three-branch form (kFwdBranches, kFwdStats): the planner hands out an item twice in a row, with its selected list and with
 // its local list; the first epilogue leaves the selected part in o (not gated yet: a weighted mean of values fits their type
 // whatever the gates are), the second weights it and adds its own and the block level's.  kFwdStats
