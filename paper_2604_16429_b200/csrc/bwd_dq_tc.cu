@@ -97,51 +97,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     planner_loop<BR ? kPlanTagged : kPlanUnion>(sm, g, block_idx, work_counter, ipu, queue, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t step = 0;   // key/value chunks issued so far (ring position)
-      int q_armed[2] = {-1, -1};  // phase parity of the last load into each tile's Q / dO buffer
-      bool ok = true;
-      for (int it = 0; ok; ++it) {
-        const int buf = it % kLists;
-        ok = mbar_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
+    uint32_t step = 0;   // key/value chunks issued so far (ring position)
+    int q_armed[2] = {-1, -1};  // phase parity of the last load into each tile's Q / dO buffer
+    bool ok = true;
+    for (int it = 0; ok; ++it) {
+      const int buf = it % kLists;
+      ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
+      if (!ok) break;
+      const ItemInfo& inf = sm.info[buf];
+      const int n = inf.n, u = inf.unit;
+      if (n < 0) break;
+      // Q and dO tiles: free once the tile's last S / dP products of the previous item have completed
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (ok) ok = warp_wait(s32(&sm.q_empty[t]), (it & 1) ^ 1, abort, status);
         if (!ok) break;
-        const ItemInfo& inf = sm.info[buf];
-        const int n = inf.n, u = inf.unit;
-        if (n < 0) break;
-        const int ukv = kv_unit(g, u);  // key/value head of this query head's group
-        // Q and dO tiles: free once the tile's last S / dP products of the previous item have completed
-        for (int t = 0; t < 2 && ok; ++t) {
-          ok = mbar_wait(s32(&sm.q_empty[t]), (it & 1) ^ 1, abort, status);
-          if (!ok) break;
+        q_armed[t] = it & 1;
+        if (elect_one()) {
           mbar_expect_tx(s32(&sm.q_full[t]), 4 * kTile);
-          q_armed[t] = it & 1;
+#pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            const int h = 2 * t + hh, by = inf.hb[h] / g.nbw, bx = inf.hb[h] - by * g.nbw;
-            tma_load_4d(s32(sm.q[t] + hh * kTile), &map_q, s32(&sm.q_full[t]), 0, bx * g.bw,
-                        by * g.bh + inf.hc[h] * g.crows, u);
-            tma_load_4d(s32(sm.d_o[t] + hh * kTile), &map_do, s32(&sm.q_full[t]), 0, bx * g.bw,
-                        by * g.bh + inf.hc[h] * g.crows, u);
+            const int x = inf.hx[2 * t + hh], y = inf.hy[2 * t + hh];
+            tma_load_4d(s32(sm.q[t] + hh * kTile), &map_q, s32(&sm.q_full[t]), 0, x, y, u);
+            tma_load_4d(s32(sm.d_o[t] + hh * kTile), &map_do, s32(&sm.q_full[t]), 0, x, y, u);
           }
         }
-        for (int e = 0; e < n && ok; ++e) {
-          const int j = sm.ids[buf][e], by = j / g.nbw, bx = j - by * g.nbw;
-          const uint32_t mk = who_attends(sm.mask[buf][e]);
-          for (int c = 0; c < g.cpb; ++c, ++step) {
-            const uint32_t st = step % kStages;
-            const uint32_t full = s32(&sm.kv_full[step % kFullBars]);
-            ok = mbar_wait(s32(&sm.kv_empty[st]), ((step / kStages) & 1) ^ 1, abort, status);
-            if (!ok) break;
-            mbar_expect_tx(full, 2 * kTile);
-            tma_load_4d(s32(sm.kv[st][0]), &map_k, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
-            tma_load_4d(s32(sm.kv[st][1]), &map_v, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
-            // a tile that does not attend this entry never looks at the stage: its release is given here
-            if (!(mk & 3u)) mbar_arrive(s32(&sm.kv_empty[st]));
-            if (!(mk & 12u)) mbar_arrive(s32(&sm.kv_empty[st]));
-          }
-        }
-        if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
+        __syncwarp();
       }
-      if (*abort) {  // copies this thread issued must land before the CTA's memory is released
+      // (key/value head of this query head's group)
+      if (ok) ok = produce_chunks<kStages>(sm, g, &map_k, &map_v, buf, n, kv_unit(g, u), step, lane, abort, status);
+      if (ok && elect_one()) mbar_arrive(s32(&sm.list_empty[buf]));
+    }
+    if (lane == 0) {
+      if (*abort) {  // copies this warp issued must land before the CTA's memory is released
         const uint32_t first = step > kStages ? step - kStages : 0;
         for (uint32_t s = first; s < step; ++s) mbar_drain(s32(&sm.kv_full[s % kFullBars]), (s / kFullBars) & 1);
         for (int t = 0; t < 2; ++t)
@@ -246,6 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t ts = tmem + lane_off + kColS + 128 * t, tdp = ts + 64, tdq = tmem + lane_off + kColDQ + 64 * t;
     const uint32_t tds = tmem + lane_off + kColDS + 64 * t;
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
+    const int row_y = (tid & 63) / g.bw, row_x = (tid & 63) - row_y * g.bw;  // the row's place in its chunk
     uint32_t nt = 0;
     bool ok = true;
     for (int it = 0; ok; ++it) {
@@ -256,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (n < 0) break;
       const bool valid = (sm.info[buf].hvalid >> h) & 1;
       const long long tok =
-          (long long)sm.info[buf].unit * g.N + chunk_token(g, sm.info[buf].hb[h], sm.info[buf].hc[h], tid & 63);
+          (long long)sm.info[buf].unit * g.N + (long long)(sm.info[buf].hy[h] + row_y) * g.nlon + sm.info[buf].hx[h] + row_x;
       // negated log-sum-exp (in base-2 units), negated D and gate of this thread's query row, per branch
       float nl[2], nd[2], gt[2];
 #pragma unroll

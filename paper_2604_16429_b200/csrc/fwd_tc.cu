@@ -172,51 +172,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     planner_loop<MODE == kFwdUnion ? kPlanUnion : kPlanSplit>(sm, g, block_idx, work_counter, ipu, queue, lane, abort, status);
   } else if (warp == 8) {
     // ------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t step = 0;   // key/value chunks issued so far (ring position)
-      int q_armed[2][2] = {{-1, -1}, {-1, -1}};  // phase parity of the last load into each query-tile buffer
-      bool ok = true;
-      for (int it = 0; ok; ++it) {
-        const int buf = it % kLists, qb = it & 1;
-        ok = mbar_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
+    uint32_t step = 0;   // key/value chunks issued so far (ring position)
+    int q_armed[2][2] = {{-1, -1}, {-1, -1}};  // phase parity of the last load into each query-tile buffer
+    bool ok = true;
+    for (int it = 0; ok; ++it) {
+      const int buf = it % kLists, qb = it & 1;
+      ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
+      if (!ok) break;
+      const ItemInfo& inf = sm.info[buf];
+      const int n = inf.n, u = inf.unit;
+      if (n < 0) break;
+      // query tiles (double-buffered by item parity): free once the softmax threads have copied the rows of
+      // the item before the previous one to TMEM, so this load runs while the previous item still computes
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (ok) ok = warp_wait(s32(&sm.q_empty[qb][t]), ((it >> 1) & 1) ^ 1, abort, status);
         if (!ok) break;
-        const ItemInfo& inf = sm.info[buf];
-        const int n = inf.n, u = inf.unit;
-        if (n < 0) break;
-        const int ukv = kv_unit(g, u);  // key/value head of this query head's group
-        // query tiles (double-buffered by item parity): free once the softmax threads have copied the rows of
-        // the item before the previous one to TMEM, so this load runs while the previous item still computes
-        for (int t = 0; t < 2 && ok; ++t) {
-          ok = mbar_wait(s32(&sm.q_empty[qb][t]), ((it >> 1) & 1) ^ 1, abort, status);
-          if (!ok) break;
+        q_armed[qb][t] = (it >> 1) & 1;
+        if (elect_one()) {
           mbar_expect_tx(s32(&sm.q_full[qb][t]), 2 * kTile);
-          q_armed[qb][t] = (it >> 1) & 1;
-          for (int hh = 0; hh < 2; ++hh) {
-            const int h = 2 * t + hh, by = inf.hb[h] / g.nbw, bx = inf.hb[h] - by * g.nbw;
-            tma_load_4d(s32(sm.q[qb][t] + hh * kTile), &map_q, s32(&sm.q_full[qb][t]), 0, bx * g.bw,
-                        by * g.bh + inf.hc[h] * g.crows, u);
-          }
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh)
+            tma_load_4d(s32(sm.q[qb][t] + hh * kTile), &map_q, s32(&sm.q_full[qb][t]), 0, inf.hx[2 * t + hh], inf.hy[2 * t + hh], u);
         }
-        for (int e = 0; e < n && ok; ++e) {
-          const int j = sm.ids[buf][e], by = j / g.nbw, bx = j - by * g.nbw;
-          const uint32_t mk = sm.mask[buf][e];
-          for (int c = 0; c < g.cpb; ++c, ++step) {
-            const uint32_t st = step % kStages;
-            const uint32_t full = s32(&sm.kv_full[step % kFullBars]);
-            ok = mbar_wait(s32(&sm.kv_empty[st]), ((step / kStages) & 1) ^ 1, abort, status);
-            if (!ok) break;
-            mbar_expect_tx(full, 2 * kTile);
-            tma_load_4d(s32(sm.kv[st][0]), &map_k, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
-            tma_load_4d(s32(sm.kv[st][1]), &map_v, full, 0, bx * g.bw, by * g.bh + c * g.crows, ukv);
-            // a tile that does not attend this entry never looks at the stage: its release is given here (the other
-            // tile's release, after its P V, is what lets the stage be reused)
-            if (!(mk & 3u)) mbar_arrive(s32(&sm.kv_empty[st]));
-            if (!(mk & 12u)) mbar_arrive(s32(&sm.kv_empty[st]));
-          }
-        }
-        if (ok) mbar_arrive(s32(&sm.list_empty[buf]));
+        __syncwarp();
       }
-      if (*abort) {  // copies this thread issued must land before the CTA's memory is released
+      // (key/value head of this query head's group)
+      if (ok) ok = produce_chunks<kStages>(sm, g, &map_k, &map_v, buf, n, kv_unit(g, u), step, lane, abort, status);
+      if (ok && elect_one()) mbar_arrive(s32(&sm.list_empty[buf]));
+    }
+    if (lane == 0) {
+      if (*abort) {  // copies this warp issued must land before the CTA's memory is released
         const uint32_t first = step > kStages ? step - kStages : 0;
         for (uint32_t s = first; s < step; ++s) mbar_drain(s32(&sm.kv_full[s % kFullBars]), (s / kFullBars) & 1);
         for (int i = 0; i < 4; ++i)
@@ -322,6 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t ts = tmem + lane_off + kColS + 128 * t, to = tmem + lane_off + kColO + 64 * t;
     const uint32_t tq = tmem + lane_off + kColQ + 32 * t;
     const uint64_t scale2 = pack2(g.scale_log2, g.scale_log2);
+    const int row_y = (tid & 63) / g.bw, row_x = (tid & 63) - row_y * g.bw;  // the row's place in its chunk
     uint32_t nt = 0;
     bool ok = true;
     // Copies this thread's query row of item `it2` from shared memory (128-byte swizzled rows) to TMEM, where it is
@@ -475,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if ((sm.info[buf].hvalid >> h) & 1) {
         const int u = sm.info[buf].unit, blk = sm.info[buf].hb[h], branch = sm.info[buf].branch;
-        const long long tok = (long long)u * g.N + chunk_token(g, blk, sm.info[buf].hc[h], tid & 63);
+        const long long tok = (long long)u * g.N + (long long)(sm.info[buf].hy[h] + row_y) * g.nlon + sm.info[buf].hx[h] + row_x;
         const float inv = l > 0.f ? 1.f / l : 0.f;  // a row that attends nothing (empty selection): O = 0
         const float lse2 = l > 0.f ? m_ref + log2f(l) : -INFINITY;
         const float* cg = MODE == kFwdUnion ? nullptr : out.ocg + ((long long)u * g.m + blk) * kD;

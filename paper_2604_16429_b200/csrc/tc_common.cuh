@@ -33,7 +33,8 @@ struct ItemInfo {
   int unit;     // (batch, head) unit
   int hvalid;   // bit h: half h exists
   int hb[4];    // query block of half h
-  int hc[4];    // 64-token chunk of that block
+  int hc[4];    // 64-token chunk of that block (key-stationary kernel)
+  int hx[4], hy[4];  // column and row of that chunk's first token in the grid (row-stationary kernels)
   int more;     // 1: the item's list continues in the next list buffer (lists longer than a buffer)
   int nsteps[2]; // entries that tile 0 and tile 1 attend
   int branch;   // split lists: 0 = the selected blocks, 1 = the local ones
@@ -670,12 +671,16 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
       if (lane == 0) {
         ItemInfo& inf = sm.info[buf];
         inf.n = n; inf.unit = u; inf.hvalid = (int)part_mask((unsigned)valid, first, width); inf.more = 0; inf.branch = part;
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int from = first + (h < width ? h : 0);
-          inf.hb[h] = from == 0 ? hb[0] : from == 1 ? hb[1] : from == 2 ? hb[2] : hb[3];
-          inf.hc[h] = from == 0 ? hc[0] : from == 1 ? hc[1] : from == 2 ? hc[2] : hc[3];
-        }
+      }
+      if (lane < 4) {
+        ItemInfo& inf = sm.info[buf];
+        const int from = first + (lane < width ? lane : 0);
+        const int b = from == 0 ? hb[0] : from == 1 ? hb[1] : from == 2 ? hb[2] : hb[3];
+        const int c = from == 0 ? hc[0] : from == 1 ? hc[1] : from == 2 ? hc[2] : hc[3];
+        const int by = quick_div(b, g.nbw, w.inv_nbw);
+        inf.hb[lane] = b;
+        inf.hx[lane] = (b - by * g.nbw) * g.bw;
+        inf.hy[lane] = by * g.bh + c * g.crows;
       }
       __syncwarp();
       ++lb;
@@ -685,6 +690,39 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
       if (lane == 0) mbar_arrive(s32(&sm.list_full[buf]));
     }
   }
+}
+
+// Producer warp: the key and value chunks of a list through the ring (`step`: ring position of the next chunk).  The whole warp
+// walks the list, and its lanes work out where 32 entries lie at once: one lane that divided for every entry took 830 cycles a
+// chunk beside the row threads (conversions and reciprocals queue behind their exponentials).  Returns false after a failed wait.
+template <int STAGES, class SM>
+__device__ __forceinline__ bool produce_chunks(SM& sm, const Geo& g, const CUtensorMap* map_k, const CUtensorMap* map_v, int buf,
+                                               int n, int ukv, uint32_t& step, int lane, volatile int* abort, int* status) {
+  for (int e0 = 0; e0 < n; e0 += 32) {
+    const int e = e0 + lane, j = e < n ? sm.ids[buf][e] : 0, by = j / g.nbw, x = (j - by * g.nbw) * g.bw, y = by * g.bh;
+    const unsigned m = e < n ? who_attends(sm.mask[buf][e]) : 0u;
+    const int here = min(32, n - e0);
+    for (int i = 0; i < here; ++i) {
+      const int cx = __shfl_sync(0xffffffffu, x, i);
+      int cy = __shfl_sync(0xffffffffu, y, i);
+      const unsigned mk = __shfl_sync(0xffffffffu, m, i);
+      for (int c = 0; c < g.cpb; ++c, ++step, cy += g.crows) {
+        const uint32_t st = step % STAGES, full = s32(&sm.kv_full[step % kFullBars]), empty = s32(&sm.kv_empty[st]);
+        if (!warp_wait(empty, ((step / STAGES) & 1) ^ 1, abort, status)) return false;
+        if (elect_one()) {
+          mbar_expect_tx(full, 2 * kTile);
+          tma_load_4d(s32(sm.kv[st][0]), map_k, full, 0, cx, cy, ukv);
+          tma_load_4d(s32(sm.kv[st][1]), map_v, full, 0, cx, cy, ukv);
+          // a tile that does not attend this entry never looks at the stage: its release is given here (the other
+          // tile's release, after its products, is what lets the stage be reused)
+          if (!(mk & 3u)) mbar_arrive(empty);
+          if (!(mk & 12u)) mbar_arrive(empty);
+        }
+        __syncwarp();
+      }
+    }
+  }
+  return true;
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
