@@ -20,7 +20,7 @@
 // a second thread as each group finishes.  A list with an odd number of chunks ends in a pair of one.
 // Lists: the planner merges the local neighbourhoods of the tile's key blocks (entries carry a mask of the
 // halves they are connected to) and appends each block's CSR list; a list longer than a list buffer
-// continues in the next buffer (ItemInfo::more).  The order of a list is a function of the pattern alone,
+// continues in the next buffer (KvItem::more).  The order of a list is a function of the pattern alone,
 // so the summation order, and with it the result, is deterministic.
 // Bound like dQ by the row threads' instruction queue, about 2600 cycles per pair of products.  Issuers that walk their loops
 // as whole warps, no divisions and no wait on the ring in the row threads: 64 units of 28800 tokens 2405 -> 1802 us, 32 units
@@ -53,6 +53,20 @@ struct Slot {
 };
 static_assert(sizeof(Slot) % 1024 == 0, "slots keep the 1024-byte alignment of the swizzled tiles");
 
+// A work item (tile of 128 key rows) with a list of the query blocks connected to it.  64 bytes, not 36: with a size that is no
+// power of two every role's index into the array is a multiplication, and the kernel, which has no register left of its 96 a
+// thread, spills 92 bytes instead of 40 (training of 32 units of 12288 tokens 1614 us with 96-byte records, now 1570; of 12
+// three-branch units of 49152 tokens 5031, now 4904).
+struct alignas(64) KvItem {
+  int n;        // entries of the list; -1 = no more work
+  int unit;     // the query unit, (batch, query head), of this buffer's list
+  int kvunit;   // the key/value unit of the tile
+  int hvalid;   // bit h: half h exists
+  int more;     // 1: the item's list continues in the next list buffer (lists longer than a buffer)
+  int hb[2];    // key block of half h
+  int hc[2];    // 64-token chunk of that block
+};
+
 struct Smem {
   unsigned char k[2 * kTile];              // 128 key rows x 128 B
   unsigned char v[2 * kTile];
@@ -63,7 +77,7 @@ struct Smem {
   unsigned long long list_full[kLists], list_empty[kLists];
   uint32_t tmem_base;
   int abort;
-  ItemInfo info[kLists];             // hb/hc/hvalid entries 0 and 1 describe the tile's two halves
+  KvItem info[kLists];
   alignas(16) int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
 };
@@ -106,7 +120,7 @@ __device__ __forceinline__ void planner_kv_loop(Smem& sm, const Geo& g, const in
     auto publish = [&](int more) {
       const int buf = lb % kLists;
       if (lane == 0) {
-        ItemInfo& inf = sm.info[buf];
+        KvItem& inf = sm.info[buf];
         inf.n = n; inf.unit = qu; inf.kvunit = u; inf.hvalid = valid; inf.more = more;
         inf.hb[0] = hb[0]; inf.hb[1] = hb[1]; inf.hc[0] = hc[0]; inf.hc[1] = hc[1];
       }
@@ -276,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int buf = lb % kLists;
         ok = mbar_wait(s32(&sm.list_full[buf]), (lb / kLists) & 1, abort, status);
         if (!ok) break;
-        const ItemInfo& inf = sm.info[buf];
+        const KvItem& inf = sm.info[buf];
         const int n = inf.n, u = inf.unit;
         if (n < 0) break;
         if (fresh) {

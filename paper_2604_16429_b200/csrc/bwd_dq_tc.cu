@@ -43,7 +43,7 @@ struct Smem {
   unsigned long long list_full[kLists], list_empty[kLists];
   uint32_t tmem_base;
   int abort;
-  ItemInfo info[kLists];
+  RowItem info[kLists];
   alignas(16) int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
   unsigned short steps[kLists][2][kMaxUnion];  // [list][tile]
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int buf = it % kLists;
       ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
       if (!ok) break;
-      const ItemInfo& inf = sm.info[buf];
+      const RowItem& inf = sm.info[buf];
       const int n = inf.n, u = inf.unit;
       if (n < 0) break;
       // Q and dO tiles: free once the tile's last S / dP products of the previous item have completed

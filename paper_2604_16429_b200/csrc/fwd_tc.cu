@@ -72,7 +72,7 @@ struct Smem {
   unsigned long long list_full[kLists], list_empty[kLists];
   uint32_t tmem_base;
   int abort;
-  ItemInfo info[kLists];
+  RowItem info[kLists];
   alignas(16) int ids[kLists][kMaxUnion];
   unsigned char mask[kLists][kMaxUnion];
   unsigned short steps[kLists][2][kMaxUnion];  // [list][tile]
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int buf = it % kLists, qb = it & 1;
       ok = warp_wait(s32(&sm.list_full[buf]), (it / kLists) & 1, abort, status);
       if (!ok) break;
-      const ItemInfo& inf = sm.info[buf];
+      const RowItem& inf = sm.info[buf];
       const int n = inf.n, u = inf.unit;
       if (n < 0) break;
       // query tiles (double-buffered by item parity): free once the softmax threads have copied the rows of

@@ -28,17 +28,16 @@ constexpr long long kSpinCycles = MOSAIC_TEST_SPIN_CYCLES;
 constexpr long long kSpinCycles = 4000000000ll;  // bound of a single wait (~2 s)
 #endif
 
-struct ItemInfo {
+// A work item of the row-stationary kernels (forward, dQ) with the list that goes with it.  Its size is a power of two so that an
+// index into the array is a shift (with 72 bytes the three-branch dQ takes 156 registers instead of 154).
+struct alignas(128) RowItem {
   int n;        // entries of the merged list; -1 = no more work
   int unit;     // (batch, head) unit
   int hvalid;   // bit h: half h exists
-  int hb[4];    // query block of half h
-  int hc[4];    // 64-token chunk of that block (key-stationary kernel)
-  int hx[4], hy[4];  // column and row of that chunk's first token in the grid (row-stationary kernels)
-  int more;     // 1: the item's list continues in the next list buffer (lists longer than a buffer)
-  int nsteps[2]; // entries that tile 0 and tile 1 attend
   int branch;   // split lists: 0 = the selected blocks, 1 = the local ones
-  int kvunit;   // key-stationary kernel: the key/value unit of the item's tile (`unit` is the query unit of this buffer's list)
+  int nsteps[2]; // entries that tile 0 and tile 1 attend
+  int hb[4];    // query block of half h
+  int hx[4], hy[4];  // column and row of the half's first token in the grid
 };
 
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -669,11 +668,11 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
       if (width < 4) n = keep_part(sm.ids[buf], sm.mask[buf], n, first, width, lane);
       tile_steps(sm.mask[buf], n, sm.steps[buf], sm.info[buf].nsteps, lane);
       if (lane == 0) {
-        ItemInfo& inf = sm.info[buf];
-        inf.n = n; inf.unit = u; inf.hvalid = (int)part_mask((unsigned)valid, first, width); inf.more = 0; inf.branch = part;
+        RowItem& inf = sm.info[buf];
+        inf.n = n; inf.unit = u; inf.hvalid = (int)part_mask((unsigned)valid, first, width); inf.branch = part;
       }
       if (lane < 4) {
-        ItemInfo& inf = sm.info[buf];
+        RowItem& inf = sm.info[buf];
         const int from = first + (lane < width ? lane : 0);
         const int b = from == 0 ? hb[0] : from == 1 ? hb[1] : from == 2 ? hb[2] : hb[3];
         const int c = from == 0 ? hc[0] : from == 1 ? hc[1] : from == 2 ? hc[2] : hc[3];
