@@ -13,7 +13,7 @@ from paper_2604_16429_b200 import build as mbuild
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 # most bytes a thread may spill (stores, loads)
-LIMITS = {"bwd_dkdv_tc.cu": (40, 48)}
+LIMITS = {"bwd_dkdv_tc.cu": (40, 48), "bwd_dq_tc.cu": (0, 0), "fwd_tc.cu": (0, 0)}
 
 
 @pytest.mark.skipif(not os.path.exists(NVCC), reason="needs nvcc")
