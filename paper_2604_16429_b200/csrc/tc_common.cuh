@@ -393,8 +393,9 @@ __device__ __forceinline__ int keep_part(int* ids, unsigned char* mask, int n, i
 }
 
 // What a planner's lane needs of the geometry for every block it lists: its place in the local set (row and column offset; in
-// group mode inside the group) and reciprocals for quick_div.  A list takes the planner 10000 cycles and more, about as long as
-// a short item: with integer divisions a selection and forward of 8 units of 28800 tokens took 188.3 us, now 185.8.
+// group mode inside the group) and reciprocals for quick_div.  A CTA's first list (64-token blocks) takes the planner 11000 to
+// 12700 cycles, 6000 of them the merge; a later one, beside busy row threads, 16000 (merge 9700), about as long as a short item:
+// with integer divisions a selection and forward of 8 units of 28800 tokens took 188.3 us instead of 185.8.
 struct Window {
   int dy, dx;
   bool in;  // the lane holds a place of the local set (columns that come round again in a narrow grid excluded)
@@ -692,8 +693,9 @@ __device__ __forceinline__ void planner_loop(SM& sm, const Geo& g, const int32_t
 }
 
 // Producer warp: the key and value chunks of a list through the ring (`step`: ring position of the next chunk).  The whole warp
-// walks the list, and its lanes work out where 32 entries lie at once: one lane that divided for every entry took 830 cycles a
-// chunk beside the row threads (conversions and reciprocals queue behind their exponentials).  Returns false after a failed wait.
+// walks the list, and its lanes work out where 32 entries lie at once: in the forward of 192 units of 28800 tokens (64-token
+// blocks) one lane that divided once per entry took 830 cycles a chunk beside the row threads (conversions and reciprocals queue
+// behind their exponentials).  Returns false after a failed wait.
 template <int STAGES, class SM>
 __device__ __forceinline__ bool produce_chunks(SM& sm, const Geo& g, const CUtensorMap* map_k, const CUtensorMap* map_v, int buf,
                                                int n, int ukv, uint32_t& step, int lane, volatile int* abort, int* status) {
